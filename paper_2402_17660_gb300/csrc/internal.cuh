@@ -1,6 +1,8 @@
 // Internal definitions shared by the libtnet CUDA sources.
 #pragma once
+#include <mutex>
 #include <utility>
+#include <vector>
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -84,6 +86,22 @@ inline void launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
     cfg.attrs = attr;
     cfg.numAttrs = n;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);  // errors surface in cudaGetLastError
+}
+
+// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per device and kernel.
+// Keyed by the kernel's host-side handle and the device (a template kernel
+// used from two translation units can have a handle in each).
+inline int ensure_smem_attr(const void *kern, int bytes) {
+    static std::mutex mu;
+    static std::vector<std::pair<const void *, int>> done;  // (kernel handle, device)
+    int dev = 0;
+    TNET_CUDA_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> g(mu);
+    for (const auto &d : done)
+        if (d.first == kern && d.second == dev) return TNET_OK;
+    TNET_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    done.emplace_back(kern, dev);
+    return TNET_OK;
 }
 
 constexpr int kMaxCellsPerAtom = 2;   // cell budget: 2 cells per atom + 8 per system + 64

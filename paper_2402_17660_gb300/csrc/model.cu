@@ -2452,7 +2452,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         } else {
             GemmShape pp = gshape(maxU, 3 * F, K, eu, K, W.dproj_w, K);
             pp.rows_dev = nu;
-            TRY(sgemm<false, true>(pp, ep, gctas, st));
+            TRY(sgemm<true>(pp, ep, gctas, sms, st));
         }
     }
 
@@ -2493,12 +2493,12 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             TRY(tcx3(tc::tshape(N, 2 * F, F), n0, N, F, wx.emb_mlp1, 2 * F, F, em1, bn2));
             TRY(tcx3(tc::tshape(N, 3 * F, 2 * F), hs1, N, 2 * F, wx.emb_mlp2, 3 * F, 2 * F, em2, bn3));
         } else {
-            TRY(sgemm<false, true>(gshape(N, 2 * F, F, n0, F, W.emb_mlp1_w, F), em1, gctas, st));
-            TRY(sgemm<false, true>(gshape(N, 3 * F, 2 * F, hs1, 2 * F, W.emb_mlp2_w, 2 * F), em2, gctas, st));
+            TRY(sgemm<true>(gshape(N, 2 * F, F, n0, F, W.emb_mlp1_w, F), em1, gctas, sms, st));
+            TRY(sgemm<true>(gshape(N, 3 * F, 2 * F, hs1, 2 * F, W.emb_mlp2_w, 2 * F), em2, gctas, sms, st));
         }
     }
     if (tcm) TRY(tcg(tc::tshape_classes(N, F), Xraw, nbf, 9LL * N, F, emix, 3 * F, F, EpiStore{Uemb, F, 0}));
-    else TRY(sgemm<false, true>(gshape_classes(N, F, Xraw, W.emb_mix_w), EpiStore{Uemb, F, 0}, gctas, st));
+    else TRY(sgemm<true>(gshape_classes(N, F, Xraw, W.emb_mix_w), EpiStore{Uemb, F, 0}, gctas, sms, st));
     float *X = f32(Lw.Xin);  // layer 0 input
     launch(k_emb_scale, grid_for((int64_t)N * F, 256, sms), 256, 0, st, Uemb, s, N, F, X);
     count_launch();
@@ -2555,15 +2555,15 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         pf.mark(P_MLP1);
         GemmShape p1 = gshape(maxU, F, K, eu, K, Lr.mlp1_w, K);
         p1.rows_dev = nu;
-        TRY(sgemm<false, true>(p1, e1, gctas, st));
+        TRY(sgemm<true>(p1, e1, gctas, sms, st));
         pf.mark(P_MLP2);
         GemmShape p2 = gshape(maxU, 2 * F, F, h1, F, Lr.mlp2_w, F);
         p2.rows_dev = nu;
-        TRY(sgemm<false, true>(p2, e2, gctas, st));
+        TRY(sgemm<true>(p2, e2, gctas, sms, st));
         pf.mark(P_MLP3);
         GemmShape p3 = gshape(maxU, 3 * F, 2 * F, h2, 2 * F, w3p(l), 2 * F);
         p3.rows_dev = nu;
-        TRY(sgemm<false, true>(p3, e3, gctas, st));
+        TRY(sgemm<true>(p3, e3, gctas, sms, st));
         return TNET_OK;
     };
     const int ew = grid_for((int64_t)N * F, 256, sms);
@@ -2578,7 +2578,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         TNET_LAUNCH_CHECK();
         pf.mark(P_NODE_MIX);
         if (tcm) TRY(tcg(tc::tshape_classes(N, F), Xn, nbf, 9LL * N, F, lb[l].mix1, 3 * F, F, EpiStore{Y, F, 0}));
-        else TRY(sgemm<false, true>(gshape_classes(N, F, Xn, W.layer[l].mix1_w), EpiStore{Y, F, 0}, gctas, st));
+        else TRY(sgemm<true>(gshape_classes(N, F, Xn, W.layer[l].mix1_w), EpiStore{Y, F, 0}, gctas, sms, st));
         TRY(edge_mlp(l, !keep_act));
         pf.mark(P_MESSAGE);
         const float *a3l = act(Lw.a3, 3 * F, l);
@@ -2600,7 +2600,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         TNET_LAUNCH_CHECK();
         pf.mark(P_NODE_MIX);
         if (tcm) TRY(tcg(tc::tshape_classes(N, F), Tn, nbf, 9LL * N, F, lb[l].mix2, 3 * F, F, EpiStore{dX, F, 0}));
-        else TRY(sgemm<false, true>(gshape_classes(N, F, Tn, W.layer[l].mix2_w), EpiStore{dX, F, 0}, gctas, st));
+        else TRY(sgemm<true>(gshape_classes(N, F, Tn, W.layer[l].mix2_w), EpiStore{dX, F, 0}, gctas, sms, st));
         pf.mark(P_NODE_ELEM);
         launch(k_residual, ew, 256, 0, st, Xn, dX, N, F, Xnext);
         count_launch();
@@ -2623,8 +2623,8 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             TRY(tcx3(tc::tshape(N, F, 3 * F), hn, N, 3 * F, wx.out, F, 3 * F, eo));
             TRY(tcx3(tc::tshape(N, H, F), o, N, F, wx.head1, H, F, eh));
         } else {
-            TRY(sgemm<false, true>(gshape(N, F, 3 * F, hn, 3 * F, W.out_w, 3 * F), eo, gctas, st));
-            TRY(sgemm<false, true>(gshape(N, H, F, o, F, W.head1_w, F), eh, gctas, st));
+            TRY(sgemm<true>(gshape(N, F, 3 * F, hn, 3 * F, W.out_w, 3 * F), eo, gctas, sms, st));
+            TRY(sgemm<true>(gshape(N, H, F, o, F, W.head1_w, F), eh, gctas, sms, st));
         }
     }
     launch(k_head, warps_grid, 256, 0, st, t, N, H, W.head2_w, W.head2_b, Ei);
@@ -2646,8 +2646,8 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         TRY(tcx3(tc::tshape(N, F, H), gat, N, H, wx.head1T, F, H, EpiGradAct{ao, F, gao, F, 0}));
         TRY(tcx3(tc::tshape(N, 3 * F, F), gao, N, F, wx.outT, 3 * F, F, EpiStore{ghn, 3 * F, 0}, bn3));
     } else {
-        TRY(sgemm<false, false>(gshape(N, F, H, gat, H, W.head1_w, F), EpiGradAct{ao, F, gao, F, 0}, gctas, st));
-        TRY(sgemm<false, false>(gshape(N, 3 * F, F, gao, F, W.out_w, 3 * F), EpiStore{ghn, 3 * F, 0}, gctas, st));
+        TRY(sgemm<false>(gshape(N, F, H, gat, H, W.head1_w, F), EpiGradAct{ao, F, gao, F, 0}, gctas, sms, st));
+        TRY(sgemm<false>(gshape(N, 3 * F, F, gao, F, W.out_w, 3 * F), EpiStore{ghn, 3 * F, 0}, gctas, sms, st));
     }
     launch(k_out_norms_bwd, N, F, 0, st, Xfin, h, ghn, lno, W.out_ln_g, N, F, gX);
     count_launch();
@@ -2680,7 +2680,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         count_launch();
         TNET_LAUNCH_CHECK();
         if (tcm) TRY(tcg(tc::tshape_classes(N, F), gdX, nbf, 9LL * N, F, lb[l].mix2T, 3 * F, F, EpiStore{gTn, F, 0}));
-        else TRY(sgemm<false, false>(gshape_classes(N, F, gdX, Lr.mix2_w), EpiStore{gTn, F, 0}, gctas, st));
+        else TRY(sgemm<false>(gshape_classes(N, F, gdX, Lr.mix2_w), EpiStore{gTn, F, 0}, gctas, sms, st));
         if (wg) TRY(wgrad_outer(rows3(gdX, Tn), wpart, wcap, gw(Gr.mix2_w), 0, sms, st));
         launch(k_T_bwd, ew, 256, 0, st, Y, M, gTn, N, F, gY, gM);
         count_launch();
@@ -2720,7 +2720,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             pf.mark(P_NODE_BWD);
             if (tcm)
                 TRY(tcg(tc::tshape_classes(N, F), gY, nbf, 9LL * N, F, lb[l].mix1T, 3 * F, F, EpiStore{gX, F, 1}));
-            else TRY(sgemm<false, false>(gshape_classes(N, F, gY, Lr.mix1_w), EpiStore{gX, F, 1}, gctas, st));
+            else TRY(sgemm<false>(gshape_classes(N, F, gY, Lr.mix1_w), EpiStore{gX, F, 1}, gctas, sms, st));
             launch(k_node_norm_bwd, ew, 256, 0, st, Xl, qn, N, F, gX);
             count_launch();
             TNET_LAUNCH_CHECK();
@@ -2744,15 +2744,15 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             pf.mark(P_MLP3_BWD);
             GemmShape q3 = gshape(maxU, 2 * F, 3 * F, gg, 3 * F, w3p(l), 2 * F);
             q3.rows_dev = nu;
-            TRY(sgemm<false, false>(q3, g3, gctas, st));
+            TRY(sgemm<false>(q3, g3, gctas, sms, st));
             pf.mark(P_MLP2_BWD);
             GemmShape q2 = gshape(maxU, F, 2 * F, ga2, 2 * F, Lr.mlp2_w, F);
             q2.rows_dev = nu;
-            TRY(sgemm<false, false>(q2, g2, gctas, st));
+            TRY(sgemm<false>(q2, g2, gctas, sms, st));
             pf.mark(P_MLP1_BWD);
             GemmShape q1 = gshape(maxU, K, F, ga1, F, Lr.mlp1_w, K);
             q1.rows_dev = nu;
-            TRY(sgemm<false, false>(q1, g1, gctas, st));
+            TRY(sgemm<false>(q1, g1, gctas, sms, st));
         }
         if (wg) {
             // gg is plane-major: map its rows back to the blob's c*3 + p order
@@ -2770,7 +2770,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         }
         pf.mark(P_NODE_BWD);
         if (tcm) TRY(tcg(tc::tshape_classes(N, F), gY, nbf, 9LL * N, F, lb[l].mix1T, 3 * F, F, EpiStore{gX, F, 1}));
-        else TRY(sgemm<false, false>(gshape_classes(N, F, gY, Lr.mix1_w), EpiStore{gX, F, 1}, gctas, st));
+        else TRY(sgemm<false>(gshape_classes(N, F, gY, Lr.mix1_w), EpiStore{gX, F, 1}, gctas, sms, st));
         launch(k_node_norm_bwd, ew, 256, 0, st, Xl, qn, N, F, gX);
         count_launch();
         TNET_LAUNCH_CHECK();
@@ -2787,12 +2787,12 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                  EpiGradAct{as1, 2 * F, gas1, 2 * F, 0}, bn2));
         TRY(tcx3(tc::tshape(N, F, 2 * F), gas1, N, 2 * F, wx.emb_mlp1T, F, 2 * F, EpiStore{gn0, F, 0}));
     } else {
-        TRY(sgemm<false, false>(gshape(N, 2 * F, 3 * F, gas2, 3 * F, W.emb_mlp2_w, 2 * F),
-                                EpiGradAct{as1, 2 * F, gas1, 2 * F, 0}, gctas, st));
-        TRY(sgemm<false, false>(gshape(N, F, 2 * F, gas1, 2 * F, W.emb_mlp1_w, F), EpiStore{gn0, F, 0}, gctas, st));
+        TRY(sgemm<false>(gshape(N, 2 * F, 3 * F, gas2, 3 * F, W.emb_mlp2_w, 2 * F),
+                                EpiGradAct{as1, 2 * F, gas1, 2 * F, 0}, gctas, sms, st));
+        TRY(sgemm<false>(gshape(N, F, 2 * F, gas1, 2 * F, W.emb_mlp1_w, F), EpiStore{gn0, F, 0}, gctas, sms, st));
     }
     if (tcm) TRY(tcg(tc::tshape_classes(N, F), gU, nbf, 9LL * N, F, emixT, 3 * F, F, EpiStore{gXraw, F, 0}));
-    else TRY(sgemm<false, false>(gshape_classes(N, F, gU, W.emb_mix_w), EpiStore{gXraw, F, 0}, gctas, st));
+    else TRY(sgemm<false>(gshape_classes(N, F, gU, W.emb_mix_w), EpiStore{gXraw, F, 0}, gctas, sms, st));
     launch(k_ln0_bwd, N, F, 0, st, Xraw, gn0, ln0, W.emb_ln_g, N, F, gXraw);
     count_launch();
     TNET_LAUNCH_CHECK();
@@ -2849,7 +2849,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         } else {
             GemmShape pg = gshape(maxU, K, 3 * F, gfu, 3 * F, W.dproj_w, K);
             pg.rows_dev = nu;
-            TRY(sgemm<false, false>(pg, EpiStore{ge, K, NL > 0}, gctas, st));
+            TRY(sgemm<false>(pg, EpiStore{ge, K, NL > 0}, gctas, sms, st));
         }
     }
     if (wg) {

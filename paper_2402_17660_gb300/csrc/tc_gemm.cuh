@@ -663,22 +663,6 @@ struct TcOperands {
     int64_t a_rows, lda, b_rows, ldb;
 };
 
-// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per device and kernel.
-// Keyed by the kernel's host-side handle and the device (a template kernel
-// used from two translation units can have a handle in each).
-inline int ensure_smem_attr(const void *kern, int bytes) {
-    static std::mutex mu;
-    static std::vector<std::pair<const void *, int>> done;  // (kernel handle, device)
-    int dev = 0;
-    TNET_CUDA_TRY(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> g(mu);
-    for (const auto &d : done)
-        if (d.first == kern && d.second == dev) return TNET_OK;
-    TNET_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    done.emplace_back(kern, dev);
-    return TNET_OK;
-}
-
 // How many clusters of `cl` CTAs of this kernel the device runs at once (0
 // if the query fails); cached per kernel handle, device and cluster size.
 inline int max_active_clusters(const void *kern, int threads, int smem, int cl) {
