@@ -515,13 +515,14 @@ struct WgradShape {
     int64_t ldb;
     int nclass;
 };
-// out[z][m][n] (+)= sum_rows A[r][m] B[r][n].  perm_f > 0: A's M = 3 perm_f
-// columns are plane-major (m = p perm_f + c); out row c*3 + p receives row m.
-int wgrad_outer(const WgradShape &P, float *partial, int64_t partial_cap, float *out, int accumulate, int sms,
+// out[z][m][n] = sum_rows A[r][m] B[r][n], and out_bias[m] = sum_rows A[r][m]
+// (one class; NULL: none).  perm_f > 0: A's M = 3 perm_f columns are
+// plane-major (m = p perm_f + c); out row c*3 + p receives row m.
+int wgrad_outer(const WgradShape &P, float *partial, int64_t partial_cap, float *out, float *out_bias, int sms,
                 cudaStream_t st, int perm_f = 0);
-// out[z][m] (+)= sum_rows A[r][m] * roww[r] (roww may be NULL); perm_f as above
-int wgrad_colsum(const WgradShape &P, const float *roww, float *partial, int64_t partial_cap, float *out,
-                 int accumulate, int sms, cudaStream_t st, int perm_f = 0);
+// out[z][m] = sum_rows A[r][m] * roww[r] (roww may be NULL)
+int wgrad_colsum(const WgradShape &P, const float *roww, float *partial, int64_t partial_cap, float *out, int sms,
+                 cudaStream_t st);
 int wgrad_layernorm(const float *gy, const float *x, const float2 *stats, int R, int C, float *partial,
                     int64_t partial_cap, float *out_g, int sms, cudaStream_t st);
 

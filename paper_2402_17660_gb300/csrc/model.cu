@@ -2656,15 +2656,10 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         launch(k_seed_atoms, (N + 255) / 256, 256, 0, st, seed, batch, N, gEi);
         count_launch();
         TNET_LAUNCH_CHECK();
-        TRY(wgrad_colsum(rows1(H, 1, N, t, H, nullptr, 0, nullptr), gEi, wpart, wcap, gw(G.head2_w), 0, sms, st));
-        TRY(wgrad_colsum(rows1(1, 1, N, gEi, 1, nullptr, 0, nullptr), nullptr, wpart, wcap, gw(G.head2_b), 0, sms,
-                         st));
-        TRY(wgrad_outer(rows1(H, F, N, gat, H, o, F, nullptr), wpart, wcap, gw(G.head1_w), 0, sms, st));
-        TRY(wgrad_colsum(rows1(H, 1, N, gat, H, nullptr, 0, nullptr), nullptr, wpart, wcap, gw(G.head1_b), 0, sms,
-                         st));
-        TRY(wgrad_outer(rows1(F, 3 * F, N, gao, F, hn, 3 * F, nullptr), wpart, wcap, gw(G.out_w), 0, sms, st));
-        TRY(wgrad_colsum(rows1(F, 1, N, gao, F, nullptr, 0, nullptr), nullptr, wpart, wcap, gw(G.out_b), 0, sms,
-                         st));
+        TRY(wgrad_colsum(rows1(H, 1, N, t, H, nullptr, 0, nullptr), gEi, wpart, wcap, gw(G.head2_w), sms, st));
+        TRY(wgrad_colsum(rows1(1, 1, N, gEi, 1, nullptr, 0, nullptr), nullptr, wpart, wcap, gw(G.head2_b), sms, st));
+        TRY(wgrad_outer(rows1(H, F, N, gat, H, o, F, nullptr), wpart, wcap, gw(G.head1_w), gw(G.head1_b), sms, st));
+        TRY(wgrad_outer(rows1(F, 3 * F, N, gao, F, hn, 3 * F, nullptr), wpart, wcap, gw(G.out_w), gw(G.out_b), sms, st));
         TRY(wgrad_layernorm(ghn, h, lno, N, 3 * F, wpart, wcap, gw(G.out_ln_g), sms, st));
     }
     // gphiu collects dE/dphi per pair (or, in table mode, dE/dd)
@@ -2681,7 +2676,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         TNET_LAUNCH_CHECK();
         if (tcm) TRY(tcg(tc::tshape_classes(N, F), gdX, nbf, 9LL * N, F, lb[l].mix2T, 3 * F, F, EpiStore{gTn, F, 0}));
         else TRY(sgemm<false>(gshape_classes(N, F, gdX, Lr.mix2_w), EpiStore{gTn, F, 0}, gctas, sms, st));
-        if (wg) TRY(wgrad_outer(rows3(gdX, Tn), wpart, wcap, gw(Gr.mix2_w), 0, sms, st));
+        if (wg) TRY(wgrad_outer(rows3(gdX, Tn), wpart, wcap, gw(Gr.mix2_w), nullptr, sms, st));
         launch(k_T_bwd, ew, 256, 0, st, Y, M, gTn, N, F, gY, gM);
         count_launch();
         TNET_LAUNCH_CHECK();
@@ -2756,17 +2751,11 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         }
         if (wg) {
             // gg is plane-major: map its rows back to the blob's c*3 + p order
-            TRY(wgrad_outer(rows1(3 * F, 2 * F, maxU, gg, 3 * F, h2, 2 * F, nu), wpart, wcap, gw(Gr.mlp3_w), 0, sms, st,
+            TRY(wgrad_outer(rows1(3 * F, 2 * F, maxU, gg, 3 * F, h2, 2 * F, nu), wpart, wcap, gw(Gr.mlp3_w), gw(Gr.mlp3_b), sms, st,
                             F));
-            TRY(wgrad_colsum(rows1(3 * F, 1, maxU, gg, 3 * F, nullptr, 0, nu), nullptr, wpart, wcap, gw(Gr.mlp3_b), 0,
-                             sms, st, F));
-            TRY(wgrad_outer(rows1(2 * F, F, maxU, ga2, 2 * F, h1, F, nu), wpart, wcap, gw(Gr.mlp2_w), 0, sms, st));
-            TRY(wgrad_colsum(rows1(2 * F, 1, maxU, ga2, 2 * F, nullptr, 0, nu), nullptr, wpart, wcap, gw(Gr.mlp2_b), 0,
-                             sms, st));
-            TRY(wgrad_outer(rows1(F, K, maxU, ga1, F, eu, K, nu), wpart, wcap, gw(Gr.mlp1_w), 0, sms, st));
-            TRY(wgrad_colsum(rows1(F, 1, maxU, ga1, F, nullptr, 0, nu), nullptr, wpart, wcap, gw(Gr.mlp1_b), 0, sms,
-                             st));
-            TRY(wgrad_outer(rows3(gY, Xn), wpart, wcap, gw(Gr.mix1_w), 0, sms, st));
+            TRY(wgrad_outer(rows1(2 * F, F, maxU, ga2, 2 * F, h1, F, nu), wpart, wcap, gw(Gr.mlp2_w), gw(Gr.mlp2_b), sms, st));
+            TRY(wgrad_outer(rows1(F, K, maxU, ga1, F, eu, K, nu), wpart, wcap, gw(Gr.mlp1_w), gw(Gr.mlp1_b), sms, st));
+            TRY(wgrad_outer(rows3(gY, Xn), wpart, wcap, gw(Gr.mix1_w), nullptr, sms, st));
         }
         pf.mark(P_NODE_BWD);
         if (tcm) TRY(tcg(tc::tshape_classes(N, F), gY, nbf, 9LL * N, F, lb[l].mix1T, 3 * F, F, EpiStore{gX, F, 1}));
@@ -2797,14 +2786,9 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     count_launch();
     TNET_LAUNCH_CHECK();
     if (wg) {
-        TRY(wgrad_outer(rows3(gU, Xraw), wpart, wcap, gw(G.emb_mix_w), 0, sms, st));
-        TRY(wgrad_outer(rows1(3 * F, 2 * F, N, gas2, 3 * F, hs1, 2 * F, nullptr), wpart, wcap, gw(G.emb_mlp2_w), 0,
-                        sms, st));
-        TRY(wgrad_colsum(rows1(3 * F, 1, N, gas2, 3 * F, nullptr, 0, nullptr), nullptr, wpart, wcap,
-                         gw(G.emb_mlp2_b), 0, sms, st));
-        TRY(wgrad_outer(rows1(2 * F, F, N, gas1, 2 * F, n0, F, nullptr), wpart, wcap, gw(G.emb_mlp1_w), 0, sms, st));
-        TRY(wgrad_colsum(rows1(2 * F, 1, N, gas1, 2 * F, nullptr, 0, nullptr), nullptr, wpart, wcap,
-                         gw(G.emb_mlp1_b), 0, sms, st));
+        TRY(wgrad_outer(rows3(gU, Xraw), wpart, wcap, gw(G.emb_mix_w), nullptr, sms, st));
+        TRY(wgrad_outer(rows1(3 * F, 2 * F, N, gas2, 3 * F, hs1, 2 * F, nullptr), wpart, wcap, gw(G.emb_mlp2_w), gw(G.emb_mlp2_b), sms, st));
+        TRY(wgrad_outer(rows1(2 * F, F, N, gas1, 2 * F, n0, F, nullptr), wpart, wcap, gw(G.emb_mlp1_w), gw(G.emb_mlp1_b), sms, st));
         TRY(wgrad_layernorm(gn0, q0, ln0, N, F, wpart, wcap, gw(G.emb_ln_g), sms, st));
     }
     pf.mark(P_EMB_EDGE_BWD);
@@ -2853,9 +2837,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         }
     }
     if (wg) {
-        TRY(wgrad_outer(rows1(3 * F, K, maxU, gfu, 3 * F, eu, K, nu), wpart, wcap, gw(G.dproj_w), 0, sms, st));
-        TRY(wgrad_colsum(rows1(3 * F, 1, maxU, gfu, 3 * F, nullptr, 0, nu), nullptr, wpart, wcap, gw(G.dproj_b), 0,
-                         sms, st));
+        TRY(wgrad_outer(rows1(3 * F, K, maxU, gfu, 3 * F, eu, K, nu), wpart, wcap, gw(G.dproj_w), gw(G.dproj_b), sms, st));
         const int zs = (int)Lw.zsplits;
         float *zpart = f32(Lw.zpart);
         launch(k_group_z, dim3(d.max_z, zs), F, 0, st, z, gA, gB, N, F, d.max_z, zs, zpart);
