@@ -367,12 +367,21 @@ __device__ __forceinline__ void mic_lower(float &x, float &y, float &z, float ax
     y = __fsub_rn(y, __fmul_rn(kb, by));
     x = __fsub_rn(x, __fmul_rn(rintf(__fdiv_rn(x, ax)), ax));
 }
+// The same, skipped for a vector well inside the brick: there every quotient
+// rounds to zero and the three steps change nothing.  Most pairs of a cell
+// list are, and the exact divisions cost more than the rest of a pair test.
+__device__ __forceinline__ void mic_fast(float &x, float &y, float &z, float ax, float bx, float by, float cx,
+                                         float cy, float cz) {
+    constexpr float kIn = 0.49f;
+    if (fabsf(x) < kIn * ax && fabsf(y) < kIn * by && fabsf(z) < kIn * cz) return;
+    mic_lower(x, y, z, ax, bx, by, cx, cy, cz);
+}
 // the same with the box as 9 floats, rows a, b, c
 __device__ __forceinline__ void mic_box(float &x, float &y, float &z, const float *__restrict__ B) {
-    mic_lower(x, y, z, B[0], B[3], B[4], B[6], B[7], B[8]);
+    mic_fast(x, y, z, B[0], B[3], B[4], B[6], B[7], B[8]);
 }
 __device__ __forceinline__ void mic(float &x, float &y, float &z, const SysInfo &s) {
-    if (s.pbc) mic_lower(x, y, z, s.L[0], s.tilt[0], s.L[1], s.tilt[1], s.tilt[2], s.L[2]);
+    if (s.pbc) mic_fast(x, y, z, s.L[0], s.tilt[0], s.L[1], s.tilt[1], s.tilt[2], s.L[2]);
 }
 
 // Radial part of the model: cosine cutoff phi(d), expnorm basis e_k(d) and

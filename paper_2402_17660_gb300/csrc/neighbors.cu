@@ -41,8 +41,29 @@ __device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *tota
     return warp_excl + x - v;
 }
 
+// What a scan hands on with its total: copies of it, and a limit the offsets
+// are clamped to (limit < 0: none), flagged as CAPACITY when the total passes
+// it (the copies keep the true total).
+struct ScanOut {
+    int32_t *total;
+    int64_t *total64;
+    int64_t limit;
+    int32_t *status;
+};
+__device__ __forceinline__ int32_t scan_clamp(int32_t v, const ScanOut &o) {
+    return o.limit >= 0 && v > o.limit ? (int32_t)o.limit : v;
+}
+__device__ __forceinline__ void scan_finish(int32_t grand, int32_t *end, const ScanOut &o) {
+    *end = scan_clamp(grand, o);
+    if (o.total) *o.total = grand;
+    if (o.total64) *o.total64 = grand;
+    if (o.limit >= 0 && grand > o.limit) set_status(o.status, TNET_ERR_CAPACITY);
+}
+
+// Exclusive scan within each tile, with the tile's sum; a lone tile is the
+// whole scan.
 __global__ void k_scan_tiles(const int32_t *__restrict__ in, int32_t *__restrict__ out, int n,
-                             int32_t *__restrict__ tile_sums, const int32_t *__restrict__ gate) {
+                             int32_t *__restrict__ tile_sums, ScanOut o, const int32_t *__restrict__ gate) {
     pdl_entry();
     if (gate && *gate == 0) return;  // gated rebuild: nothing to do
     __shared__ int32_t sm[32];
@@ -56,54 +77,40 @@ __global__ void k_scan_tiles(const int32_t *__restrict__ in, int32_t *__restrict
     }
     int32_t total;
     int32_t run = block_exclusive_scan(sum, &total, sm);
+    const bool lone = gridDim.x == 1;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        if (base + k < n) out[base + k] = run;
+        if (base + k < n) out[base + k] = lone ? scan_clamp(run, o) : run;
         run += v[k];
     }
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
+    if (threadIdx.x == 0) {
+        if (lone) scan_finish(total, out + n, o);
+        else tile_sums[blockIdx.x] = total;
+    }
 }
 
-// single block: exclusive scan of the tile sums (nt <= kScanTile)
-__global__ void k_scan_top(int32_t *__restrict__ tile_sums, int nt, int32_t *__restrict__ grand,
+// Adds to each tile the sum of the tiles before it: every block adds up those
+// tile sums itself (at most kScanTile of them, one read of a few KB from L2),
+// which saves the launch that would scan them.
+__global__ void k_scan_add(int32_t *__restrict__ out, int n, const int32_t *__restrict__ tile_sums, int nt, ScanOut o,
                            const int32_t *__restrict__ gate) {
     pdl_entry();
     if (gate && *gate == 0) return;  // gated rebuild: nothing to do
     __shared__ int32_t sm[32];
-    const int base = threadIdx.x * kScanItems;
-    int32_t v[kScanItems];
-    int32_t sum = 0;
+    const int mine = blockIdx.x;
+    int32_t before = 0;
+    for (int t = threadIdx.x; t < mine; t += blockDim.x) before += tile_sums[t];
+    int32_t offset;
+    (void)block_exclusive_scan(before, &offset, sm);
+    const int64_t base = (int64_t)mine * kScanTile;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        v[k] = (base + k < nt) ? tile_sums[base + k] : 0;
-        sum += v[k];
+        const int64_t i = base + k * kScanThreads + threadIdx.x;
+        if (i < n) out[i] = scan_clamp(out[i] + offset, o);
     }
-    int32_t total;
-    int32_t run = block_exclusive_scan(sum, &total, sm);
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        if (base + k < nt) tile_sums[base + k] = run;
-        run += v[k];
-    }
-    if (threadIdx.x == 0) *grand = total;
+    if (mine == nt - 1 && threadIdx.x == 0) scan_finish(offset + tile_sums[mine], out + n, o);
 }
 
-__global__ void k_scan_add(int32_t *__restrict__ out, int n, const int32_t *__restrict__ tile_sums,
-                           const int32_t *__restrict__ grand, int32_t *__restrict__ total_dev,
-                           int64_t *__restrict__ total64_dev, const int32_t *__restrict__ gate) {
-    pdl_entry();
-    if (gate && *gate == 0) return;  // gated rebuild: nothing to do
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] += tile_sums[i / kScanTile];
-    if (i == 0) {
-        out[n] = *grand;
-        if (total_dev) *total_dev = *grand;
-        if (total64_dev) *total64_dev = *grand;
-    }
-}
-
-// out[0..n] = exclusive scan of in[0..n), out[n] = total.  tmp needs
-// ceil(n / 4096) + 1 ints.  n <= 4096 * 4096.
 // dst[0..n) = 0 unless a gate is given and clear (the gated form of a memset)
 __global__ void k_zero_i32(int32_t *__restrict__ dst, int64_t n, const int32_t *__restrict__ gate) {
     pdl_entry();
@@ -112,105 +119,137 @@ __global__ void k_zero_i32(int32_t *__restrict__ dst, int64_t n, const int32_t *
         dst[t] = 0;
 }
 
-int scan_exclusive_i32(const int32_t *in, int32_t *out, int n, int32_t *tmp, int32_t *total_dev,
-                       int64_t *total64_dev, cudaStream_t st, const int32_t *gate) {
-    const int nt = (n + kScanTile - 1) / kScanTile;
+// out[0..n] = exclusive scan of in[0..n), out[n] = total.  tmp needs
+// ceil(n / 4096) ints.  n <= 4096 * 4096.  One launch up to 4,096 entries,
+// two above.
+static int scan_with(const int32_t *in, int32_t *out, int n, int32_t *tmp, const ScanOut &o, cudaStream_t st,
+                     const int32_t *gate) {
+    const int nt = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
     if (nt > kScanTile) return TNET_ERR_ARG;
-    const int ntl = nt > 0 ? nt : 1;
-    if (n > 0) {
-        launch(k_scan_tiles, nt, kScanThreads, 0, st, in, out, n, tmp, gate);
+    launch(k_scan_tiles, nt, kScanThreads, 0, st, in, out, n, tmp, o, gate);
+    count_launch();
+    if (nt > 1) {
+        launch(k_scan_add, nt, kScanThreads, 0, st, out, n, tmp, nt, o, gate);
         count_launch();
     }
-    else if (gate) {
-        launch(k_zero_i32, 1, 32, 0, st, tmp, 1, gate);
-        count_launch();
-    } else TNET_CUDA_TRY(cudaMemsetAsync(tmp, 0, sizeof(int32_t), st));
-    launch(k_scan_top, 1, kScanThreads, 0, st, tmp, ntl, tmp + ntl, gate);
-    count_launch();
-    launch(k_scan_add, (n + 255) / 256 + 1, 256, 0, st, out, n, tmp, tmp + ntl, total_dev, total64_dev, gate);
-    count_launch();
     TNET_LAUNCH_CHECK();
     return TNET_OK;
 }
 
+int scan_exclusive_i32(const int32_t *in, int32_t *out, int n, int32_t *tmp, int32_t *total_dev,
+                       int64_t *total64_dev, cudaStream_t st, const int32_t *gate) {
+    return scan_with(in, out, n, tmp, ScanOut{total_dev, total64_dev, -1, nullptr}, st, gate);
+}
+
 // --------------------------------------------------------------- systems ---
-__global__ void k_sys_bounds(const int32_t *__restrict__ batch, int N, int S,
-                             int32_t *__restrict__ sys_start, int32_t *__restrict__ sys_end,
-                             int32_t *status, const int32_t *__restrict__ gate) {
-    pdl_entry();
-    if (gate && *gate == 0) return;  // gated rebuild: nothing to do
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+// First and last atoms of the systems; returns atom n's system, -1 when it is
+// out of range.
+__device__ __forceinline__ int mark_bounds(const int32_t *__restrict__ batch, int n, int N, int S,
+                                           int32_t *__restrict__ sys_start, int32_t *__restrict__ sys_end,
+                                           int32_t *status) {
     const int b = batch ? batch[n] : 0;
     if (b < 0 || b >= S) {
         set_status(status, TNET_ERR_ARG);
-        return;
+        return -1;
     }
     const int bp = (n > 0) ? (batch ? batch[n - 1] : 0) : -1;
     const int bn = (n + 1 < N) ? (batch ? batch[n + 1] : 0) : S;
     if (bp > b) set_status(status, TNET_ERR_ARG);  // not sorted
     if (bp != b) sys_start[b] = n;
     if (bn != b) sys_end[b] = n + 1;
+    return b;
+}
+
+__global__ void k_sys_bounds(const int32_t *__restrict__ batch, int N, int S, int32_t *__restrict__ sys_start,
+                             int32_t *__restrict__ sys_end, int32_t *status) {
+    pdl_entry();
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (n < N) mark_bounds(batch, n, N, S, sys_start, sys_end, status);
 }
 
 int sys_bounds(const int32_t *batch, int N, int S, int32_t *sys_start, int32_t *sys_end,
                int32_t *status, cudaStream_t st) {
-    launch(k_sys_bounds, (N + 255) / 256, 256, 0, st, batch, N, S, sys_start, sys_end, status, nullptr);
+    launch(k_sys_bounds, (N + 255) / 256, 256, 0, st, batch, N, S, sys_start, sys_end, status);
     count_launch();
     TNET_LAUNCH_CHECK();
     return TNET_OK;
 }
 
-// One block per system: bounding box, finiteness, box checks and cell grid.
-__global__ void k_sys_setup(const float *__restrict__ pos, const float *__restrict__ box, float cutoff,
-                            const int32_t *__restrict__ sys_start, const int32_t *__restrict__ sys_end,
-                            SysInfo *__restrict__ info, int32_t *__restrict__ ncell, int32_t *status,
+// Order-preserving map of floats to unsigned (zero is below every value).
+__device__ __forceinline__ uint32_t float_key(float x) {
+    const uint32_t u = __float_as_uint(x);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float key_float(uint32_t k) {
+    return __uint_as_float((k & 0x80000000u) ? k & 0x7fffffffu : ~k);
+}
+
+// The system bounds with each system's extent (without a box, which gives the
+// extent itself) and the check for non-finite positions: a thread per atom, a
+// warp reduction per system the warp meets, and atomic maxima of the keys (of
+// the upper corner in inv_cell, of the lower corner's complement in origin)
+// only where they would raise the stored value.  One block per system, the
+// form before, read a 176,000-atom box at the speed of one SM (332 us; now 5).
+__global__ void k_sys_extent(const float *__restrict__ pos, const int32_t *__restrict__ batch, int N, int S,
+                             int periodic, int32_t *__restrict__ sys_start, int32_t *__restrict__ sys_end,
+                             SysInfo *__restrict__ info, int32_t *status, const int32_t *__restrict__ gate) {
+    pdl_entry();
+    if (gate && *gate == 0) return;  // gated rebuild: nothing to do
+    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = n < N ? mark_bounds(batch, n, N, S, sys_start, sys_end, status) : -1;
+    float x[3] = {0.f, 0.f, 0.f};
+    bool fine = true;
+    if (n < N) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k] = pos[3LL * n + k];
+            fine = fine && isfinite(x[k]);
+        }
+    }
+    if (!fine) set_status(status, TNET_ERR_NAN);
+    if (periodic) return;
+    unsigned todo = __ballot_sync(0xffffffffu, b >= 0 && fine);
+    while (todo) {  // the same in every lane
+        const int lead = __ffs(todo) - 1;
+        const int sys = __shfl_sync(0xffffffffu, b, lead);
+        const bool in = b == sys && fine;
+        todo &= ~__ballot_sync(0xffffffffu, in);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t key = float_key(x[k]);
+            const uint32_t hi = __reduce_max_sync(0xffffffffu, in ? key : 0u);
+            const uint32_t lo = __reduce_max_sync(0xffffffffu, in ? ~key : 0u);
+            if ((int)(threadIdx.x & 31) == lead) {
+                uint32_t *ph = reinterpret_cast<uint32_t *>(&info[sys].inv_cell[k]);
+                uint32_t *pl = reinterpret_cast<uint32_t *>(&info[sys].origin[k]);
+                if (*reinterpret_cast<volatile uint32_t *>(ph) < hi) atomicMax(ph, hi);
+                if (*reinterpret_cast<volatile uint32_t *>(pl) < lo) atomicMax(pl, lo);
+            }
+        }
+    }
+}
+
+// One thread per system: box checks and cell grid.  A lone system also gets
+// its (zero) cell offset here; `over` (the row slab's flag, or NULL) is cleared.
+__global__ void k_sys_setup(const float *__restrict__ box, float cutoff, int S, const int32_t *__restrict__ sys_start,
+                            const int32_t *__restrict__ sys_end, SysInfo *__restrict__ info,
+                            int32_t *__restrict__ ncell, int32_t *__restrict__ over, int32_t *status,
                             const int32_t *__restrict__ gate) {
     pdl_entry();
     if (gate && *gate == 0) return;  // gated rebuild: nothing to do
-    const int s = blockIdx.x;
-    const int a0 = sys_start[s], a1 = sys_end[s];
-    float lo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, hi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
-    int bad = 0;
-    for (int n = a0 + threadIdx.x; n < a1; n += blockDim.x) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const float x = pos[3LL * n + k];
-            if (!isfinite(x)) bad = 1;
-            lo[k] = fminf(lo[k], x);
-            hi[k] = fmaxf(hi[k], x);
-        }
-    }
-    __shared__ float slo[3][32], shi[3][32];
-    __shared__ int sbad;
-    if (threadIdx.x == 0) sbad = 0;
-    __syncthreads();
-    if (bad) atomicOr(&sbad, 1);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s == 0 && over) *over = 0;
+    if (s >= S) return;
+    const int na = sys_end[s] - sys_start[s];
+    float lo[3], hi[3];
+    bool any = false;  // a finite position was seen
     for (int k = 0; k < 3; ++k) {
-        float l = lo[k], h = hi[k];
-        for (int o = 16; o; o >>= 1) {
-            l = fminf(l, __shfl_xor_sync(0xffffffffu, l, o));
-            h = fmaxf(h, __shfl_xor_sync(0xffffffffu, h, o));
-        }
-        if (lane == 0) {
-            slo[k][wid] = l;
-            shi[k][wid] = h;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    const int nw = blockDim.x >> 5;
-    for (int k = 0; k < 3; ++k) {
-        for (int w = 1; w < nw; ++w) {
-            slo[k][0] = fminf(slo[k][0], slo[k][w]);
-            shi[k][0] = fmaxf(shi[k][0], shi[k][w]);
-        }
+        const uint32_t kl = __float_as_uint(info[s].origin[k]), kh = __float_as_uint(info[s].inv_cell[k]);
+        any = kh != 0u;
+        lo[k] = key_float(~kl);
+        hi[k] = key_float(kh);
     }
     SysInfo si;
-    const int na = a1 - a0;
-    if (sbad) set_status(status, TNET_ERR_NAN);
     if (box) {
         // rows a = (ax,0,0), b = (bx,by,0), c = (cx,cy,cz): rectangular or
         // triclinic.  Cells are cut along a, b, c in fractional coordinates,
@@ -241,8 +280,8 @@ __global__ void k_sys_setup(const float *__restrict__ pos, const float *__restri
         for (int k = 0; k < 3; ++k) {
             si.L[k] = 0.f;
             si.tilt[k] = 0.f;
-            const float ext = na > 0 ? (shi[k][0] - slo[k][0]) : 0.f;
-            si.origin[k] = na > 0 ? slo[k][0] : 0.f;
+            const float ext = any ? hi[k] - lo[k] : 0.f;
+            si.origin[k] = any ? lo[k] : 0.f;
             int nc = (ext > 0.f && isfinite(ext)) ? (int)floorf(ext / cutoff) : 1;
             si.nc[k] = nc < 1 ? 1 : (nc > 1024 ? 1024 : nc);
         }
@@ -256,13 +295,15 @@ __global__ void k_sys_setup(const float *__restrict__ pos, const float *__restri
         si.nc[k] = si.nc[k] / 2 > 1 ? si.nc[k] / 2 : 1;
     }
     for (int k = 0; k < 3; ++k) {  // (PBC: cells per unit of fractional coordinate)
-        const float width = si.pbc ? 1.0f : (na > 0 ? shi[k][0] - slo[k][0] : 0.f);
+        const float width = si.pbc ? 1.0f : (any ? hi[k] - lo[k] : 0.f);
         si.inv_cell[k] = width > 0.f ? si.nc[k] / width : 0.f;
     }
     si.cell_off = 0;
     si.pad = 0;
     info[s] = si;
-    ncell[s] = na > 0 ? si.nc[0] * si.nc[1] * si.nc[2] : 0;
+    const int cells = na > 0 ? si.nc[0] * si.nc[1] * si.nc[2] : 0;
+    ncell[s] = S > 1 ? cells : 0;
+    if (S == 1) ncell[1] = cells;
 }
 
 __device__ __forceinline__ int cell_index(float u, int nc) {
@@ -450,101 +491,110 @@ __global__ void k_pair_count(const float *__restrict__ pos, const int32_t *__res
                              float rc2, int32_t *__restrict__ rowcnt, const int32_t *__restrict__ gate) {
     pdl_entry();
     if (gate && *gate == 0) return;  // gated rebuild: nothing to do
-    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (i >= N) return;
-    int cnt = 0;
-    for_candidates(i, pos, batch, info, cell_off, cell_start, spos, rc2, [&](int j, bool ok) {
-        cnt += __popc(__ballot_sync(0xffffffffu, ok));
-    });
-    if ((threadIdx.x & 31) == 0) rowcnt[i] = cnt;
-}
-
-// More pairs than the capacity: flag it (n_pairs keeps the required count)
-// and clamp the row offsets to the capacity, so that the truncated list
-// never sends a reader past the end of col.
-__global__ void k_cap_check(const int64_t *__restrict__ n_pairs, int64_t cap, int32_t *__restrict__ row_ptr, int N,
-                            int32_t *status, const int32_t *__restrict__ gate) {
-    pdl_entry();
-    if (gate && *gate == 0) return;  // gated rebuild: nothing to do
-    if (*n_pairs <= cap) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) set_status(status, TNET_ERR_CAPACITY);
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t <= N; t += (int64_t)gridDim.x * blockDim.x)
-        if (row_ptr[t] > cap) row_ptr[t] = (int32_t)cap;
+    // (grid-stride: a gated launch that has nothing to do stays small)
+    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < N;
+         i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        int cnt = 0;
+        for_candidates((int)i, pos, batch, info, cell_off, cell_start, spos, rc2, [&](int, bool ok) {
+            cnt += __popc(__ballot_sync(0xffffffffu, ok));
+        });
+        if ((threadIdx.x & 31) == 0) rowcnt[i] = cnt;
+    }
 }
 
 constexpr int kFillWarps = 4;
 
+// Sorts the first cnt entries of a warp's buffer ascending (room for the next
+// power of two).
+__device__ __forceinline__ void warp_sort(int32_t *sb, int cnt, int lane) {
+    int P = 1;
+    while (P < cnt) P <<= 1;
+    for (int k = cnt + lane; k < P; k += 32) sb[k] = 0x7fffffff;
+    __syncwarp();
+    for (int k = 2; k <= P; k <<= 1) {
+        for (int jj = k >> 1; jj > 0; jj >>= 1) {
+            for (int t = lane; t < P; t += 32) {
+                const int u = t ^ jj;
+                if (u > t) {
+                    const int32_t a = sb[t], b = sb[u];
+                    const bool up = (t & k) == 0;
+                    if ((a > b) == up) {
+                        sb[t] = b;
+                        sb[u] = a;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// The CSR's columns, one warp per row, each within the row offsets (clamped to
+// the capacity when the list overflowed): copied from the row slab, or, when a
+// row did not fit it (`over`) or there is none (slab NULL), found by a second
+// candidate walk and sorted.  Grid-stride, so a gated launch that has nothing
+// to do stays small.
 __global__ void __launch_bounds__(kFillWarps * 32)
-k_pair_fill(const float *__restrict__ pos, const int32_t *__restrict__ batch, int N,
+k_pair_emit(const float *__restrict__ pos, const int32_t *__restrict__ batch, int N,
             const SysInfo *__restrict__ info, const int32_t *__restrict__ cell_off,
             const int32_t *__restrict__ cell_start, const float4 *__restrict__ spos, float rc2,
-            const int32_t *__restrict__ row_ptr, int32_t *__restrict__ col, int64_t cap,
-            const int32_t *__restrict__ gate) {
+            const int32_t *__restrict__ row_ptr, int32_t *__restrict__ col, const int32_t *__restrict__ slab,
+            const int32_t *__restrict__ over, const int32_t *__restrict__ gate) {
     pdl_entry();
     if (gate && *gate == 0) return;  // gated rebuild: nothing to do
     __shared__ int32_t buf[kFillWarps][kMaxRowSorted];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int i = blockIdx.x * kFillWarps + w;
-    if (i >= N) return;
-    const int64_t r0 = row_ptr[i];
-    const int rlen = row_ptr[i + 1] - row_ptr[i];
-    int32_t *sb = buf[w];
-    const bool in_smem = rlen <= kMaxRowSorted;
-    int cnt = 0;
-    // rlen is the count pass's result, clamped when the list overflowed the
-    // capacity: write no more than that
-    for_candidates(i, pos, batch, info, cell_off, cell_start, spos, rc2, [&](int j, bool ok) {
-        const unsigned m = __ballot_sync(0xffffffffu, ok);
-        const int slot = cnt + __popc(m & ((1u << lane) - 1u));
-        if (ok && slot < rlen) {
-            if (in_smem) sb[slot] = j;
-            else col[r0 + slot] = j;
+    const bool copy = slab && !*over;
+    for (int64_t ii = blockIdx.x * kFillWarps + w; ii < N; ii += (int64_t)gridDim.x * kFillWarps) {
+        const int i = (int)ii;
+        if (copy) {
+            const int r0 = row_ptr[i], n = row_ptr[i + 1] - r0;
+            const int32_t *src = slab + ii * kSlabWidth;
+            for (int k = lane; k < n; k += 32) col[r0 + k] = src[k];
+            continue;
         }
-        cnt += __popc(m);
-    });
-    cnt = cnt < rlen ? cnt : rlen;
-    __syncwarp();
-    if (in_smem) {
-        int P = 1;
-        while (P < cnt) P <<= 1;
-        for (int k = cnt + lane; k < P; k += 32) sb[k] = 0x7fffffff;
+        const int64_t r0 = row_ptr[i];
+        const int rlen = row_ptr[i + 1] - row_ptr[i];
+        int32_t *sb = buf[w];
+        const bool in_smem = rlen <= kMaxRowSorted;
+        int cnt = 0;
+        // rlen is the count pass's result, clamped when the list overflowed the
+        // capacity: write no more than that
+        for_candidates(i, pos, batch, info, cell_off, cell_start, spos, rc2, [&](int j, bool ok) {
+            const unsigned m = __ballot_sync(0xffffffffu, ok);
+            const int slot = cnt + __popc(m & ((1u << lane) - 1u));
+            if (ok && slot < rlen) {
+                if (in_smem) sb[slot] = j;
+                else col[r0 + slot] = j;
+            }
+            cnt += __popc(m);
+        });
+        cnt = cnt < rlen ? cnt : rlen;
         __syncwarp();
-        for (int k = 2; k <= P; k <<= 1) {
-            for (int jj = k >> 1; jj > 0; jj >>= 1) {
-                for (int t = lane; t < P; t += 32) {
-                    const int u = t ^ jj;
-                    if (u > t) {
-                        const int32_t a = sb[t], b = sb[u];
-                        const bool up = (t & k) == 0;
-                        if ((a > b) == up) {
-                            sb[t] = b;
-                            sb[u] = a;
-                        }
-                    }
+        if (in_smem) {
+            warp_sort(sb, cnt, lane);
+            for (int k = lane; k < cnt; k += 32) col[r0 + k] = sb[k];
+        } else if (lane == 0) {
+            // pathological row: sort in place in global memory
+            for (int a = 1; a < cnt; ++a) {
+                const int32_t v = col[r0 + a];
+                int b = a - 1;
+                while (b >= 0 && col[r0 + b] > v) {
+                    col[r0 + b + 1] = col[r0 + b];
+                    --b;
                 }
-                __syncwarp();
+                col[r0 + b + 1] = v;
             }
         }
-        for (int k = lane; k < cnt; k += 32) col[r0 + k] = sb[k];
-    } else if (lane == 0) {
-        // pathological row: sort in place in global memory
-        for (int a = 1; a < cnt; ++a) {
-            const int32_t v = col[r0 + a];
-            int b = a - 1;
-            while (b >= 0 && col[r0 + b] > v) {
-                col[r0 + b + 1] = col[r0 + b];
-                --b;
-            }
-            col[r0 + b + 1] = v;
-        }
+        __syncwarp();  // the buffer is read before the next row fills it
     }
 }
 
 // Single candidate pass: one warp per atom collects its neighbours (one walk
 // of the 27 cells), sorts them in shared memory and writes the sorted row to
 // the atom's slot of the slab (kSlabWidth columns), with the row's count.  A
-// row longer than kSlabWidth raises `over`; the two-pass fill then runs
-// instead of the copy (gated on it), so the result never depends on the slab.
+// row longer than kSlabWidth raises `over`; the rows are then walked again
+// instead of copied, so the result never depends on the slab.
 __global__ void __launch_bounds__(kFillWarps * 32)
 k_pair_fill_slab(const float *__restrict__ pos, const int32_t *__restrict__ batch, int N,
                  const SysInfo *__restrict__ info, const int32_t *__restrict__ cell_off,
@@ -569,44 +619,9 @@ k_pair_fill_slab(const float *__restrict__ pos, const int32_t *__restrict__ batc
         return;
     }
     __syncwarp();
-    int P = 1;
-    while (P < cnt) P <<= 1;
-    for (int k = cnt + lane; k < P; k += 32) sb[k] = 0x7fffffff;
-    __syncwarp();
-    for (int k = 2; k <= P; k <<= 1) {
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-            for (int t = lane; t < P; t += 32) {
-                const int u = t ^ jj;
-                if (u > t) {
-                    const int32_t a = sb[t], b = sb[u];
-                    const bool up = (t & k) == 0;
-                    if ((a > b) == up) {
-                        sb[t] = b;
-                        sb[u] = a;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-    }
+    warp_sort(sb, cnt, lane);
     int32_t *dst = slab + (int64_t)i * kSlabWidth;
     for (int k = lane; k < cnt; k += 32) dst[k] = sb[k];
-}
-
-// Rows of the slab into the CSR (warp per row), each within the row offsets
-// (clamped to the capacity when the list overflowed).  Skipped when a row did
-// not fit the slab: the gated two-pass fill writes the list then.
-__global__ void k_slab_copy(const int32_t *__restrict__ slab, const int32_t *__restrict__ row_ptr, int N,
-                            int32_t *__restrict__ col, const int32_t *__restrict__ over) {
-    pdl_entry();
-    if (*over) return;
-    const int lane = threadIdx.x & 31;
-    for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < N;
-         i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int r0 = row_ptr[i], n = row_ptr[i + 1] - r0;
-        const int32_t *src = slab + i * kSlabWidth;
-        for (int k = lane; k < n; k += 32) col[r0 + k] = src[k];
-    }
 }
 
 int neighbors_impl(tnet_ctx *ctx, int N, int S, const float *pos, const int32_t *batch,
@@ -634,63 +649,60 @@ int neighbors_impl(tnet_ctx *ctx, int N, int S, const float *pos, const int32_t 
         count_launch();
         return TNET_OK;
     };
-    int zrc = zero(sys_start, S);
-    if (!zrc) zrc = zero(sys_end, S);
-    if (!zrc) zrc = zero(cell_count, cells + 1LL);
-    if (!zrc) zrc = zero(cell_fill, cells);
+    // system bounds and extents (adjacent in the layout), then cell counts and
+    // fill counters (with the offsets between them, which the scan writes)
+    int zrc = zero(sys_start, (int64_t)(L.sys_ncell - L.sys_start) / 4);
+    if (!zrc) zrc = zero(cell_count, (int64_t)(L.cell_of - L.cell_count) / 4);
     if (zrc) return zrc;
+    // one candidate pass into the row slab, unless the context has none or
+    // the call is a gated rebuild (MD): then a count pass and a second walk
+    const bool one_pass = L.slab_width > 0 && !gate && N > 0;
+    int32_t *over = one_pass ? wsp<int32_t>(ctx, L.slab_over) : nullptr;
+    const int nb = (N + 255) / 256;
+    const int wave = 16 * (ctx->num_sms > 0 ? ctx->num_sms : 148);  // blocks of the grid-stride passes
+    auto rows_grid = [&](int per_block) {
+        const int g = (N + per_block - 1) / per_block;
+        return g < wave ? g : wave;
+    };
     if (N > 0) {
-        launch(k_sys_bounds, (N + 255) / 256, 256, 0, st, batch, N, S, sys_start, sys_end, status, gate);
+        launch(k_sys_extent, nb, 256, 0, st, pos, batch, N, S, box ? 1 : 0, sys_start, sys_end, info, status, gate);
         count_launch();
         TNET_LAUNCH_CHECK();
     }
-    launch(k_sys_setup, S, 256, 0, st, pos, box, cutoff, sys_start, sys_end, info, ncell, status, gate);
+    launch(k_sys_setup, (S + 127) / 128, 128, 0, st, box, cutoff, S, sys_start, sys_end, info, ncell, over, status,
+           gate);
     count_launch();
     TNET_LAUNCH_CHECK();
-    int rc = scan_exclusive_i32(ncell, ncell, S, tmp, nullptr, nullptr, st, gate);
-    if (rc) return rc;
+    int rc = TNET_OK;
+    if (S > 1 && (rc = scan_exclusive_i32(ncell, ncell, S, tmp, nullptr, nullptr, st, gate))) return rc;
     if (N > 0) {
-        launch(k_bin, (N + 255) / 256, 256, 0, st, pos, batch, N, info, ncell, cell_of, cell_count, cells, gate);
+        launch(k_bin, nb, 256, 0, st, pos, batch, N, info, ncell, cell_of, cell_count, cells, gate);
         count_launch();
         TNET_LAUNCH_CHECK();
     }
     rc = scan_exclusive_i32(cell_count, cell_start, cells, tmp, nullptr, nullptr, st, gate);
     if (rc) return rc;
-    // one candidate pass into the row slab, unless the context has none or
-    // the call is a gated rebuild (MD): then a count pass and a fill pass
-    const bool one_pass = L.slab_width > 0 && !gate && N > 0;
-    int32_t *over = one_pass ? wsp<int32_t>(ctx, L.slab_over) : nullptr;
     if (N > 0) {
-        launch(k_scatter, (N + 255) / 256, 256, 0, st, pos, N, cell_of, cell_start, cell_fill, sorted, spos, gate);
+        launch(k_scatter, nb, 256, 0, st, pos, N, cell_of, cell_start, cell_fill, sorted, spos, gate);
         count_launch();
         TNET_LAUNCH_CHECK();
-        if (one_pass) {
-            TNET_CUDA_TRY(cudaMemsetAsync(over, 0, sizeof(int32_t), st));
+        if (one_pass)
             launch(k_pair_fill_slab, (N + kFillWarps - 1) / kFillWarps, kFillWarps * 32, 0, st, pos, batch, N, info,
                    ncell, cell_start, spos, cutoff * cutoff, rowcnt, wsp<int32_t>(ctx, L.slab), over);
-        } else {
-            launch(k_pair_count, (int)(((int64_t)N * 32 + 255) / 256), 256, 0, st, pos, batch, N, info, ncell,
-                   cell_start, spos, cutoff * cutoff, rowcnt, gate);
-        }
+        else
+            launch(k_pair_count, rows_grid(8), 256, 0, st, pos, batch, N, info, ncell, cell_start, spos,
+                   cutoff * cutoff, rowcnt, gate);
         count_launch();
         TNET_LAUNCH_CHECK();
     }
-    rc = scan_exclusive_i32(rowcnt, row_ptr, N, tmp, nullptr, n_pairs_dev, st, gate);
+    // row offsets: when the pairs exceed the capacity, clamped to it (so the
+    // truncated list never sends a reader past the end of col) and flagged;
+    // n_pairs keeps the required count
+    rc = scan_with(rowcnt, row_ptr, N, tmp, ScanOut{nullptr, n_pairs_dev, cap, status}, st, gate);
     if (rc) return rc;
-    launch(k_cap_check, (N + 256) / 256 < 1024 ? (N + 256) / 256 : 1024, 256, 0, st, n_pairs_dev, cap, row_ptr, N,
-           status, gate);
-    count_launch();
-    TNET_LAUNCH_CHECK();
     if (N > 0) {
-        if (one_pass) {
-            const int nb = (int)(((int64_t)N * 32 + 255) / 256);
-            launch(k_slab_copy, nb < 4096 ? nb : 4096, 256, 0, st, wsp<int32_t>(ctx, L.slab), row_ptr, N, col, over);
-            count_launch();
-            TNET_LAUNCH_CHECK();
-        }
-        // the fill pass; in one-pass mode gated on a row that did not fit
-        launch(k_pair_fill, (N + kFillWarps - 1) / kFillWarps, kFillWarps * 32, 0, st, pos, batch, N, info, ncell,
-               cell_start, spos, cutoff * cutoff, row_ptr, col, cap, one_pass ? over : gate);
+        launch(k_pair_emit, rows_grid(kFillWarps), kFillWarps * 32, 0, st, pos, batch, N, info, ncell, cell_start,
+               spos, cutoff * cutoff, row_ptr, col, one_pass ? wsp<int32_t>(ctx, L.slab) : nullptr, over, gate);
         count_launch();
         TNET_LAUNCH_CHECK();
     }
