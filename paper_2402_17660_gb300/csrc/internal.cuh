@@ -400,6 +400,11 @@ __device__ __forceinline__ float cutoff_dphi(float d, const RadialParams &p) {
     return d < p.rc ? -0.5f * 3.14159265358979f / p.rc * sinpif(d / p.rc) : 0.0f;
 }
 // k-th basis value (including the phi factor) and its d-derivative
+// (ex = exp(alpha (rl - d)), the same for all k of a pair)
+__device__ __forceinline__ float expnorm_value(float ex, int k, const RadialParams &p, float phi) {
+    const float t = ex - (p.mu0 + k * p.dmu);
+    return phi * expf(-p.beta * t * t);
+}
 __device__ __forceinline__ void expnorm_k(float d, int k, const RadialParams &p, float phi, float dphi,
                                           float &e, float &de) {
     const float ex = expf(p.alpha * (p.rl - d));
@@ -407,6 +412,24 @@ __device__ __forceinline__ void expnorm_k(float d, int k, const RadialParams &p,
     const float rho = expf(-p.beta * t * t);
     e = phi * rho;
     de = dphi * rho + phi * rho * (2.0f * p.beta * t * p.alpha * ex);
+}
+
+// First and last atoms of the systems; returns atom n's system, -1 (and status
+// ARG) when it is out of range.
+__device__ __forceinline__ int mark_bounds(const int32_t *__restrict__ batch, int n, int N, int S,
+                                           int32_t *__restrict__ sys_start, int32_t *__restrict__ sys_end,
+                                           int32_t *status) {
+    const int b = batch ? batch[n] : 0;
+    if (b < 0 || b >= S) {
+        set_status(status, TNET_ERR_ARG);
+        return -1;
+    }
+    const int bp = (n > 0) ? (batch ? batch[n - 1] : 0) : -1;
+    const int bn = (n + 1 < N) ? (batch ? batch[n + 1] : 0) : S;
+    if (bp > b) set_status(status, TNET_ERR_ARG);  // not sorted
+    if (bp != b) sys_start[b] = n;
+    if (bn != b) sys_end[b] = n + 1;
+    return b;
 }
 
 // ------------------------------------------------------------ workspace ---
@@ -546,8 +569,6 @@ __host__ inline T *wsp(tnet_ctx *c, size_t off) {
 int scan_exclusive_i32(const int32_t *in, int32_t *out, int n, int32_t *tmp, int32_t *total_dev,
                        int64_t *total64_dev, cudaStream_t st, const int32_t *gate = nullptr);
 int tnet_kernel_setup(tnet_ctx *c);
-int sys_bounds(const int32_t *batch, int N, int S, int32_t *sys_start, int32_t *sys_end,
-               int32_t *status, cudaStream_t st);
 int64_t weight_offsets(const tnet_model_desc *d, const float *base, struct Weights *w);
 int neighbors_impl(tnet_ctx *ctx, int n_atoms, int n_systems, const float *pos, const int32_t *batch,
                    const float *box, float cutoff, int32_t *row_ptr, int32_t *col, int64_t cap,

@@ -63,6 +63,7 @@ __global__ void k_record(const float *__restrict__ vel, const float *__restrict_
     pdl_entry();
     __shared__ double sm[32];
     double acc = 0.0;
+#pragma unroll 4
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         const double vx = vel[3LL * i], vy = vel[3LL * i + 1], vz = vel[3LL * i + 2];
         acc += 0.5 * (vx * vx + vy * vy + vz * vz) / (double)inv_m[i];

@@ -95,50 +95,63 @@ __device__ __forceinline__ void pair_vec(const float *__restrict__ pos, const fl
 }
 
 // ------------------------------------------------------- graph prep ---
-// rev[e] = position of (j, i) in row j; one warp per row.
-__global__ void k_rev(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int N,
-                      int32_t *__restrict__ rev, int32_t *status) {
-    pdl_entry();
-    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (i >= N) return;
-    const int lane = threadIdx.x & 31;
-    const int e0 = row_ptr[i];
-    for (int e = e0 + lane; e < row_ptr[i + 1]; e += 32) {
-        const int j = col[e];
-        if (j < 0 || j >= N || (e > e0 && col[e - 1] >= j)) {  // rows must ascend strictly
-            set_status(status, TNET_ERR_ARG);
-            rev[e] = e;
-            continue;
-        }
-        int lo = row_ptr[j], hi = row_ptr[j + 1];
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (col[mid] < i) lo = mid + 1;
-            else hi = mid;
-        }
-        if (lo < row_ptr[j + 1] && col[lo] == i) rev[e] = lo;
-        else {
-            set_status(status, TNET_ERR_ARG);  // pair list not symmetric
-            rev[e] = e;
-        }
-    }
+// Row offsets are read clamped to [0, cap] (cap = the context's pair capacity,
+// which sizes every per-edge buffer), so a caller's CSR never sends a kernel
+// outside those buffers.
+__device__ __forceinline__ int32_t row_offset(const int32_t *__restrict__ row_ptr, int64_t t, int64_t cap) {
+    const int32_t v = row_ptr[t];
+    return v < 0 ? 0 : (v > cap ? (int32_t)cap : v);
 }
 
-// Upper (j > i) edges with d < rc, counted per row.
-__global__ void k_upper_count(const float *__restrict__ pos, const float *__restrict__ box,
-                              const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
-                              const int32_t *__restrict__ col, int N, float rc,
-                              int32_t *__restrict__ ucnt) {
+// One warp per row: the clamped copy of the row offsets that every later
+// kernel reads (offsets out of range or decreasing are reported as ARG, or
+// CAPACITY when they pass the capacity), the system bounds, the reverse edges
+// rev[e] = position of (j, i) in row j, and the count of the row's upper
+// (j > i) edges with d < rc.  Every edge starts inactive.  One launch in the
+// place of four (launches and their gaps were most of the time of small
+// systems' graph preparation).
+__global__ void k_graph_rows(const float *__restrict__ pos, const float *__restrict__ box,
+                             const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
+                             const int32_t *__restrict__ col, int N, int S, int64_t cap, float rc,
+                             int32_t *__restrict__ safe, int32_t *__restrict__ sys_start,
+                             int32_t *__restrict__ sys_end, int32_t *__restrict__ rev, int32_t *__restrict__ pair_of,
+                             int32_t *__restrict__ ucnt, int32_t *status) {
     pdl_entry();
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (i >= N) return;
     const int lane = threadIdx.x & 31;
+    const int e0 = row_offset(row_ptr, i, cap), e1 = row_offset(row_ptr, (int64_t)i + 1, cap);
+    if (lane == 0) {
+        mark_bounds(batch, i, N, S, sys_start, sys_end, status);
+        const int32_t v0 = row_ptr[i], v1 = row_ptr[i + 1];
+        if (v0 < 0 || (i == 0 && v0 != 0) || v1 < 0 || v0 > v1) set_status(status, TNET_ERR_ARG);
+        if (v0 > cap || v1 > cap) set_status(status, TNET_ERR_CAPACITY);
+        safe[i] = e0;
+        if (i == N - 1) safe[N] = e1;
+    }
     int cnt = 0;
-    for (int e0 = row_ptr[i]; e0 < row_ptr[i + 1]; e0 += 32) {
-        const int e = e0 + lane;
+    for (int eb = e0; eb < e1; eb += 32) {
+        const int e = eb + lane;
         bool up = false;
-        if (e < row_ptr[i + 1]) {
+        if (e < e1) {
             const int j = col[e];
+            int r = e;  // e itself: no reverse edge
+            if (j < 0 || j >= N || (e > e0 && col[e - 1] >= j)) {  // rows must ascend strictly
+                set_status(status, TNET_ERR_ARG);
+            } else {
+                int lo = row_offset(row_ptr, j, cap);
+                const int end = row_offset(row_ptr, (int64_t)j + 1, cap);
+                int hi = end;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (col[mid] < i) lo = mid + 1;
+                    else hi = mid;
+                }
+                if (lo < end && col[lo] == i) r = lo;
+                else set_status(status, TNET_ERR_ARG);  // pair list not symmetric
+            }
+            rev[e] = r;
+            pair_of[e] = -1;
             if (j > i && j < N) {
                 float x, y, zz;
                 pair_vec(pos, box, batch, i, j, x, y, zz);
@@ -150,9 +163,11 @@ __global__ void k_upper_count(const float *__restrict__ pos, const float *__rest
     if (lane == 0) ucnt[i] = cnt;
 }
 
+// Numbers the active undirected pairs by their upper edges and tells both
+// directed edges (a lower edge without a reverse stays inactive).
 __global__ void k_upper_assign(const float *__restrict__ pos, const float *__restrict__ box,
                                const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
-                               const int32_t *__restrict__ col, int N, float rc,
+                               const int32_t *__restrict__ col, const int32_t *__restrict__ rev, int N, float rc,
                                const int32_t *__restrict__ uoff, int32_t *__restrict__ pair_of,
                                int2 *__restrict__ uij, int32_t *__restrict__ ue) {
     pdl_entry();
@@ -173,31 +188,15 @@ __global__ void k_upper_assign(const float *__restrict__ pos, const float *__res
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, up);
-        if (e < row_ptr[i + 1] && j > i) {
-            if (up) {
-                const int u = base + __popc(m & ((1u << lane) - 1u));
-                pair_of[e] = u;
-                uij[u] = make_int2(i, j);
-                ue[u] = e;
-            } else {
-                pair_of[e] = -1;
-            }
+        if (up) {
+            const int u = base + __popc(m & ((1u << lane) - 1u));
+            pair_of[e] = u;
+            uij[u] = make_int2(i, j);
+            ue[u] = e;
+            const int r = rev[e];
+            if (r != e) pair_of[r] = u;
         }
         base += __popc(m);
-    }
-}
-
-__global__ void k_lower_assign(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                               const int32_t *__restrict__ rev, int N, int32_t *__restrict__ pair_of) {
-    pdl_entry();
-    const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    if (i >= N) return;
-    const int lane = threadIdx.x & 31;
-    for (int e = row_ptr[i] + lane; e < row_ptr[i + 1]; e += 32) {
-        const int j = col[e];
-        // rev[e] == e marks a column that is out of range or has no reverse
-        // edge (status ARG is set): the edge stays inactive
-        if (j <= i) pair_of[e] = (j == i || rev[e] == e) ? -1 : pair_of[rev[e]];
     }
 }
 
@@ -212,7 +211,7 @@ __global__ void k_edge_rbf(const float *__restrict__ pos, const float *__restric
     // a block takes groups of P = blockDim.x (<= 256) pairs: one thread per
     // pair computes its geometry, then all threads evaluate the P x K basis
     // values from it (coalesced writes of eu)
-    __shared__ float s_d[256], s_phi[256];
+    __shared__ float s_ex[256], s_phi[256];
     const int U = *nu, K = rp.K;
     const int P = blockDim.x < 256 ? blockDim.x : 256;
     for (int64_t u0 = (int64_t)blockIdx.x * P; u0 < U; u0 += (int64_t)gridDim.x * P) {
@@ -224,7 +223,7 @@ __global__ void k_edge_rbf(const float *__restrict__ pos, const float *__restric
             pair_vec(pos, box, batch, p.x, p.y, x, y, zz);
             const float d = sqrtf(norm2_rn(x, y, zz));
             const float phi = cutoff_phi(d, rp);
-            s_d[threadIdx.x] = d;
+            s_ex[threadIdx.x] = expf(rp.alpha * (rp.rl - d));
             s_phi[threadIdx.x] = phi;
             phiu[u] = phi;
             const float inv = 1.0f / d;
@@ -233,8 +232,7 @@ __global__ void k_edge_rbf(const float *__restrict__ pos, const float *__restric
         __syncthreads();
         for (int idx = threadIdx.x; idx < np * K; idx += blockDim.x) {
             const int q = idx / K, k = idx % K;
-            float e, de;
-            expnorm_k(s_d[q], k, rp, s_phi[q], 0.f, e, de);
+            const float e = expnorm_value(s_ex[q], k, rp, s_phi[q]);
             const int64_t t = (u0 + q) * K + k;
             eu[t] = e;
             opcopy_store(eu_cp, t, e);
@@ -425,18 +423,16 @@ __global__ void k_pair_geo(const float *__restrict__ pos, const float *__restric
 }
 
 // Per-element pair-embedding tables: Ta[z] = W_e[:, :F] emb[z],
-// Tb[z] = W_e[:, F:] emb[z] + b_e, so that Z_ij = Ta[z_i] + Tb[z_j].
-__global__ void k_elem_tables(const float *__restrict__ emb, const float *__restrict__ W,
-                              const float *__restrict__ b, int F, float *__restrict__ Ta,
-                              float *__restrict__ Tb) {
-    pdl_entry();
-    // block per element z; warp per output row of W (lanes along the row, so
-    // the reads of W are coalesced), a fixed-order warp reduction
-    extern __shared__ float e[];
-    const int z = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k = threadIdx.x; k < F; k += blockDim.x) e[k] = emb[(int64_t)z * F + k];
-    __syncthreads();
-    for (int r = warp; r < 2 * F; r += nw) {  // rows c (Ta) and F + c (Tb)
+// Tb[z] = W_e[:, F:] emb[z] + b_e, so that Z_ij = Ta[z_i] + Tb[z_j].  One warp
+// per output row of W (lanes along the row, so the reads of W are coalesced),
+// a fixed-order warp reduction; part of `parts` of element z's rows.
+__device__ __forceinline__ void elem_tables(int z, int part, int parts, const float *__restrict__ emb,
+                                            const float *__restrict__ W, const float *__restrict__ b, int F,
+                                            float *__restrict__ Ta, float *__restrict__ Tb) {
+    const int lane = threadIdx.x & 31, nw = (blockDim.x >> 5) * parts;
+    const float *e = emb + (int64_t)z * F;
+#pragma unroll 4
+    for (int r = part * (blockDim.x >> 5) + (threadIdx.x >> 5); r < 2 * F; r += nw) {  // rows c (Ta) and F + c (Tb)
         const int c = r % F, half = r / F;
         const float *w = W + (int64_t)c * 2 * F + half * F;
         float s = 0.f;
@@ -795,13 +791,15 @@ __global__ void k_head(const float *__restrict__ t, int N, int H, const float *_
     if (lane == 0) Ei[i] = s + b2[0];
 }
 
-// E_s = sum of E_i over the system, in FP64 (one block per system)
+// E_s = sum of E_i over the system, in FP64 (one block per system; eight loads
+// in flight per thread)
 __global__ void k_energy(const float *__restrict__ Ei, const int32_t *__restrict__ sys_start,
                          const int32_t *__restrict__ sys_end, double *__restrict__ energy) {
     pdl_entry();
     __shared__ double sm[32];
     const int s = blockIdx.x;
     double acc = 0.0;
+#pragma unroll 8
     for (int n = sys_start[s] + threadIdx.x; n < sys_end[s]; n += blockDim.x) acc += (double)Ei[n];
 #pragma unroll
     for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -1888,25 +1886,46 @@ __global__ void k_pair_vec(const float *__restrict__ pos, const float *__restric
 }
 
 // F_i = -dE/dr_i = -sum over the active edges of row i of +-Gp[pair]
-// (+ when i is the pair's first atom, r_ij = r_i - r_j), in row order.
+// (+ when i is the pair's first atom, r_ij = r_i - r_j), in row order, so the
+// inactive edges of a skin list change nothing.  Eight lanes per atom load
+// eight edges at a time and then add them up one after the other; a thread per
+// atom spent its time on one chain of dependent loads (12 us at any size up to
+// a few thousand atoms, 5 now).
+constexpr int kForceLanes = 8;
 __global__ void k_forces(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                          const int32_t *__restrict__ pair_of, const float *__restrict__ Gp, int N,
                          float *__restrict__ forces) {
     pdl_entry();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int i = (int)(t / kForceLanes), sub = (int)(t % kForceLanes);
+    const unsigned group = 0xffu << (threadIdx.x & 24);
+    if (i >= N) return;  // whole groups
     float fx = 0.f, fy = 0.f, fz = 0.f;
-    for (int e = row_ptr[i]; e < row_ptr[i + 1]; ++e) {
-        const int u = pair_of[e];
-        if (u < 0) continue;
-        const float sgn = col[e] > i ? 1.0f : -1.0f;
-        fx = fmaf(sgn, Gp[3LL * u], fx);
-        fy = fmaf(sgn, Gp[3LL * u + 1], fy);
-        fz = fmaf(sgn, Gp[3LL * u + 2], fz);
+    const int e1 = row_ptr[i + 1];
+    for (int e0 = row_ptr[i]; e0 < e1; e0 += kForceLanes) {
+        const int e = e0 + sub;
+        float gx = 0.f, gy = 0.f, gz = 0.f;
+        if (e < e1) {
+            const int u = pair_of[e];
+            if (u >= 0) {
+                const float sgn = col[e] > i ? 1.0f : -1.0f;
+                gx = sgn * Gp[3LL * u];
+                gy = sgn * Gp[3LL * u + 1];
+                gz = sgn * Gp[3LL * u + 2];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kForceLanes; ++k) {
+            fx += __shfl_sync(group, gx, k, kForceLanes);
+            fy += __shfl_sync(group, gy, k, kForceLanes);
+            fz += __shfl_sync(group, gz, k, kForceLanes);
+        }
     }
-    forces[3LL * i] = -fx;
-    forces[3LL * i + 1] = -fy;
-    forces[3LL * i + 2] = -fz;
+    if (sub == 0) {
+        forces[3LL * i] = -fx;
+        forces[3LL * i + 1] = -fy;
+        forces[3LL * i + 2] = -fz;
+    }
 }
 
 // Per-element sums of the pair-embedding adjoints (split over atom ranges):
@@ -1982,63 +2001,94 @@ __global__ void k_seed_atoms(const float *__restrict__ seed, const int32_t *__re
     if (i < N) gEi[i] = seed ? seed[batch ? batch[i] : 0] : 1.0f;
 }
 
-// Plane-major copy of each layer's last radial-MLP layer: row p*F + c of the
-// copy is row c*3 + p of the blob (weight [3F][2F], then bias [3F]), so the
-// per-pair filters g_ij and their adjoints are three contiguous F-channel
-// planes I, A, S and the message kernels read and write them coalesced.
-struct FilterRows {
-    const float *w[8], *b[8];
-};
-__global__ void k_filter_rows(const __grid_constant__ FilterRows R, int F, float *__restrict__ out) {
-    pdl_entry();
-    const int l = blockIdx.y;
-    const int64_t nw = 6LL * F * F, per = nw + 3 * F;
-    const int cols = 2 * F;
-    float *o = out + l * per;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < per; t += (int64_t)gridDim.x * blockDim.x) {
-        if (t < nw) {
-            const int r = (int)(t / cols), k = (int)(t % cols);
-            o[t] = R.w[l][(int64_t)((r % F) * 3 + r / F) * cols + k];
-        } else {
-            const int r = (int)(t - nw);
-            o[t] = R.b[l][(r % F) * 3 + r / F];
-        }
-    }
-}
-
-// Weight operands of the tensor-core modes: job j reads a [rows][cols] float
-// matrix (transposed when tr[j], for backward operands) and writes a bf16
-// copy (mode[j] = 1) or its TF32 split hi + lo (mode[j] = 2, the 3xTF32
-// GEMMs).
+// What a call makes of its weights before the first layer, in one launch: job
+// j reads a [rows][cols] float matrix and writes a bf16 copy (mode 1), its
+// TF32 split hi + lo (mode 2, the 3xTF32 GEMMs) or an FP32 copy (mode 3),
+// transposed when tr[j] (backward operands).  perm[j] = F > 0: row p*F + c of
+// the result is row c*3 + p of the source (the last radial layer, whose blob
+// order is channel-major), so the per-pair filters g_ij and their adjoints are
+// three contiguous F-channel planes I, A, S and the message kernels read and
+// write them coalesced.  32 x 32 tiles through shared memory, so a transposed
+// matrix is read and written along its rows.  The blocks past the jobs form
+// the element tables (see elem_tables).
+// Latency-bound; as three launches (filter rows, weight copies, tables with
+// one block per element) 57 us a call at F = 128, now 7.
 constexpr int kMaxCvtJobs = 128;
+constexpr int kElemParts = 8;  // blocks per element
 struct CvtJobs {
     const float *src[kMaxCvtJobs];
     void *hi[kMaxCvtJobs];
     void *lo[kMaxCvtJobs];
-    int rows[kMaxCvtJobs], cols[kMaxCvtJobs], tr[kMaxCvtJobs], mode[kMaxCvtJobs];
+    int rows[kMaxCvtJobs], cols[kMaxCvtJobs];
+    short perm[kMaxCvtJobs];
+    signed char tr[kMaxCvtJobs], mode[kMaxCvtJobs];
     int n;
+};
+struct ElemTables {
+    const float *emb, *W, *b;
+    int F, max_z;
+    float *Ta, *Tb;
 };
 struct WOp {  // a weight operand: bf16 matrix, or fp32 high part + residual
     const void *b;
     const void *blo;
 };
-__global__ void k_cvt_weights(const __grid_constant__ CvtJobs J) {
+__global__ void __launch_bounds__(256) k_prep_weights(const __grid_constant__ CvtJobs J, ElemTables E) {
     pdl_entry();
+    __shared__ float tile[32][33];
     const int j = blockIdx.y;
-    if (j >= J.n) return;
-    const int R = J.rows[j], C = J.cols[j];
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < R * C; t += gridDim.x * blockDim.x) {
-        const int r = t / C, c = t % C;
-        const float v = J.src[j][t];
-        const int64_t o = J.tr[j] ? (int64_t)c * R + r : (int64_t)t;
+    if (j >= J.n) {
+        const int q = (j - J.n) * gridDim.x + blockIdx.x;
+        if (q / kElemParts < E.max_z)
+            elem_tables(q / kElemParts, q % kElemParts, kElemParts, E.emb, E.W, E.b, E.F, E.Ta, E.Tb);
+        return;
+    }
+    const int R = J.rows[j], C = J.cols[j], pf = J.perm[j];
+    const int tc = (C + 31) / 32, tiles = ((R + 31) / 32) * tc;
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    auto put = [&](int64_t o, float v) {
         if (J.mode[j] == 1) {
             static_cast<__nv_bfloat16 *>(J.hi[j])[o] = __float2bfloat16_rn(v);
+        } else if (J.mode[j] == 3) {
+            static_cast<float *>(J.hi[j])[o] = v;
         } else {
             float hi, lo;
             tf32_split(v, hi, lo);
             static_cast<float *>(J.hi[j])[o] = hi;
             static_cast<float *>(J.lo[j])[o] = lo;
         }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int r0 = (t / tc) * 32, c0 = (t % tc) * 32;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int r = r0 + row + 8 * k, c = c0 + lane;
+            if (r < R && c < C) {
+                const int sr = pf > 0 ? (r % pf) * 3 + r / pf : r;
+                const float v = J.src[j][(int64_t)sr * C + c];
+                if (J.tr[j]) tile[row + 8 * k][lane] = v;
+                else put((int64_t)r * C + c, v);
+            }
+        }
+        if (!J.tr[j]) continue;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int c = c0 + row + 8 * k, r = r0 + lane;
+            if (r < R && c < C) put((int64_t)c * R + r, tile[lane][row + 8 * k]);
+        }
+    }
+}
+
+// FP32 plane-major copies of a layer's last radial weight and bias
+static void filter_row_jobs(CvtJobs &J, const LayerW &L, int F, float *w3p, float *b3p) {
+    const float *src[2] = {L.mlp3_w, L.mlp3_b};
+    float *dst[2] = {w3p, b3p};
+    for (int q = 0; q < 2; ++q) {
+        const int j = J.n++;
+        J.src[j] = src[q]; J.hi[j] = dst[q]; J.lo[j] = nullptr;
+        J.rows[j] = 3 * F; J.cols[j] = q ? 1 : 2 * F; J.perm[j] = (short)F; J.tr[j] = 0; J.mode[j] = 3;
     }
 }
 
@@ -2103,25 +2153,6 @@ static inline int grid_for(int64_t n, int threads, int num_sms) {
         if (rc_) return rc_;        \
     } while (0)
 
-// Row offsets clamped to [0, cap] (cap = the context's pair capacity, which
-// sizes every per-edge buffer): a caller's CSR can then never send a kernel
-// outside those buffers.  Offsets outside the range or decreasing are
-// reported as ARG (or CAPACITY when they pass the capacity).
-__global__ void k_rows_in_range(const int32_t *__restrict__ row_ptr, int N, int64_t cap,
-                                int32_t *__restrict__ safe, int32_t *status) {
-    pdl_entry();
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t <= N; t += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = row_ptr[t];
-        int32_t w = v < 0 ? 0 : v;
-        if (w > cap) {
-            w = (int32_t)cap;
-            set_status(status, TNET_ERR_CAPACITY);
-        }
-        if (v < 0 || (t == 0 && v != 0) || (t > 0 && row_ptr[t - 1] > v)) set_status(status, TNET_ERR_ARG);
-        safe[t] = w;
-    }
-}
-
 // Radial-function tables (radial_table = n > 0): the projections f (table 0)
 // and each layer's filter g (table 1 + l) as [n-1][4][3F] Hermite
 // coefficients on the grid d_k = k h, h = rc/(n - 1).  f, g are functions of
@@ -2147,9 +2178,10 @@ int radial_tables_impl(tnet_ctx *ctx, const float *wblob, cudaStream_t st) {
     auto w3p = [&](int l) { return f32(Lw.w3p) + l * w3_per; };
     auto b3p = [&](int l) { return f32(Lw.w3p) + l * w3_per + 6LL * F * F; };
     if (NL > 0) {
-        FilterRows FR{};
-        for (int l = 0; l < NL; ++l) { FR.w[l] = W.layer[l].mlp3_w; FR.b[l] = W.layer[l].mlp3_b; }
-        launch(k_filter_rows, dim3(48, NL), 256, 0, st, FR, F, f32(Lw.w3p));
+        CvtJobs J;
+        J.n = 0;
+        for (int l = 0; l < NL; ++l) filter_row_jobs(J, W.layer[l], F, w3p(l), b3p(l));
+        launch(k_prep_weights, dim3(64, J.n), 256, 0, st, J, ElemTables{});
         count_launch();
         TNET_LAUNCH_CHECK();
     }
@@ -2216,10 +2248,6 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     int32_t *rev = i32(Lw.rev), *pair_of = i32(Lw.pair_of), *ucnt = i32(Lw.ucnt);
     // every kernel below reads the clamped copy of the row offsets
     int32_t *row_ptr = i32(Lw.rp_safe);
-    launch(k_rows_in_range, (N + 256) / 256 < 1024 ? (N + 256) / 256 : 1024, 256, 0, st, row_ptr_in, N,
-           ctx->max_pairs, row_ptr, status);
-    count_launch();
-    TNET_LAUNCH_CHECK();
     int32_t *nu = i32(Lw.nu), *ue = i32(Lw.ue);
     int2 *uij = wsp<int2>(ctx, Lw.uedge);
     float *Ta = f32(Lw.Ta), *Tb = f32(Lw.Tb);
@@ -2288,16 +2316,11 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     const int64_t w3_per = 6LL * F * F + 3 * F;
     auto w3p = [&](int l) { return f32(Lw.w3p) + l * w3_per; };  // plane-major mlp3 weight
     auto b3p = [&](int l) { return f32(Lw.w3p) + l * w3_per + 6LL * F * F; };
-    if (NL > 0 && !tab) {
-        FilterRows FR{};
-        for (int l = 0; l < NL; ++l) { FR.w[l] = W.layer[l].mlp3_w; FR.b[l] = W.layer[l].mlp3_b; }
-        launch(k_filter_rows, dim3(48, NL), 256, 0, st, FR, F, f32(Lw.w3p));
-        count_launch();
-        TNET_LAUNCH_CHECK();
-    }
+    CvtJobs J;
+    J.n = 0;
+    if (!tab)
+        for (int l = 0; l < NL; ++l) filter_row_jobs(J, W.layer[l], F, w3p(l), b3p(l));
     if (tcm) {
-        CvtJobs J;
-        J.n = 0;
         char *wb = ctx->ws + Lw.wbf;
         int64_t woff = 0;  // bytes
         auto alloc = [&](int64_t elems, int esz) {
@@ -2307,13 +2330,14 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         };
         // forward operands keep the (out, in) = K-major layout; backward
         // operands are transposed
-        auto job_m = [&](const float *src, int rows, int cols, int tr, int mode) {
+        auto job_m = [&](const float *src, int rows, int cols, int tr, int mode, int perm = 0) {
             WOp w{};
             const int esz = mode == 1 ? 2 : 4;
             void *hi = alloc((int64_t)rows * cols, esz);
             void *lo = mode == 2 ? alloc((int64_t)rows * cols, esz) : nullptr;
             J.src[J.n] = src; J.hi[J.n] = hi; J.lo[J.n] = lo;
-            J.rows[J.n] = rows; J.cols[J.n] = cols; J.tr[J.n] = tr; J.mode[J.n] = mode;
+            J.rows[J.n] = rows; J.cols[J.n] = cols; J.tr[J.n] = (signed char)tr; J.mode[J.n] = (signed char)mode;
+            J.perm[J.n] = (short)perm;
             ++J.n;
             w.b = hi;
             w.blo = lo;
@@ -2331,7 +2355,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                 J.src[J.n] = src + q * ff;
                 J.hi[J.n] = hi + q * ff * esz;
                 J.lo[J.n] = lo ? lo + q * ff * esz : nullptr;
-                J.rows[J.n] = F; J.cols[J.n] = F; J.tr[J.n] = 1; J.mode[J.n] = prec;
+                J.rows[J.n] = F; J.cols[J.n] = F; J.tr[J.n] = 1; J.mode[J.n] = (signed char)prec; J.perm[J.n] = 0;
                 ++J.n;
             }
             return WOp{hi, lo};
@@ -2346,9 +2370,9 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             lb[l].mix2T = job_classes_T(Lr.mix2_w);
             if (tab) continue;  // no per-pair radial MLP
             lb[l].mlp2 = job(Lr.mlp2_w, 2 * F, F, 0);
-            lb[l].mlp3 = job(w3p(l), 3 * F, 2 * F, 0);
+            lb[l].mlp3 = job_m(Lr.mlp3_w, 3 * F, 2 * F, 0, prec, F);
             lb[l].mlp2T = job(Lr.mlp2_w, 2 * F, F, 1);
-            lb[l].mlp3T = job(w3p(l), 3 * F, 2 * F, 1);
+            lb[l].mlp3T = job_m(Lr.mlp3_w, 3 * F, 2 * F, 1, prec, F);
             lb[l].mlp1 = job3(Lr.mlp1_w, F, K, 0);
             lb[l].mlp1T = job3(Lr.mlp1_w, F, K, 1);
         }
@@ -2366,8 +2390,12 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             wx.head1 = job3(W.head1_w, H, F, 0);
             wx.head1T = job3(W.head1_w, H, F, 1);
         }
-        if (woff > Lw.wbf_bytes || J.n > kMaxCvtJobs) return TNET_ERR_WORKSPACE;
-        launch(k_cvt_weights, dim3(64, J.n), 256, 0, st, J);
+        if (woff > Lw.wbf_bytes) return TNET_ERR_WORKSPACE;
+    }
+    {
+        const ElemTables et{W.emb, W.emb2_w, W.emb2_b, F, d.max_z, Ta, Tb};
+        const int extra = (d.max_z * kElemParts + 63) / 64;  // grid rows of the element tables
+        launch(k_prep_weights, dim3(64, J.n + extra), 256, 0, st, J, et);
         count_launch();
         TNET_LAUNCH_CHECK();
     }
@@ -2404,18 +2432,15 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         }
         return tcx3(P, A32, a_rows, lda, w, b_rows, ldb, epi, bn);
     };
-    TNET_CUDA_TRY(cudaMemsetAsync(sys_start, 0, sizeof(int32_t) * S, st));
-    TNET_CUDA_TRY(cudaMemsetAsync(sys_end, 0, sizeof(int32_t) * S, st));
-    TRY(sys_bounds(batch, N, S, sys_start, sys_end, status, st));
-    launch(k_rev, warps_grid, 256, 0, st, row_ptr, col, N, rev, status);
-    count_launch();
-    launch(k_upper_count, warps_grid, 256, 0, st, pos, box, batch, row_ptr, col, N, rp.rc, ucnt);
+    // (sys_start and sys_end are adjacent in the layout)
+    TNET_CUDA_TRY(cudaMemsetAsync(sys_start, 0, Lw.sysinfo - Lw.sys_start, st));
+    launch(k_graph_rows, warps_grid, 256, 0, st, pos, box, batch, row_ptr_in, col, N, S, ctx->max_pairs, rp.rc, row_ptr,
+           sys_start, sys_end, rev, pair_of, ucnt, status);
     count_launch();
     TNET_LAUNCH_CHECK();
     TRY(scan_exclusive_i32(ucnt, ucnt, N, i32(Lw.scan_tmp), nu, nullptr, st));
-    launch(k_upper_assign, warps_grid, 256, 0, st, pos, box, batch, row_ptr, col, N, rp.rc, ucnt, pair_of, uij, ue);
-    count_launch();
-    launch(k_lower_assign, warps_grid, 256, 0, st, row_ptr, col, rev, N, pair_of);
+    launch(k_upper_assign, warps_grid, 256, 0, st, pos, box, batch, row_ptr, col, rev, N, rp.rc, ucnt, pair_of, uij,
+           ue);
     count_launch();
     TNET_LAUNCH_CHECK();
     float *eu = f32(Lw.eu), *phiu = f32(Lw.phiu), *fu = f32(Lw.fu);
@@ -2437,8 +2462,6 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         launch(k_edge_rbf, pair_grid, 256, 0, st, pos, box, batch, uij, nu, maxU, rp, eu, phiu, geo, eu_cp);
         count_launch();
     }
-    launch(k_elem_tables, d.max_z, 256, sizeof(float) * F, st, W.emb, W.emb2_w, W.emb2_b, F, Ta, Tb);
-    count_launch();
     TNET_LAUNCH_CHECK();
     if (!tab) {   // radial projections f^p = W^p e(d) + b^p, once per undirected pair
         // FP32 in both modes: K = num_rbf is small, and rounding the narrow
@@ -2629,7 +2652,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     }
     launch(k_head, warps_grid, 256, 0, st, t, N, H, W.head2_w, W.head2_b, Ei);
     count_launch();
-    launch(k_energy, S, 256, 0, st, Ei, sys_start, sys_end, energy);
+    launch(k_energy, S, N / S > 1024 ? 1024 : 128, 0, st, Ei, sys_start, sys_end, energy);
     count_launch();
     TNET_LAUNCH_CHECK();
     if (!forces && !grad_w) return TNET_OK;
@@ -2854,7 +2877,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     launch(k_pair_vec, pair_grid, 256, 0, st, pos, box, batch, uij, ue, rev, nu, rp, tab ? nullptr : ge,
            (NL > 0 && !tab) ? gphiu : nullptr, edge_g, tab ? gphiu : nullptr, Gp);
     count_launch();
-    launch(k_forces, (N + 127) / 128, 128, 0, st, row_ptr, col, pair_of, Gp, N, forces);
+    launch(k_forces, (unsigned)(((int64_t)N * kForceLanes + 127) / 128), 128, 0, st, row_ptr, col, pair_of, Gp, N, forces);
     count_launch();
     TNET_LAUNCH_CHECK();
     return TNET_OK;

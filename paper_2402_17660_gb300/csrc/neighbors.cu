@@ -142,39 +142,6 @@ int scan_exclusive_i32(const int32_t *in, int32_t *out, int n, int32_t *tmp, int
 }
 
 // --------------------------------------------------------------- systems ---
-// First and last atoms of the systems; returns atom n's system, -1 when it is
-// out of range.
-__device__ __forceinline__ int mark_bounds(const int32_t *__restrict__ batch, int n, int N, int S,
-                                           int32_t *__restrict__ sys_start, int32_t *__restrict__ sys_end,
-                                           int32_t *status) {
-    const int b = batch ? batch[n] : 0;
-    if (b < 0 || b >= S) {
-        set_status(status, TNET_ERR_ARG);
-        return -1;
-    }
-    const int bp = (n > 0) ? (batch ? batch[n - 1] : 0) : -1;
-    const int bn = (n + 1 < N) ? (batch ? batch[n + 1] : 0) : S;
-    if (bp > b) set_status(status, TNET_ERR_ARG);  // not sorted
-    if (bp != b) sys_start[b] = n;
-    if (bn != b) sys_end[b] = n + 1;
-    return b;
-}
-
-__global__ void k_sys_bounds(const int32_t *__restrict__ batch, int N, int S, int32_t *__restrict__ sys_start,
-                             int32_t *__restrict__ sys_end, int32_t *status) {
-    pdl_entry();
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n < N) mark_bounds(batch, n, N, S, sys_start, sys_end, status);
-}
-
-int sys_bounds(const int32_t *batch, int N, int S, int32_t *sys_start, int32_t *sys_end,
-               int32_t *status, cudaStream_t st) {
-    launch(k_sys_bounds, (N + 255) / 256, 256, 0, st, batch, N, S, sys_start, sys_end, status);
-    count_launch();
-    TNET_LAUNCH_CHECK();
-    return TNET_OK;
-}
-
 // Order-preserving map of floats to unsigned (zero is below every value).
 __device__ __forceinline__ uint32_t float_key(float x) {
     const uint32_t u = __float_as_uint(x);
