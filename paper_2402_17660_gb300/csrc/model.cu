@@ -1728,100 +1728,133 @@ __global__ void k_emb_bwd_pairs(const float4 *__restrict__ geo, const int32_t *_
 }
 
 // The same adjoint with four consecutive channels per lane (F = 128, exact
-// mode, forces only): every gathered row of gX_raw, the pair's projections
-// and the element tables are float4 loads, a quarter of the load and address
-// instructions of the strided form above.  Offsets are 32-bit (the host
-// checks the sizes).
+// mode, forces only), and both uses of the pair taken together: with
+// q = Z_ij g_i +- Z_ji g_j per coordinate (minus for the skew part, which is
+// odd in u), dE/df = phi (q basis), and one sum per pair serves dE/dphi and
+// dE/du of the two uses, which enter the forces only as their sum and their
+// difference:
+//   pair_g[u] = (dE/dphi(i,j) + dE/dphi(j,i), dE/du(i,j) - dE/du(j,i)).
+// 48 operations per channel instead of 110, two channels per instruction.
+// Warps take runs of consecutive pairs, which share their first atom: row i of
+// gX_raw and its table rows stay in registers until i changes, so a pair
+// gathers only row j.  The runs go round the warps, so the pairs in flight
+// sweep the atoms together and the gathered rows stay in L2 (one long run per
+// warp: 2.77 ms).  Bound by the latency of the gathers (6.1 KB a pair through
+// L2), HBM at 57%.  96,000-atom water (2.58 M pairs): 3.04 -> 2.06 ms; 3,000
+// atoms 105 -> 54 us.  Offsets are 32-bit (the host checks the sizes).
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+constexpr int kPairRun = 32;    // consecutive pairs a warp takes at a time
+constexpr int kPairBlocks = 4;  // resident blocks per SM, and the grid: one wave
+struct F4 {  // four FP32 values as two packed pairs
+    uint64_t v[2];
+};
+__device__ __forceinline__ F4 ld4p(const float *__restrict__ p) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+    return F4{{t.x, t.y}};
+}
 template <int F>
-__global__ void __launch_bounds__(256) k_emb_bwd_pairs_v4(const float4 *__restrict__ geo,
+__global__ void __launch_bounds__(128, kPairBlocks) k_emb_bwd_pairs_v4(const float4 *__restrict__ geo,
                                                           const int32_t *__restrict__ z,
-                                                          const int2 *__restrict__ uij, const int32_t *__restrict__ ue,
-                                                          const int32_t *__restrict__ rev,
+                                                          const int2 *__restrict__ uij,
                                                           const int32_t *__restrict__ nu, int N, int max_z,
                                                           const float *__restrict__ fu, const float *__restrict__ Ta,
                                                           const float *__restrict__ Tb,
                                                           const float *__restrict__ gXraw, float *__restrict__ gfu,
-                                                          float4 *__restrict__ edge_g, OpCopy gfu_cp) {
+                                                          float4 *__restrict__ pair_g) {
     pdl_entry();
     static_assert(F == 128, "one float4 per lane and row");
     const int lane = threadIdx.x & 31;
     const int U = *nu;
     const uint32_t c4 = 4u * lane;
-    for (int64_t uu = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; uu < U;
-         uu += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int u = (int)uu;
-        const int2 p = uij[u];
-        const int i = p.x, j = p.y;
-        const float4 gu = geo[u];
-        const float ux = gu.x, uy = gu.y, uz = gu.z, phi = gu.w;
-        const float bxx = ux * ux - (1.0f / 3.0f), byy = uy * uy - (1.0f / 3.0f);
-        const float bxy = ux * uy, bxz = ux * uz, byz = uy * uz;
-        int zi = z[i], zj = z[j];
-        zi = (zi < 0 || zi >= max_z) ? 0 : zi;
-        zj = (zj < 0 || zj >= max_z) ? 0 : zj;
-        const uint32_t fb = (uint32_t)u * 3u * F + c4;
-        const float4 f0 = ld4(fu + fb), f1 = ld4(fu + fb + F), f2 = ld4(fu + fb + 2 * F);
-        float4 gi[9], gj[9];
+    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t share = (U + warps - 1) / warps;
+    const int per = (int)(share < kPairRun ? share : kPairRun);
+    int cur = -1;
+    F4 gi[9], tai, tbi;
+    auto elem = [&](int a) {
+        const int q = z[a];
+        return (q < 0 || q >= max_z) ? 0 : q;
+    };
+    for (int64_t u0 = wid * per; u0 < U; u0 += warps * per) {
+        const int u_end = (int)(u0 + per < U ? u0 + per : U);
+        for (int u = (int)u0; u < u_end; ++u) {
+            const int2 p = uij[u];
+            const float4 gu = geo[u];
+            if (p.x != cur) {  // the same in every lane
+                cur = p.x;
+                const uint32_t zi = (uint32_t)elem(cur) * F + c4;
+                tai = ld4p(Ta + zi);
+                tbi = ld4p(Tb + zi);
 #pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            gi[q] = ld4(gXraw + coord_row(q, (uint32_t)i, (uint32_t)N, F) + c4);
-            gj[q] = ld4(gXraw + coord_row(q, (uint32_t)j, (uint32_t)N, F) + c4);
-        }
-        const float4 tai = ld4(Ta + (uint32_t)zi * F + c4), tbj = ld4(Tb + (uint32_t)zj * F + c4);
-        const float4 taj = ld4(Ta + (uint32_t)zj * F + c4), tbi = ld4(Tb + (uint32_t)zi * F + c4);
-        float a_phi = 0.f, ax = 0.f, ay = 0.f, az = 0.f;
-        float b_phi = 0.f, bx = 0.f, by = 0.f, bz = 0.f;
-        const float vx = -ux, vy = -uy, vz = -uz;
-        float o[3][4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            auto el = [k](const float4 &v) { return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w)); };
-            float g[9], h[9];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) {
-                g[q] = el(gi[q]);
-                h[q] = el(gj[q]);
+                for (int q = 0; q < 9; ++q) gi[q] = ld4p(gXraw + coord_row(q, (uint32_t)cur, (uint32_t)N, F) + c4);
             }
-            const float F0 = el(f0), F1 = el(f1), F2 = el(f2);
-            const float Zij = el(tai) + el(tbj), Zji = el(taj) + el(tbi);
-            const float gc0 = g[0];
-            const float gcA = g[1] * ux + g[2] * uy + g[3] * uz;
-            const float gcS = g[4] * bxx + g[5] * byy + g[6] * bxy + g[7] * bxz + g[8] * byz;
-            a_phi = fmaf(Zij, gc0 * F0 + gcA * F1 + gcS * F2, a_phi);
-            {
-                const float cA = phi * Zij * F1, cS = phi * Zij * F2;
-                ax += cA * g[1] + cS * (2.f * ux * g[4] + uy * g[6] + uz * g[7]);
-                ay += cA * g[2] + cS * (2.f * uy * g[5] + ux * g[6] + uz * g[8]);
-                az += cA * g[3] + cS * (ux * g[7] + uy * g[8]);
-            }
-            const float hc0 = h[0];
-            const float hcA = h[1] * vx + h[2] * vy + h[3] * vz;
-            const float hcS = h[4] * bxx + h[5] * byy + h[6] * bxy + h[7] * bxz + h[8] * byz;
-            b_phi = fmaf(Zji, hc0 * F0 + hcA * F1 + hcS * F2, b_phi);
-            {
-                const float cA = phi * Zji * F1, cS = phi * Zji * F2;
-                bx += cA * h[1] + cS * (2.f * vx * h[4] + vy * h[6] + vz * h[7]);
-                by += cA * h[2] + cS * (2.f * vy * h[5] + vx * h[6] + vz * h[8]);
-                bz += cA * h[3] + cS * (vx * h[7] + vy * h[8]);
-            }
-            o[0][k] = phi * (Zij * gc0 + Zji * hc0);
-            o[1][k] = phi * (Zij * gcA + Zji * hcA);
-            o[2][k] = phi * (Zij * gcS + Zji * hcS);
-        }
+            const uint32_t zj = (uint32_t)elem(p.y) * F + c4;
+            const uint32_t fb = (uint32_t)u * 3u * F + c4;
+            F4 h[9];
 #pragma unroll
-        for (int pl = 0; pl < 3; ++pl) {
-            st4(gfu + fb + pl * F, make_float4(o[pl][0], o[pl][1], o[pl][2], o[pl][3]));
-            if (gfu_cp.mode) {
+            for (int q = 0; q < 9; ++q) h[q] = ld4p(gXraw + coord_row(q, (uint32_t)p.y, (uint32_t)N, F) + c4);
+            const F4 f0 = ld4p(fu + fb), f1 = ld4p(fu + fb + F), f2 = ld4p(fu + fb + 2 * F);
+            const F4 taj = ld4p(Ta + zj), tbj = ld4p(Tb + zj);
+            const float ux = gu.x, uy = gu.y, uz = gu.z;
+            auto dup = [](float x) { return f2_pack(x, x); };
+            const uint64_t x2 = dup(ux), y2 = dup(uy), z2 = dup(uz), xx2 = dup(2.f * ux), yy2 = dup(2.f * uy);
+            const uint64_t bxx = dup(ux * ux - (1.0f / 3.0f)), byy = dup(uy * uy - (1.0f / 3.0f));
+            const uint64_t bxy = dup(ux * uy), bxz = dup(ux * uz), byz = dup(uy * uz);
+            const uint64_t ph2 = dup(gu.w), neg = dup(-1.f);
+            uint64_t sp = 0, sx = 0, sy = 0, sz = 0;
+            F4 o[3];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) opcopy_store(gfu_cp, fb + pl * F + k, o[pl][k]);
+            for (int k = 0; k < 2; ++k) {
+                const uint64_t zij = f2_add(tai.v[k], tbj.v[k]), zji = f2_add(taj.v[k], tbi.v[k]);
+                const uint64_t nji = f2_mul(zji, neg);
+                uint64_t q[9];
+#pragma unroll
+                for (int c = 0; c < 9; ++c)
+                    q[c] = f2_fma((c >= 1 && c < 4) ? nji : zji, h[c].v[k], f2_mul(zij, gi[c].v[k]));
+                const uint64_t q1 = f2_fma(z2, q[3], f2_fma(y2, q[2], f2_mul(x2, q[1])));
+                const uint64_t q2 = f2_fma(byz, q[8], f2_fma(bxz, q[7], f2_fma(bxy, q[6], f2_fma(byy, q[5], f2_mul(bxx, q[4])))));
+                sp = f2_fma(f2.v[k], q2, f2_fma(f1.v[k], q1, f2_fma(f0.v[k], q[0], sp)));
+                const uint64_t dx = f2_fma(z2, q[7], f2_fma(y2, q[6], f2_mul(xx2, q[4])));
+                const uint64_t dy = f2_fma(z2, q[8], f2_fma(x2, q[6], f2_mul(yy2, q[5])));
+                const uint64_t dz = f2_fma(y2, q[8], f2_mul(x2, q[7]));
+                sx = f2_fma(f2.v[k], dx, f2_fma(f1.v[k], q[1], sx));
+                sy = f2_fma(f2.v[k], dy, f2_fma(f1.v[k], q[2], sy));
+                sz = f2_fma(f2.v[k], dz, f2_fma(f1.v[k], q[3], sz));
+                o[0].v[k] = f2_mul(ph2, q[0]);
+                o[1].v[k] = f2_mul(ph2, q1);
+                o[2].v[k] = f2_mul(ph2, q2);
             }
-        }
-        a_phi = warp_sum(a_phi); ax = warp_sum(ax); ay = warp_sum(ay); az = warp_sum(az);
-        b_phi = warp_sum(b_phi); bx = warp_sum(bx); by = warp_sum(by); bz = warp_sum(bz);
-        if (lane == 0) {
-            const int e = ue[u];
-            edge_g[e] = make_float4(a_phi, ax, ay, az);
-            edge_g[rev[e]] = make_float4(b_phi, bx, by, bz);
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl)
+                *reinterpret_cast<ulonglong2 *>(gfu + fb + pl * F) = make_ulonglong2(o[pl].v[0], o[pl].v[1]);
+            // four warp sums in six exchanges: each step halves the values a lane
+            // carries, so lanes 0, 8, 16, 24 end with one sum each
+            auto fold = [](uint64_t v) {
+                const float2 t = f2_unpack(v);
+                return t.x + t.y;
+            };
+            float a0 = fold(sp), a1 = fold(sx), a2 = fold(sy), a3 = fold(sz);
+            const bool hi = lane & 16, hj = lane & 8;
+            const float r0 = __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 16), r1 = __shfl_xor_sync(0xffffffffu, hi ? a1 : a3, 16);
+            a0 = (hi ? a2 : a0) + r0;
+            a1 = (hi ? a3 : a1) + r1;
+            const float r2 = __shfl_xor_sync(0xffffffffu, hj ? a0 : a1, 8);
+            a0 = (hj ? a1 : a0) + r2;
+            a0 += __shfl_xor_sync(0xffffffffu, a0, 4);
+            a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+            a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+            if ((lane & 7) == 0)
+                reinterpret_cast<float *>(pair_g)[4LL * u + (lane >> 3)] = lane == 0 ? a0 : gu.w * a0;
         }
     }
 }
@@ -1830,13 +1863,15 @@ __global__ void __launch_bounds__(256) k_emb_bwd_pairs_v4(const float4 *__restri
 //   dE/dd   = sum_k ge[u][k] de_k/dd + (gphi_mlp[u] + gphi(i,j) + gphi(j,i)) dphi/dd
 //             + dEdd[u]  (the tabulated functions' share, table mode)
 //   dE/du   = gu(i,j) - gu(j,i)                       (u_ji = -u_ij)
+// (both from edge_g, or already taken together from pair_g)
 //   Gp[u]   = dE/dd u + (dE/du - (dE/du . u) u) / d
 __global__ void k_pair_vec(const float *__restrict__ pos, const float *__restrict__ box,
                            const int32_t *__restrict__ batch, const int2 *__restrict__ uij,
                            const int32_t *__restrict__ ue, const int32_t *__restrict__ rev,
                            const int32_t *__restrict__ nu, RadialParams rp, const float *__restrict__ ge,
                            const float *__restrict__ gphi_mlp, const float4 *__restrict__ edge_g,
-                           const float *__restrict__ dEdd, float *__restrict__ Gp) {
+                           const float4 *__restrict__ pair_g, const float *__restrict__ dEdd,
+                           float *__restrict__ Gp) {
     pdl_entry();
     const int U = *nu;
     // one thread per pair (a warp keeps 32 pairs' loads in flight); the
@@ -1870,13 +1905,19 @@ __global__ void k_pair_vec(const float *__restrict__ pos, const float *__restric
             }
         }
         {
-            const int e = ue[u];
-            const float4 a = edge_g[e], b = edge_g[rev[e]];
-            const float gphi = (gphi_mlp ? gphi_mlp[u] : 0.f) + a.x + b.x;
+            float4 g;
+            if (pair_g) {
+                g = pair_g[u];
+            } else {
+                const int e = ue[u];
+                const float4 a = edge_g[e], b = edge_g[rev[e]];
+                g = make_float4(a.x + b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+            }
+            const float gphi = (gphi_mlp ? gphi_mlp[u] : 0.f) + g.x;
             const float gd = s + gphi * dphi + (dEdd ? dEdd[u] : 0.f);
             const float inv = 1.0f / d;
             const float ux = x * inv, uy = y * inv, uz = zz * inv;
-            const float gx = a.y - b.y, gy = a.z - b.z, gz = a.w - b.w;
+            const float gx = g.y, gy = g.z, gz = g.w;
             const float dot = gx * ux + gy * uy + gz * uz;
             Gp[3 * u] = gd * ux + (gx - dot * ux) * inv;
             Gp[3 * u + 1] = gd * uy + (gy - dot * uy) * inv;
@@ -2830,9 +2871,10 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     else                                                                                                     \
         launch(k_emb_bwd_pairs<CPL, false>, pair_grid, 256, 0, st, geo, z, uij, ue, rev, nu, N, d.max_z, fu, tf0, Ta, \
                                                              Tb, gXraw, gfu, edge_g, gfu_cp, nullptr)
-    if (!wg && !tab && warp_rows)
-        launch(k_emb_bwd_pairs_v4<128>, pair_grid, 256, 0, st, geo, z, uij, ue, rev, nu, N, d.max_z, fu, Ta, Tb, gXraw,
-               gfu, edge_g, gfu_cp);
+    const bool by_pair = !wg && !tab && warp_rows;
+    if (by_pair)
+        launch(k_emb_bwd_pairs_v4<128>, kPairBlocks * sms, 128, 0, st, geo, z, uij, nu, N, d.max_z, fu, Ta, Tb, gXraw, gfu,
+               edge_g);
     else
     switch (F / 32) {
         case 2: EMB_BWD(2); break;
@@ -2875,7 +2917,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     if (!forces) return TNET_OK;
     pf.mark(P_FORCES);
     launch(k_pair_vec, pair_grid, 256, 0, st, pos, box, batch, uij, ue, rev, nu, rp, tab ? nullptr : ge,
-           (NL > 0 && !tab) ? gphiu : nullptr, edge_g, tab ? gphiu : nullptr, Gp);
+           (NL > 0 && !tab) ? gphiu : nullptr, edge_g, by_pair ? edge_g : nullptr, tab ? gphiu : nullptr, Gp);
     count_launch();
     launch(k_forces, (unsigned)(((int64_t)N * kForceLanes + 127) / 128), 128, 0, st, row_ptr, col, pair_of, Gp, N, forces);
     count_launch();
