@@ -321,18 +321,28 @@ __device__ __forceinline__ void group_sync(int g) {
     }
 }
 
-// SiLU and its derivative (fast-math exp and divide: a few ulp, far inside
-// the FP32 path's error budget)
-__device__ __forceinline__ float silu_f(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
-__device__ __forceinline__ float silu_grad_f(float x) {
-    const float s = __fdividef(1.0f, 1.0f + __expf(-x));
-    return s * (1.0f + x * (1.0f - s));
+// Logistic function, SiLU and its derivative: e^-x as 2^(-x log2 e) and the
+// reciprocal on the special-function unit, a few ulp, far inside the FP32
+// path's error budget.  Subnormals are flushed (.ftz), which changes nothing
+// here: 1 + e^-x is at least 1, and a reciprocal that underflows is 0 either
+// way; without it every evaluation carries the range tests of both
+// instructions.
+__device__ __forceinline__ float sigmoid_f(float x) {
+    float e, r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * -1.4426950408889634f));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+    return r;
 }
+__device__ __forceinline__ float silu_f(float x) { return x * sigmoid_f(x); }
 // silu(x) and silu'(x) from one sigmoid evaluation
 __device__ __forceinline__ void silu_and_grad_f(float x, float &v, float &d) {
-    const float s = __fdividef(1.0f, 1.0f + __expf(-x));
+    const float s = sigmoid_f(x);
     v = x * s;
     d = s * (1.0f + x * (1.0f - s));
+}
+__device__ __forceinline__ float silu_grad_f(float x) {
+    const float s = sigmoid_f(x);
+    return s * (1.0f + x * (1.0f - s));
 }
 
 // ------------------------------------------------------------- geometry ---
