@@ -123,7 +123,7 @@ int build_layout(const tnet_model_desc *d, int N, int S, int64_t E, Layout *L) {
     L->ga2 = take(f * U * 2 * F * rm);
     L->ga1 = take(f * U * F * rm);
     L->ge = take(f * U * K * rm);
-    L->gphiu = take(f * U);
+    L->gphiu = take(f * 2 * U);  // one sum per channel half
     L->gvec = take(f * 3 * E);
     L->fu = take(f * U * 3 * F * rm);
     L->gfu = take(f * U * 3 * F * rm);

@@ -1123,24 +1123,34 @@ __global__ void __launch_bounds__(F * RB, (512 / (F * RB)) > 0 ? 512 / (F * RB) 
     }
 }
 
-// ------------------------------------------- warp-per-row message kernels ---
-// The same sums as k_message and k_message_bwd (exact mode), with one warp per
-// row and four consecutive channels per lane: every gathered row of F floats
-// is one float4 load per lane (F / 128 of them), so the load, address and
-// index instructions per edge fall by four against a thread per channel, the
-// dE/dphi sum of a pair is one warp reduction (no shared-memory partials or
-// block barriers), and each warp keeps two edges' gathers in flight.  Built
-// for F = 128 (the adjoint's per-warp staging of row i is 9 KB).  Offsets are
-// 32-bit (the host checks 9 N F < 2^31).
-constexpr int kV4Warps = 4;  // warps (rows in flight) per block
-
-__device__ __forceinline__ float4 ld4(const float *__restrict__ p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ void st4(float *__restrict__ p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
-__device__ __forceinline__ void fma4(float4 &a, float s, const float4 &x) {
-    a.x = fmaf(s, x.x, a.x); a.y = fmaf(s, x.y, a.y); a.z = fmaf(s, x.z, a.z); a.w = fmaf(s, x.w, a.w);
+// ------------------------------------------------ staged message kernels ---
+// The same sums as k_message and k_message_bwd (exact mode, F = 128), with the
+// gathered node rows shared by a group of rows.  A block takes up to G
+// consecutive rows at a time.  One warp merges the rows' column lists (they
+// ascend), three copy each distinct column's node rows into a ring of
+// shared-memory slots, once for the whole group: consecutive atoms share most
+// of their neighbours (in a water box 12 rows use a column 4.4 times, 6 rows
+// 3.2 times).  Consumer warps, one per row with four channels a lane (the
+// adjoint: two per row with two, so that row i's own Y and gM stay in
+// registers), take the slots their row needs in column order, the same order
+// of additions as the gathers.  The pair's a3 rows, which nothing else in the
+// group uses, come through a ring per warp, a few edges ahead.
+// What bounded the gathers was not bandwidth but latency (long-scoreboard
+// stalls, 12 warps with 24 row loads each in flight, 115 SM cycles an edge with
+// every pipe below half); both rings keep their loads ahead of the warps.  Now
+// the consumers' own instructions bound the adjoint (half of the issue slots,
+// three to four warps a scheduler) and the merge (about 250 cycles a column)
+// the messages.  Per launch, 96,000 atoms (5.2 M edges): messages 2.00 -> 1.46
+// ms, adjoint 4.16 -> 3.46; 3,000 atoms 76 -> 55 us and 148 -> 140.
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
-__device__ __forceinline__ void fma4v(float4 &a, const float4 &s, const float4 &x) {
-    a.x = fmaf(s.x, x.x, a.x); a.y = fmaf(s.y, x.y, a.y); a.z = fmaf(s.z, x.z, a.z); a.w = fmaf(s.w, x.w, a.w);
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
 }
 // first element (in floats) of coordinate row q (0..8) of atom n in a node
 // tensor laid out as I rows [0, N), A rows [N, 4N), S rows [4N, 9N)
@@ -1150,291 +1160,400 @@ __device__ __forceinline__ uint32_t coord_row(int q, uint32_t n, uint32_t N, uin
 // plane p (I, A, S) of coordinate q
 __device__ __forceinline__ constexpr int plane_of(int q) { return q == 0 ? 0 : (q < 4 ? 1 : 2); }
 
-template <int F>
-__global__ void __launch_bounds__(32 * kV4Warps, 3) k_message_v4(const int32_t *__restrict__ row_ptr,
-                                                              const int32_t *__restrict__ col,
-                                                              const int32_t *__restrict__ pair_of,
-                                                              const float *__restrict__ a3,
-                                                              const float *__restrict__ phiu,
-                                                              const float *__restrict__ Y, int N,
-                                                              float *__restrict__ M) {
-    pdl_entry();
-    static_assert(F % 128 == 0, "four channels per lane");
-    constexpr int PER = F / 128;  // float4 per lane per row
-    constexpr int KM = 2;         // edges in flight per warp
-    const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * kV4Warps;
-    for (int i = blockIdx.x * kV4Warps + (threadIdx.x >> 5); i < N; i += nw) {
-        float4 m[9][PER];
+// 2 NP consecutive channels of a lane as NP packed pairs
+template <int NP>
+struct Ch {
+    uint64_t v[NP];
+};
+template <int NP>
+__device__ __forceinline__ Ch<NP> ldc(const float *__restrict__ p) {
+    Ch<NP> r;
+    if constexpr (NP == 2) {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+        r.v[0] = t.x; r.v[1] = t.y;
+    } else {
+        r.v[0] = *reinterpret_cast<const unsigned long long *>(p);
+    }
+    return r;
+}
+template <int NP>
+__device__ __forceinline__ void stc(float *__restrict__ p, const Ch<NP> &c) {
+    if constexpr (NP == 2) *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(c.v[0], c.v[1]);
+    else *reinterpret_cast<unsigned long long *>(p) = c.v[0];
+}
+template <int NP>
+__device__ __forceinline__ void opcopy_store_c(const OpCopy &o, int64_t idx, const Ch<NP> &c) {
+    if (o.mode != 1) return;
 #pragma unroll
-        for (int q = 0; q < 9; ++q)
-#pragma unroll
-            for (int r = 0; r < PER; ++r) m[q][r] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int e0 = row_ptr[i], e1 = row_ptr[i + 1];
-        for (int eb = e0; eb < e1; eb += 32) {
-            const int n = e1 - eb < 32 ? e1 - eb : 32;
-            int u_l = -1, j_l = 0;
-            float ph_l = 0.f;
-            if (lane < n) {
-                u_l = pair_of[eb + lane];
-                j_l = col[eb + lane];
-                if (u_l >= 0) ph_l = phiu[u_l];
-            }
-            for (int k0 = 0; k0 < n; k0 += KM) {
-                int uu[KM], jj[KM];
-                float ph[KM];
-#pragma unroll
-                for (int k = 0; k < KM; ++k) {
-                    const int src = k0 + k < n ? k0 + k : 0;
-                    uu[k] = __shfl_sync(0xffffffffu, u_l, src);
-                    jj[k] = __shfl_sync(0xffffffffu, j_l, src);
-                    ph[k] = __shfl_sync(0xffffffffu, ph_l, src);
-                    if (k0 + k >= n) uu[k] = -1;
-                }
-                float4 g[KM][3][PER], y[KM][9][PER];
-#pragma unroll
-                for (int k = 0; k < KM; ++k) {
-                    if (uu[k] < 0) continue;
-                    const uint32_t ab = (uint32_t)uu[k] * 3u * F + 4u * lane;
-#pragma unroll
-                    for (int p = 0; p < 3; ++p)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) g[k][p][r] = ld4(a3 + ab + p * F + 128 * r);
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        const uint32_t yb = coord_row(q, (uint32_t)jj[k], (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) y[k][q][r] = ld4(Y + yb + 128 * r);
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < KM; ++k) {
-                    if (uu[k] < 0) continue;
-#pragma unroll
-                    for (int p = 0; p < 3; ++p)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) {
-                            float4 &v = g[k][p][r];
-                            v.x = silu_f(v.x) * ph[k]; v.y = silu_f(v.y) * ph[k];
-                            v.z = silu_f(v.z) * ph[k]; v.w = silu_f(v.w) * ph[k];
-                        }
-#pragma unroll
-                    for (int q = 0; q < 9; ++q)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) fma4v(m[q][r], g[k][plane_of(q)][r], y[k][q][r]);
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const uint32_t mb = coord_row(q, (uint32_t)i, (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-            for (int r = 0; r < PER; ++r) st4(M + mb + 128 * r, m[q][r]);
-        }
+    for (int k = 0; k < NP; ++k) {
+        const float2 t = f2_unpack(c.v[k]);
+        *reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(o.p) + idx + 2 * k) =
+            __floats2bfloat162_rn(t.x, t.y);
     }
 }
+// asynchronous copy of a lane's 16 or 8 bytes, in the thread's copy groups
+template <int BYTES>
+__device__ __forceinline__ void cp_lane(void *dst, const void *src) {
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+// one arrival of this thread on a barrier once its copies so far have landed
+__device__ __forceinline__ void cp_arrive(uint64_t *bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
 
-// Adjoint, warp per row: gY_i += sum_j g_ij gM_j over the row; for the upper
-// edges (j > i) also dE/dg of the pair, dE/da3 = dE/dg phi SiLU'(a3) and
-// dE/dphi += sum dE/dg SiLU(a3) (one warp reduction, in the lane order).
-// Row i's own Y and gM sit in shared memory (per warp) for the upper edges'
-// dot products.  One lower edge's gathers are in flight at a time, and an
-// upper edge gathers gM_j (with a3) and then Y_j, which keeps the kernel
-// within 255 registers without spills (two blocks, eight warps per SM).
-template <int F, int MINB>
-__global__ void __launch_bounds__(32 * kV4Warps, MINB)
-    k_message_bwd_v4(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                     const int32_t *__restrict__ pair_of, const float *__restrict__ Y,
-                     const float *__restrict__ gM, const float *__restrict__ a3, const float *__restrict__ phiu,
-                     int N, float *__restrict__ gY, OpCopy gY_cp, float *__restrict__ ga3, OpCopy ga3_cp,
-                     float *__restrict__ gphi) {
+// Shape of the staged kernels: warps per row, rows per group, slots per stage
+// and stages of the node ring, depth of the a3 rings, copying warps, and the
+// edges of a row listed at a time (longer rows take several passes over the
+// group).  Sixteen warps leave 128 registers to each, which the adjoint needs
+// (row i's Y, gM and sum, 54 of them): with twenty and 96 it spills, and with
+// nearly all of L1 given to shared memory a spill goes to L2 (15.3 ms against
+// 6.9).  Measured at 96,000 atoms, both launches of a call: messages with 16
+// rows (twenty warps) 3.00 ms, 13 rows 3.06, 12 rows 2.91; adjoint with 7 rows
+// and one copying warp 7.50, 6 and three 6.91, 5 and two 8.27.
+template <int F, bool BWD>
+struct MsgTile {
+    static constexpr int HW = BWD ? 2 : 1, G = BWD ? 6 : 12, NS = BWD ? 4 : 8, ST = BWD ? 4 : 3, D = BWD ? 4 : 3;
+    static constexpr int CAP = 100, C = G * HW, CW = 3, THREADS = 32 * (C + 1 + CW), FH = F / HW, NP = FH / 64;
+    static constexpr int NODE = 9 * F * 4, SLOT = (BWD ? 2 : 1) * NODE, A3 = 3 * FH * 4;
+    static constexpr int o_ring = ST * NS * SLOT, o_col = o_ring + C * D * A3, o_u = o_col + 2 * G * CAP * 4;
+    static constexpr int o_ph = o_u + 2 * G * CAP * 4, o_cnt = o_ph + 2 * G * CAP * 4, o_more = o_cnt + 2 * G * 4;
+    static constexpr int o_mask = o_more + 2 * G * 4, o_j = o_mask + ST * NS * 4, o_meta = o_j + ST * NS * 4, o_bar = (o_meta + ST * 4 + 15) & ~15;
+    static constexpr int BARS = 3 * ST + 4, SMEM = o_bar + 8 * BARS;
+    static_assert(NP >= 1 && FH == 64 * NP && SMEM <= 232448 - 256, "shared memory above 227 KB");
+};
+
+// BWD false: V = Y, out = M, M_i = sum_j g_ij Y_j.
+// BWD true: V = gM, V2 = Y, out = gY (added to), and per upper edge (j > i)
+// dE/dg = <gM_i, Y_j> + <gM_j, Y_i>, ga3 = dE/dg phi SiLU'(a3) and gphi[half][u]
+// += sum dE/dg SiLU(a3) over the warp's channels.
+// Every wait is bounded: on expiry the block records TIMEOUT, the roles stop
+// and each warp waits for its own copies.
+template <int F, bool BWD>
+__global__ void __launch_bounds__(MsgTile<F, BWD>::THREADS, 1)
+    k_message_tile(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                   const int32_t *__restrict__ pair_of, const float *__restrict__ a3, const float *__restrict__ phiu,
+                   const float *__restrict__ V, const float *__restrict__ V2, int N, int R, float *__restrict__ out,
+                   OpCopy out_cp, float *__restrict__ ga3, OpCopy ga3_cp, float *__restrict__ gphi,
+                   int64_t gphi_stride, int32_t *status) {
     pdl_entry();
-    static_assert(F % 128 == 0, "four channels per lane");
-    constexpr int PER = F / 128;
-    constexpr int KM = 1;   // lower edges in flight per warp
-    __shared__ float4 s_own[kV4Warps][2][9][F / 4];  // row i's Y and gM
+    using T = MsgTile<F, BWD>;
+    constexpr int NP = T::NP, FH = T::FH, G = T::G, HW = T::HW, NS = T::NS, ST = T::ST, D = T::D, C = T::C, CAP = T::CAP;
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ int s_abort;
+    int *l_col = reinterpret_cast<int *>(sm + T::o_col);          // [2][G][CAP] columns of the active edges
+    int *l_u = reinterpret_cast<int *>(sm + T::o_u);              // their pairs
+    float *l_ph = reinterpret_cast<float *>(sm + T::o_ph);        // and cutoff factors
+    int *l_cnt = reinterpret_cast<int *>(sm + T::o_cnt);          // [2][G] edges listed
+    int *l_more = reinterpret_cast<int *>(sm + T::o_more);        // [2][G] the row has edges beyond this pass
+    uint32_t *s_mask = reinterpret_cast<uint32_t *>(sm + T::o_mask);  // [ST][NS] rows that use the slot
+    int *s_j = reinterpret_cast<int *>(sm + T::o_j);              // [ST][NS] the slot's atom; ~j: its V2 rows too
+    int *s_meta = reinterpret_cast<int *>(sm + T::o_meta);        // [ST] slots filled, + 256 on a pass's last stage
+                                                                  // (+ 512 on the block's last)
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + T::o_bar), *empty = full + ST, *l_full = empty + ST, *l_empty = l_full + 2, *named = l_empty + 2;
+    volatile int *abort_flag = &s_abort;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    float4(*s_y)[F / 4] = s_own[w][0];
-    float4(*s_gm)[F / 4] = s_own[w][1];
-    const int nw = gridDim.x * kV4Warps;
-    for (int i = blockIdx.x * kV4Warps + w; i < N; i += nw) {
-        // row i's Y and gM into shared memory, one coordinate row at a time
-#pragma unroll 1
-        for (int q = 0; q < 9; ++q) {
-            const uint32_t b = coord_row(q, (uint32_t)i, (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-            for (int r = 0; r < PER; ++r) {
-                s_y[q][lane + 32 * r] = ld4(Y + b + 128 * r);
-                s_gm[q][lane + 32 * r] = ld4(gM + b + 128 * r);
-            }
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < ST; ++s) {
+            tc::mbar_init(&full[s], 32 * T::CW + 1);
+            tc::mbar_init(&empty[s], C);
+            tc::mbar_init(&named[s], 1);
         }
-        float4 acc[9][PER];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const uint32_t b = coord_row(q, (uint32_t)i, (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-            for (int r = 0; r < PER; ++r) acc[q][r] = ld4(gY + b + 128 * r);
+        for (int b = 0; b < 2; ++b) {
+            tc::mbar_init(&l_full[b], G);
+            tc::mbar_init(&l_empty[b], C + 1);
         }
-        // each lane reads back only what it wrote: no barrier needed
-        const int e0 = row_ptr[i], e1 = row_ptr[i + 1];
-        int eu = e0, hi = e1;  // first edge with col > i
-        while (eu < hi) {
-            const int mid = (eu + hi) >> 1;
-            if (col[mid] <= i) eu = mid + 1;
-            else hi = mid;
+        s_abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    const int groups = (N + R - 1) / R;
+    bool ok = true;
+    auto wait = [&](uint64_t *bar, uint32_t parity) {
+        if (!tc::mbar_wait(bar, parity, abort_flag)) {
+            if (!*abort_flag) set_status(status, TNET_ERR_TIMEOUT);
+            *abort_flag = 1;
+            ok = false;
         }
-        for (int eb = e0; eb < e1; eb += 32) {
-            const int n = e1 - eb < 32 ? e1 - eb : 32;
-            int u_l = -1, j_l = 0;
-            float ph_l = 0.f;
-            if (lane < n) {
-                u_l = pair_of[eb + lane];
-                j_l = col[eb + lane];
-                if (u_l >= 0) ph_l = phiu[u_l];
-            }
-            const int nl = eu - eb < 0 ? 0 : (eu - eb < n ? eu - eb : n);  // lower edges of the batch
-            for (int k0 = 0; k0 < nl; k0 += KM) {
-                int uu[KM], jj[KM];
-                float ph[KM];
-#pragma unroll
-                for (int k = 0; k < KM; ++k) {
-                    const int src = k0 + k < nl ? k0 + k : 0;
-                    uu[k] = __shfl_sync(0xffffffffu, u_l, src);
-                    jj[k] = __shfl_sync(0xffffffffu, j_l, src);
-                    ph[k] = __shfl_sync(0xffffffffu, ph_l, src);
-                    if (k0 + k >= nl) uu[k] = -1;
+        return ok;
+    };
+    // whether any row of list buffer b goes on beyond its pass
+    auto any_more = [&](int b) { return __any_sync(0xffffffffu, lane < G && l_more[b * G + lane] != 0); };
+
+    if (w == C) {  // ------------------------------------- merges the rows' columns
+        int n_stage = 0;
+        int g = blockIdx.x;
+        for (int t = 0; ok && g < groups; ++t) {
+            const int b = t & 1;
+            if (!wait(&l_full[b], (t >> 1) & 1)) break;
+            const bool more = any_more(b);
+            const int g_next = more ? g : g + gridDim.x;
+            // this lane's row: its next two columns, the one after them loaded
+            // ahead of each step (two entries of INT_MAX end a list)
+            const int *mine = l_col + (b * G + (lane < G ? lane : 0)) * CAP;
+            int cur = lane < G ? mine[0] : 0x7fffffff, nxt = lane < G ? mine[1] : 0x7fffffff, k = 2, slot = 0;
+            if (cur == 0x7fffffff) nxt = cur;
+            for (;;) {
+                const int s = n_stage % ST;
+                if (slot == 0 && n_stage >= ST && !wait(&empty[s], ((n_stage / ST) - 1) & 1)) break;
+                const int after = mine[k < CAP ? k : CAP - 1];
+                const int j = __reduce_min_sync(0xffffffffu, cur);
+                const bool end = j == 0x7fffffff;
+                if (!end) {
+                    // no branches on the lane: every lane writes the same words
+                    const bool use = cur == j;
+                    const unsigned rows = __ballot_sync(0xffffffffu, use);
+                    cur = use ? nxt : cur;
+                    nxt = use ? (nxt == 0x7fffffff ? nxt : after) : nxt;
+                    k += use;
+                    s_mask[s * NS + slot] = rows;
+                    // Y_j serves upper edges alone
+                    s_j[s * NS + slot] = BWD && j > g * R + __ffs(rows) - 1 ? ~j : j;
+                    ++slot;
                 }
-                float4 g[KM][3][PER], gm[KM][9][PER];
+                if (end || slot == NS) {
+                    __syncwarp();
+                    if (lane == 0) {
+                        s_meta[s] = slot | (end ? 256 : 0) | (end && g_next >= groups ? 512 : 0);
+                        tc::mbar_arrive(&named[s]);
+                        tc::mbar_arrive(&full[s]);
+                    }
+                    ++n_stage;
+                    slot = 0;
+                    if (end) break;
+                }
+            }
+            if (!ok) break;
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&l_empty[b]);
+            g = g_next;
+        }
+    } else if (w > C) {  // -------------------------------- copy the node rows in
+        for (int n_stage = 0;; ++n_stage) {
+            const int s = n_stage % ST;
+            if (!wait(&named[s], (n_stage / ST) & 1)) break;
+            const int meta = s_meta[s];
+            for (int slot = w - C - 1; slot < (meta & 255); slot += T::CW) {
+                int j = s_j[s * NS + slot];
+                const bool both = j < 0;
+                if (both) j = ~j;
+                uint8_t *dst = sm + (s * NS + slot) * T::SLOT + 16 * lane;
+                const float *rI = V + (int64_t)j * F + 4 * lane, *rA = V + ((int64_t)N + 3LL * j) * F + 4 * lane,
+                            *rS = V + (4LL * N + 5LL * j) * F + 4 * lane;
+                if (4 * lane < F) {
 #pragma unroll
-                for (int k = 0; k < KM; ++k) {
-                    if (uu[k] < 0) continue;
-                    const uint32_t ab = (uint32_t)uu[k] * 3u * F + 4u * lane;
+                    for (int q = 0; q < 9; ++q)
+                        cp_lane<16>(dst + q * F * 4, q == 0 ? rI : (q < 4 ? rA + (q - 1) * F : rS + (q - 4) * F));
+                    if (both) {
+                        const int64_t d = V2 - V;
 #pragma unroll
-                    for (int p = 0; p < 3; ++p)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) g[k][p][r] = ld4(a3 + ab + p * F + 128 * r);
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        const uint32_t b = coord_row(q, (uint32_t)jj[k], (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) gm[k][q][r] = ld4(gM + b + 128 * r);
+                        for (int q = 0; q < 9; ++q)
+                            cp_lane<16>(dst + T::NODE + q * F * 4,
+                                        d + (q == 0 ? rI : (q < 4 ? rA + (q - 1) * F : rS + (q - 4) * F)));
                     }
                 }
+            }
+            cp_arrive(&full[s]);  // each lane, once its copies have landed
+            if (meta & 512) break;
+        }
+        cp_wait<0>();  // own copies land before the block exits
+    } else {  // ----------------------------------------------------- consumers
+        const int r = w / HW, half = w % HW;
+        const uint32_t c0 = half * FH + 2 * NP * lane;
+        // the lane's own a3 values: D edges of three planes
+        uint8_t *ring = sm + T::o_ring + w * D * T::A3 + 8 * NP * lane;
+        if (BWD) gphi += half * gphi_stride;
+        int e_next = 0, e_end = 0;  // edges of the row not listed yet
+        auto row_of = [&](int g) {
+            const int64_t i = (int64_t)g * R + r;
+            return r < R && g < groups && i < N ? (int)i : -1;
+        };
+        auto open_row = [&](int g) {
+            const int i = row_of(g);
+            e_next = i >= 0 ? row_ptr[i] : 0;
+            e_end = i >= 0 ? row_ptr[i + 1] : 0;
+        };
+        // the row's next active edges into list buffer b (both halves keep
+        // count, the first writes)
+        auto list_row = [&](int b) {
+            int n = 0;
+            const int at = (b * G + r) * CAP;
+            while (e_next < e_end && n <= CAP - 34) {
+                const int e = e_next + lane;
+                const int u = e < e_end ? pair_of[e] : -1;
+                const int j = e < e_end ? col[e] : 0;
+                const unsigned m = __ballot_sync(0xffffffffu, u >= 0);
+                if (half == 0 && u >= 0) {
+                    const int q = at + n + __popc(m & ((1u << lane) - 1u));
+                    l_col[q] = j;
+                    l_u[q] = u;
+                    l_ph[q] = phiu[u];
+                }
+                n += __popc(m);
+                e_next += 32;
+            }
+            if (half == 0) {
+                if (lane < 2) l_col[at + n + lane] = 0x7fffffff;  // two past the end, for the merge
+                if (lane == 0) {
+                    l_cnt[b * G + r] = n;
+                    l_more[b * G + r] = e_next < e_end;
+                }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&l_full[b]);
+            }
+        };
+        // edge u's a3 into ring place d, one copy group per edge
+        auto fetch = [&](int u, int d) {
+            const float *src = a3 + (int64_t)u * 3 * F + c0;
 #pragma unroll
-                for (int k = 0; k < KM; ++k) {
-                    if (uu[k] < 0) continue;
+            for (int p = 0; p < 3; ++p) cp_lane<8 * NP>(ring + d * T::A3 + p * FH * 4, src + p * F);
+        };
+        int g = blockIdx.x, n_stage = 0;
+        open_row(g);
+        if (g < groups) list_row(0);
+        Ch<NP> acc[9], yi[9], gi[9];
+        bool fresh = true;  // the group's first pass
+        for (int t = 0; ok && g < groups; ++t) {
+            const int b = t & 1;
+            if (!wait(&l_full[b], (t >> 1) & 1)) break;
+            const bool more = any_more(b);
+            const int i = row_of(g), n = l_cnt[b * G + r], at = (b * G + r) * CAP;
+            int k = 0, place = 0;  // edges done; ring place of the next one
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                if (d < n) fetch(l_u[at + d], d);
+                cp_commit();
+            }
+            if (fresh) {
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+#pragma unroll
+                    for (int x = 0; x < NP; ++x) acc[q].v[x] = 0;
+                    if (BWD && i >= 0) {
+                        const uint32_t o = coord_row(q, (uint32_t)i, (uint32_t)N, F) + c0;
+                        yi[q] = ldc<NP>(V2 + o);
+                        gi[q] = ldc<NP>(V + o);
+                        acc[q] = ldc<NP>(out + o);
+                    }
+                }
+            }
+            const int g_next = more ? g : g + gridDim.x;
+            for (bool first = true;; first = false) {
+                const int s = n_stage % ST;
+                if (!wait(&full[s], (n_stage / ST) & 1)) break;
+                const int meta = s_meta[s];
+                unsigned slots = __ballot_sync(0xffffffffu, lane < (meta & 255) && ((s_mask[s * NS + (lane < NS ? lane : 0)] >> r) & 1u));
+                while (slots && ok) {
+                    const int sl = __ffs(slots) - 1;
+                    slots &= slots - 1;
+                    const float *node = reinterpret_cast<const float *>(sm + (s * NS + sl) * T::SLOT) + c0;
+                    const int u = l_u[at + k], j = l_col[at + k];
+                    const float ph = l_ph[at + k];
+                    cp_wait<D - 1>();  // one group per edge: the oldest has landed
+                    const float *sa = reinterpret_cast<const float *>(ring + place * T::A3);
+                    Ch<NP> a[3], sg[3], gv[3];
+#pragma unroll
+                    for (int p = 0; p < 3; ++p) a[p] = ldc<NP>(sa + p * FH);
+                    const bool upper = BWD && j > i;  // the same in every lane
+                    Ch<NP> v[9], sp[3];
+                    const uint64_t ph2 = f2_pack(ph, ph);
 #pragma unroll
                     for (int p = 0; p < 3; ++p)
 #pragma unroll
-                        for (int r = 0; r < PER; ++r) {
-                            float4 &v = g[k][p][r];
-                            v.x = silu_f(v.x) * ph[k]; v.y = silu_f(v.y) * ph[k];
-                            v.z = silu_f(v.z) * ph[k]; v.w = silu_f(v.w) * ph[k];
+                        for (int x = 0; x < NP; ++x) {
+                            const float2 t = f2_unpack(a[p].v[x]);
+                            if constexpr (BWD) {  // the sigmoid, kept for SiLU'
+                                sg[p].v[x] = f2_pack(sigmoid_f(t.x), sigmoid_f(t.y));
+                                gv[p].v[x] = f2_mul(f2_mul(a[p].v[x], sg[p].v[x]), ph2);
+                            } else {
+                                gv[p].v[x] = f2_mul(f2_pack(silu_f(t.x), silu_f(t.y)), ph2);
+                            }
                         }
+                    // the place is read: the edge D further on takes it
+                    if (k + D < n) fetch(l_u[at + k + D], place);
+                    cp_commit();
+                    ++k;
+                    place = place + 1 == D ? 0 : place + 1;
+#pragma unroll
+                    for (int q = 0; q < 9; ++q) v[q] = ldc<NP>(node + q * F);
 #pragma unroll
                     for (int q = 0; q < 9; ++q)
 #pragma unroll
-                        for (int r = 0; r < PER; ++r) fma4v(acc[q][r], g[k][plane_of(q)][r], gm[k][q][r]);
+                        for (int x = 0; x < NP; ++x)
+                            acc[q].v[x] = f2_fma(gv[plane_of(q)].v[x], v[q].v[x], acc[q].v[x]);
+                    if constexpr (BWD) {
+                        if (!upper) continue;
+#pragma unroll
+                        for (int q = 0; q < 9; ++q)
+#pragma unroll
+                            for (int x = 0; x < NP; ++x)
+                                sp[plane_of(q)].v[x] = f2_fma(v[q].v[x], yi[q].v[x],
+                                                              (q == 0 || q == 1 || q == 4) ? 0 : sp[plane_of(q)].v[x]);
+#pragma unroll
+                        for (int q = 0; q < 9; ++q) {
+                            const Ch<NP> yj = ldc<NP>(node + (9 + q) * F);
+#pragma unroll
+                            for (int x = 0; x < NP; ++x)
+                                sp[plane_of(q)].v[x] = f2_fma(gi[q].v[x], yj.v[x], sp[plane_of(q)].v[x]);
+                        }
+                        const uint32_t ab = (uint32_t)u * 3u * F + c0;
+                        uint64_t r2 = 0;
+                        const uint64_t one = f2_pack(1.f, 1.f), neg = f2_pack(-1.f, -1.f);
+#pragma unroll
+                        for (int p = 0; p < 3; ++p) {
+                            Ch<NP> ga;
+#pragma unroll
+                            for (int x = 0; x < NP; ++x) {
+                                const uint64_t v = a[p].v[x], sv = sg[p].v[x], d = sp[p].v[x];
+                                r2 = f2_fma(d, f2_mul(v, sv), r2);
+                                // SiLU' = s (1 + x (1 - s))
+                                const uint64_t sd = f2_mul(sv, f2_fma(v, f2_fma(sv, neg, one), one));
+                                ga.v[x] = f2_mul(f2_mul(d, ph2), sd);
+                            }
+                            if (ga3) stc<NP>(ga3 + ab + p * F, ga);
+                            opcopy_store_c<NP>(ga3_cp, ab + p * F, ga);
+                        }
+                        const float2 rr = f2_unpack(r2);
+                        float rsum = rr.x + rr.y;
+                        rsum = warp_sum(rsum);
+                        if (lane == 0) gphi[u] += rsum;
+                    }
+                }
+                if (!ok) break;
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&empty[s]);
+                ++n_stage;
+                if (first && g_next < groups) {
+                    // the next pass's list, while this one's copies run: its
+                    // buffer is free once every warp is through with pass t - 1
+                    if (t >= 1 && !wait(&l_empty[b ^ 1], ((t - 1) >> 1) & 1)) break;
+                    if (!more) open_row(g_next);
+                    list_row(b ^ 1);
+                }
+                if (meta & 256) break;
+            }
+            if (!ok) break;
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&l_empty[b]);
+            fresh = !more;
+            if (!more && i >= 0) {
+#pragma unroll
+                for (int q = 0; q < 9; ++q) {
+                    const uint32_t o = coord_row(q, (uint32_t)i, (uint32_t)N, F) + c0;
+                    stc<NP>(out + o, acc[q]);
+                    if (BWD) opcopy_store_c<NP>(out_cp, o, acc[q]);
                 }
             }
-            for (int k = nl; k < n; ++k) {  // upper edges, one at a time
-                const int u = __shfl_sync(0xffffffffu, u_l, k);
-                const int j = __shfl_sync(0xffffffffu, j_l, k);
-                const float ph = __shfl_sync(0xffffffffu, ph_l, k);
-                if (u < 0) continue;
-                // two rounds of gathers (gM_j with a3, then Y_j), so that only
-                // one 9-row block is live at a time
-                const uint32_t ab = (uint32_t)u * 3u * F + 4u * lane;
-                float4 sp[3][PER], gv[3][PER];
-                float rsum = 0.f;
-                {
-                    float4 a[3][PER], gm[9][PER];
-#pragma unroll
-                    for (int p = 0; p < 3; ++p)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) {
-                            a[p][r] = ld4(a3 + ab + p * F + 128 * r);
-                            sp[p][r] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        const uint32_t bq = coord_row(q, (uint32_t)j, (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) gm[q][r] = ld4(gM + bq + 128 * r);
-                    }
-#pragma unroll
-                    for (int p = 0; p < 3; ++p)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) {
-                            const float4 v = a[p][r];
-                            gv[p][r] = make_float4(silu_f(v.x) * ph, silu_f(v.y) * ph, silu_f(v.z) * ph,
-                                                   silu_f(v.w) * ph);
-                        }
-#pragma unroll
-                    for (int q = 0; q < 9; ++q)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) {
-                            fma4v(acc[q][r], gv[plane_of(q)][r], gm[q][r]);
-                            fma4v(sp[plane_of(q)][r], gm[q][r], s_y[q][lane + 32 * r]);
-                        }
-                }
-                {
-                    float4 yj[9][PER];
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) {
-                        const uint32_t bq = coord_row(q, (uint32_t)j, (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) yj[q][r] = ld4(Y + bq + 128 * r);
-                    }
-#pragma unroll
-                    for (int q = 0; q < 9; ++q)
-#pragma unroll
-                        for (int r = 0; r < PER; ++r) fma4v(sp[plane_of(q)][r], s_gm[q][lane + 32 * r], yj[q][r]);
-                }
-#pragma unroll
-                for (int p = 0; p < 3; ++p)
-#pragma unroll
-                    for (int r = 0; r < PER; ++r) {
-                        // a3 again (just read by this warp: an L1 or L2 hit) rather
-                        // than held through both gather rounds
-                        const float4 ar = ld4(a3 + ab + p * F + 128 * r);
-                        const float av[4] = {ar.x, ar.y, ar.z, ar.w};
-                        const float sv4[4] = {sp[p][r].x, sp[p][r].y, sp[p][r].z, sp[p][r].w};
-                        float gav[4];
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            float sv, sd;
-                            silu_and_grad_f(av[c], sv, sd);
-                            rsum = fmaf(sv4[c], sv, rsum);
-                            gav[c] = sv4[c] * ph * sd;
-                        }
-                        const uint32_t o = ab + p * F + 128 * r;
-                        if (ga3) st4(ga3 + o, make_float4(gav[0], gav[1], gav[2], gav[3]));
-                        if (ga3_cp.mode) {
-                            opcopy_store(ga3_cp, o, gav[0]);
-                            opcopy_store(ga3_cp, o + 1, gav[1]);
-                            opcopy_store(ga3_cp, o + 2, gav[2]);
-                            opcopy_store(ga3_cp, o + 3, gav[3]);
-                        }
-                    }
-                rsum = warp_sum(rsum);
-                if (lane == 0) gphi[u] += rsum;
-            }
+            g = g_next;
         }
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const uint32_t b = coord_row(q, (uint32_t)i, (uint32_t)N, F) + 4u * lane;
-#pragma unroll
-            for (int r = 0; r < PER; ++r) {
-                st4(gY + b + 128 * r, acc[q][r]);
-                if (gY_cp.mode) {
-                    opcopy_store(gY_cp, b + 128 * r, acc[q][r].x);
-                    opcopy_store(gY_cp, b + 128 * r + 1, acc[q][r].y);
-                    opcopy_store(gY_cp, b + 128 * r + 2, acc[q][r].z);
-                    opcopy_store(gY_cp, b + 128 * r + 3, acc[q][r].w);
-                }
-            }
-        }
+        cp_wait<0>();
     }
 }
 
@@ -1742,16 +1861,6 @@ __global__ void k_emb_bwd_pairs(const float4 *__restrict__ geo, const int32_t *_
 // warp: 2.77 ms).  Bound by the latency of the gathers (6.1 KB a pair through
 // L2), HBM at 57%.  96,000-atom water (2.58 M pairs): 3.04 -> 2.06 ms; 3,000
 // atoms 105 -> 54 us.  Offsets are 32-bit (the host checks the sizes).
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 constexpr int kPairRun = 32;    // consecutive pairs a warp takes at a time
 constexpr int kPairBlocks = 4;  // resident blocks per SM, and the grid: one wave
 struct F4 {  // four FP32 values as two packed pairs
@@ -1869,7 +1978,7 @@ __global__ void k_pair_vec(const float *__restrict__ pos, const float *__restric
                            const int32_t *__restrict__ batch, const int2 *__restrict__ uij,
                            const int32_t *__restrict__ ue, const int32_t *__restrict__ rev,
                            const int32_t *__restrict__ nu, RadialParams rp, const float *__restrict__ ge,
-                           const float *__restrict__ gphi_mlp, const float4 *__restrict__ edge_g,
+                           const float *__restrict__ gphi_mlp, int64_t gphi_stride, const float4 *__restrict__ edge_g,
                            const float4 *__restrict__ pair_g, const float *__restrict__ dEdd,
                            float *__restrict__ Gp) {
     pdl_entry();
@@ -1913,7 +2022,7 @@ __global__ void k_pair_vec(const float *__restrict__ pos, const float *__restric
                 const float4 a = edge_g[e], b = edge_g[rev[e]];
                 g = make_float4(a.x + b.x, a.y - b.y, a.z - b.z, a.w - b.w);
             }
-            const float gphi = (gphi_mlp ? gphi_mlp[u] : 0.f) + g.x;
+            const float gphi = (gphi_mlp ? gphi_mlp[u] + gphi_mlp[u + gphi_stride] : 0.f) + g.x;
             const float gd = s + gphi * dphi + (dEdd ? dEdd[u] : 0.f);
             const float inv = 1.0f / d;
             const float ux = x * inv, uy = y * inv, uz = zz * inv;
@@ -2526,16 +2635,20 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
           *hs1 = f32(Lw.hs1), *as2 = f32(Lw.as2), *s = f32(Lw.s), *q0 = f32(Lw.q0);
     float2 *ln0 = wsp<float2>(ctx, Lw.ln0);
     const int atom_blocks = N < sms * ctx->tune[T_ROW_BLOCKS] ? N : sms * ctx->tune[T_ROW_BLOCKS];
-    // message kernels (and the pair-parallel embedding adjoint): knob 0 =
-    // one warp per row (pair) with four channels per lane (exact mode,
-    // F = 128, 32-bit offsets; the adjoint at two blocks per SM), 3 = the
-    // same with the adjoint at three blocks per SM, 1 or 4 = that many
-    // consecutive rows per block of F threads (one thread per channel)
+    // message kernels (and the pair-parallel embedding adjoint): knob 0 or 3 =
+    // the staged kernels (exact mode, F = 128, 32-bit offsets), 1 or 4 = that
+    // many consecutive rows per block of F threads (one thread per channel)
     const int rows_pb = ctx->tune[T_MSG_KERNEL] == 4 ? 4 : 1;
     const bool warp_rows = (ctx->tune[T_MSG_KERNEL] == 0 || ctx->tune[T_MSG_KERNEL] == 3) && !tab && F == 128 &&
                            9LL * N * F < (1LL << 31) && (int64_t)maxU * 3 * F < (1LL << 31);
-    const int v4_blocks = (int)((N + kV4Warps - 1) / kV4Warps < atom_blocks ? (N + kV4Warps - 1) / kV4Warps
-                                                                             : atom_blocks);
+    // rows per group of the staged message kernels: at most `most`, and as few
+    // as let every SM have the same number of groups
+    auto msg_shape = [&](int most, int &run, int &grid) {
+        const int64_t rounds = (N + (int64_t)most * sms - 1) / ((int64_t)most * sms);
+        run = (int)((N + rounds * sms - 1) / (rounds * sms));
+        const int groups = (N + run - 1) / run;
+        grid = groups < sms ? groups : sms;
+    };
 #define EMB_FWD(FF)                                                                                           \
     if (tab)                                                                                                  \
         launch(k_emb_edges<FF, true>, atom_blocks, FF, 0, st, geo, z, row_ptr, col, pair_of, N, d.max_z, fu, tf0, Ta, \
@@ -2651,8 +2764,14 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                                       N, M);                                                                 \
     else launch_message<FF, false>(rows_pb, atom_blocks, st, row_ptr, col, pair_of, a3l, phiu, tabfn(1 + l), Y, \
                                    N, M)
-        if (warp_rows) launch(k_message_v4<128>, v4_blocks, 32 * kV4Warps, 0, st, row_ptr, col, pair_of, a3l, phiu, Y,
-                              N, M);
+        if (warp_rows) {
+            using T = MsgTile<128, false>;
+            TRY(ensure_smem_attr((const void *)k_message_tile<128, false>, T::SMEM));
+            int run, grid;
+            msg_shape(T::G, run, grid);
+            launch(k_message_tile<128, false>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3l, phiu, Y,
+                   (const float *)nullptr, N, run, M, none, (float *)nullptr, none, (float *)nullptr, (int64_t)0, status);
+        }
         else {
             TNET_F_SWITCH(F, MSG_FWD);
         }
@@ -2727,7 +2846,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         TRY(wgrad_layernorm(ghn, h, lno, N, 3 * F, wpart, wcap, gw(G.out_ln_g), sms, st));
     }
     // gphiu collects dE/dphi per pair (or, in table mode, dE/dd)
-    if (NL > 0 || tab) TNET_CUDA_TRY(cudaMemsetAsync(gphiu, 0, sizeof(float) * maxU, st));
+    if (NL > 0 || tab) TNET_CUDA_TRY(cudaMemsetAsync(gphiu, 0, sizeof(float) * 2 * maxU, st));
     for (int l = NL - 1; l >= 0; --l) {
         const LayerW &Lr = W.layer[l];
         const LayerW &Gr = G.layer[l];
@@ -2762,12 +2881,12 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         if (tab) {
             TNET_F_SWITCH(F, MSG_BWD_TAB);
         } else if (warp_rows) {
-            if (ctx->tune[T_MSG_KERNEL] == 3)
-                launch(k_message_bwd_v4<128, 3>, v4_blocks, 32 * kV4Warps, 0, st, row_ptr, col, pair_of, Y, gM, a3,
-                       phiu, N, gY, nbf, ga3_out, ga3_cp, gphiu);
-            else
-                launch(k_message_bwd_v4<128, 2>, v4_blocks, 32 * kV4Warps, 0, st, row_ptr, col, pair_of, Y, gM, a3,
-                       phiu, N, gY, nbf, ga3_out, ga3_cp, gphiu);
+            using T = MsgTile<128, true>;
+            TRY(ensure_smem_attr((const void *)k_message_tile<128, true>, T::SMEM));
+            int run, grid;
+            msg_shape(T::G, run, grid);
+            launch(k_message_tile<128, true>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3, phiu, gM, Y, N,
+                   run, gY, nbf, ga3_out, ga3_cp, gphiu, (int64_t)maxU, status);
         } else {
             TNET_F_SWITCH(F, MSG_BWD);
         }
@@ -2917,7 +3036,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     if (!forces) return TNET_OK;
     pf.mark(P_FORCES);
     launch(k_pair_vec, pair_grid, 256, 0, st, pos, box, batch, uij, ue, rev, nu, rp, tab ? nullptr : ge,
-           (NL > 0 && !tab) ? gphiu : nullptr, edge_g, by_pair ? edge_g : nullptr, tab ? gphiu : nullptr, Gp);
+           (NL > 0 && !tab) ? gphiu : nullptr, (int64_t)maxU, edge_g, by_pair ? edge_g : nullptr, tab ? gphiu : nullptr, Gp);
     count_launch();
     launch(k_forces, (unsigned)(((int64_t)N * kForceLanes + 127) / 128), 128, 0, st, row_ptr, col, pair_of, Gp, N, forces);
     count_launch();
