@@ -72,7 +72,6 @@ int build_layout(const tnet_model_desc *d, int N, int S, int64_t E, Layout *L) {
     L->as2 = take(f * N * 3 * F);
     L->s = take(f * N * 3 * F);
     L->ln0 = take(8LL * N);
-    L->Xin = take(f * n9 * (NL > 0 ? NL : 1));
     L->qn = take(f * N * F * NL);
     L->Xn = take(f * n9 * NL);
     L->Y = take(f * n9 * NL);

@@ -455,7 +455,7 @@ struct Layout {
     size_t rev, pair_of, uedge, ucnt, nu, rp_safe;
     // node buffers
     size_t Ta, Tb, Xraw, Uemb, n0, as1, hs1, as2, s, ln0;
-    size_t Xin, qn, Xn, Y, M, Tn, dX;  // per layer (stride given below)
+    size_t qn, Xn, Y, M, Tn, dX;  // per layer (stride given below)
     size_t Xfin, h, hn, lno, ao, o, at, t, Ei;
     // edge MLP (undirected active edges)
     size_t eu, phiu, geo, a1, h1, a2, h2, a3;
