@@ -354,8 +354,8 @@ __device__ __forceinline__ int axis_neighbors(int c, int nc, int pbc, int out[3]
 // cell-sorted order.  Lane r first loads the bounds of range r (at most 27,
 // 9 without wrap), a warp scan lays the ranges end to end, and the warp then
 // walks the concatenated candidates 32 at a time, two chunks' loads in
-// flight: each lane finds the range of its candidate by a five-step search
-// over the scanned offsets (shuffles, the same steps in every lane).
+// flight: each lane moves on from the range of its last candidate until it
+// holds the next one (shuffles, the same steps in every lane).
 template <class Fn>
 __device__ __forceinline__ void for_candidates(int i, const float *__restrict__ pos,
                                                const int32_t *__restrict__ batch,
@@ -413,6 +413,7 @@ __device__ __forceinline__ void for_candidates(int i, const float *__restrict__ 
     }
     const int excl = incl - len;
     const int total = __shfl_sync(0xffffffffu, incl, 31);
+    int r = 0;  // the range of this lane's last candidate
     for (int c0 = 0; c0 < total; c0 += 64) {
         float4 q[2];
         bool has[2];
@@ -421,15 +422,14 @@ __device__ __forceinline__ void for_candidates(int i, const float *__restrict__ 
             const int tc = c0 + 32 * u + lane;
             has[u] = tc < total;
             if (c0 + 32 * u >= total) continue;  // the same in every lane
-            // last range whose offset is <= tc (it holds tc when tc < total)
-            int r = 0;
-            if (R > 1) {  // the same in every lane
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1) {
-                    const int cand = r + step;
-                    const int e = __shfl_sync(0xffffffffu, excl, cand & 31);
-                    if (cand < R && e <= tc) r = cand;
-                }
+            // first range that ends beyond tc (it holds tc when tc < total);
+            // candidates ascend, so the range only moves on, seldom by more
+            // than one (empty ranges apart)
+            for (;;) {
+                const int end = __shfl_sync(0xffffffffu, incl, r);
+                const bool on = end <= tc && r + 1 < R;
+                if (!__any_sync(0xffffffffu, on)) break;
+                r += on;
             }
             const int rp0 = __shfl_sync(0xffffffffu, p0, r);
             const int rex = __shfl_sync(0xffffffffu, excl, r);
@@ -470,6 +470,54 @@ __global__ void k_pair_count(const float *__restrict__ pos, const int32_t *__res
 }
 
 constexpr int kFillWarps = 4;
+
+// Ascending bitonic sort of 32 PER values, value PER * lane + r of the warp in
+// v[r]: partners nearer than PER apart are in the lane's own registers, the
+// others one exchange away, and no step touches memory (in shared memory the
+// sort of a 90-entry row cost as much as its candidate walk).
+template <int PER>
+__device__ __forceinline__ void warp_sort_regs(int32_t v[PER], int lane) {
+#pragma unroll
+    for (int k = 2; k <= 32 * PER; k <<= 1) {
+#pragma unroll
+        for (int jj = k >> 1; jj > 0; jj >>= 1) {
+            if (jj >= PER) {
+                const bool low = ((lane * PER) & jj) == 0;
+#pragma unroll
+                for (int r = 0; r < PER; ++r) {
+                    const bool up = ((lane * PER + r) & k) == 0;
+                    const int32_t o = __shfl_xor_sync(0xffffffffu, v[r], jj / PER);
+                    v[r] = low == up ? min(v[r], o) : max(v[r], o);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < PER; ++r)
+                    if ((r & jj) == 0) {
+                        const bool up = ((lane * PER + r) & k) == 0;
+                        const int32_t a = v[r], c = v[r | jj];
+                        v[r] = up ? min(a, c) : max(a, c);
+                        v[r | jj] = up ? max(a, c) : min(a, c);
+                    }
+            }
+        }
+    }
+}
+template <int PER>
+__device__ __forceinline__ void warp_sort_write(const int32_t *sb, int cnt, int lane, int32_t *__restrict__ dst) {
+    int32_t v[PER];
+#pragma unroll
+    for (int r = 0; r < PER; ++r) v[r] = PER * lane + r < cnt ? sb[PER * lane + r] : 0x7fffffff;
+    warp_sort_regs<PER>(v, lane);
+#pragma unroll
+    for (int r = 0; r < PER; ++r)
+        if (PER * lane + r < cnt) dst[PER * lane + r] = v[r];
+}
+// the first cnt <= 128 entries of a warp's buffer, ascending, to dst
+__device__ __forceinline__ void warp_sort_short(const int32_t *sb, int cnt, int lane, int32_t *__restrict__ dst) {
+    if (cnt <= 32) warp_sort_write<1>(sb, cnt, lane, dst);
+    else if (cnt <= 64) warp_sort_write<2>(sb, cnt, lane, dst);
+    else warp_sort_write<4>(sb, cnt, lane, dst);
+}
 
 // Sorts the first cnt entries of a warp's buffer ascending (room for the next
 // power of two).
@@ -538,7 +586,9 @@ k_pair_emit(const float *__restrict__ pos, const int32_t *__restrict__ batch, in
         });
         cnt = cnt < rlen ? cnt : rlen;
         __syncwarp();
-        if (in_smem) {
+        if (cnt <= 128 && in_smem) {
+            warp_sort_short(sb, cnt, lane, col + r0);
+        } else if (in_smem) {
             warp_sort(sb, cnt, lane);
             for (int k = lane; k < cnt; k += 32) col[r0 + k] = sb[k];
         } else if (lane == 0) {
@@ -586,9 +636,8 @@ k_pair_fill_slab(const float *__restrict__ pos, const int32_t *__restrict__ batc
         return;
     }
     __syncwarp();
-    warp_sort(sb, cnt, lane);
-    int32_t *dst = slab + (int64_t)i * kSlabWidth;
-    for (int k = lane; k < cnt; k += 32) dst[k] = sb[k];
+    static_assert(kSlabWidth <= 128, "sorted in registers");
+    warp_sort_short(sb, cnt, lane, slab + (int64_t)i * kSlabWidth);
 }
 
 int neighbors_impl(tnet_ctx *ctx, int N, int S, const float *pos, const int32_t *batch,
