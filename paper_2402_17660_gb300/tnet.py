@@ -200,13 +200,17 @@ class EnergyFn(torch.autograd.Function):
     """E_s(pos, weights) with gradients from libtnet's reverse pass.
 
     forward(pos, weights, model, z, nl, batch, box, n_systems) -> E [S] f64.
-    d/dpos = -forces scaled per system by the incoming gradient; d/dweights
-    comes from a second reverse pass seeded with the incoming gradient."""
+    For positions alone the forward pass also runs the reverse pass, and
+    d/dpos = -forces scaled per system by the incoming gradient.  When the
+    weights need gradients, backward runs one pass seeded with the incoming
+    gradient, which gives d/dweights and d/dpos together, and forward
+    evaluates the energies alone."""
 
     @staticmethod
     def forward(ctx, pos, weights, model: TensorNet, z, nl, batch, box, n_systems):
         model.set_weights(weights)
-        E, Fo, _ = model.energy_forces(z, pos.detach(), nl, batch, box, n_systems, forces=True)
+        want_pos, want_w = ctx.needs_input_grad[:2]
+        E, Fo, _ = model.energy_forces(z, pos.detach(), nl, batch, box, n_systems, forces=want_pos and not want_w)
         ctx.model, ctx.args = model, (z, nl, batch, box, n_systems)
         ctx.save_for_backward(pos, weights, Fo)
         return E
@@ -216,14 +220,16 @@ class EnergyFn(torch.autograd.Function):
         pos, weights, Fo = ctx.saved_tensors
         z, nl, batch, box, n_systems = ctx.args
         model = ctx.model
+        want_pos, want_w = ctx.needs_input_grad[:2]
         gpos = gw = None
-        if ctx.needs_input_grad[0]:
+        if want_w:
+            model.set_weights(weights)
+            _, Fs, gw = model.energy_forces(z, pos.detach(), nl, batch, box, n_systems, forces=want_pos,
+                                            grad_weights=True, seed=gE.to(torch.float32).contiguous())
+            gpos = -Fs if want_pos else None
+        elif want_pos:
             scale = gE.to(torch.float32)[batch.long()] if batch is not None else gE.to(torch.float32)[0]
             gpos = -Fo * (scale[:, None] if batch is not None else scale)
-        if ctx.needs_input_grad[1]:
-            model.set_weights(weights)
-            _, _, gw = model.energy_forces(z, pos.detach(), nl, batch, box, n_systems, forces=True,
-                                           grad_weights=True, seed=gE.to(torch.float32).contiguous())
         return gpos, gw, None, None, None, None, None, None
 
 
