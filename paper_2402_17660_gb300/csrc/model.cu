@@ -15,6 +15,8 @@
 //   reverse      the adjoint of every step in reverse order, ending in one
 //                3-vector dE/dr_ij per directed edge; forces are assembled
 //                per atom from its row and the reverse edges (no atomics).
+#include <type_traits>
+
 #include "gemm.cuh"
 #include "internal.cuh"
 #include "tc_gemm.cuh"
@@ -1222,9 +1224,11 @@ __device__ __forceinline__ void cp_arrive(uint64_t *bar) {
 // 6.9).  Measured at 96,000 atoms, both launches of a call: messages with 16
 // rows (twenty warps) 3.00 ms, 13 rows 3.06, 12 rows 2.91; adjoint with 7 rows
 // and one copying warp 7.50, 6 and three 6.91, 5 and two 8.27.
+template <int N>
+using Channels = std::integral_constant<int, N>;
 template <int F, bool BWD>
 struct MsgTile {
-    static constexpr int HW = BWD ? 2 : 1, G = BWD ? 6 : 12, NS = BWD ? 4 : 8, ST = BWD ? 4 : 3, D = BWD ? 4 : 3;
+    static constexpr int HW = BWD ? 2 : 1, G = 12 / HW, NS = BWD ? 4 : 8, ST = BWD ? 4 : 3, D = BWD ? 4 : 3;
     static constexpr int CAP = 100, C = G * HW, CW = 3, THREADS = 32 * (C + 1 + CW), FH = F / HW, NP = FH / 64;
     static constexpr int NODE = 9 * F * 4, SLOT = (BWD ? 2 : 1) * NODE, A3 = 3 * FH * 4;
     static constexpr int o_ring = ST * NS * SLOT, o_col = o_ring + C * D * A3, o_u = o_col + 2 * G * CAP * 4;
@@ -1880,11 +1884,16 @@ __global__ void k_emb_bwd_pairs(const float4 *__restrict__ geo, const int32_t *_
 // gX_raw and its table rows stay in registers until i changes, so a pair
 // gathers only row j.  The runs go round the warps, so the pairs in flight
 // sweep the atoms together and the gathered rows stay in L2 (one long run per
-// warp: 2.77 ms).  Bound by the latency of the gathers (6.1 KB a pair through
-// L2), HBM at 57%.  96,000-atom water (2.58 M pairs): 3.04 -> 2.06 ms; 3,000
-// atoms 105 -> 54 us.  Offsets are 32-bit (the host checks the sizes).
-constexpr int kPairRun = 32;    // consecutive pairs a warp takes at a time
-constexpr int kPairBlocks = 4;  // resident blocks per SM, and the grid: one wave
+// warp: 2.77 ms against 2.06).  Row j and f come through a ring in shared
+// memory, two pairs ahead (in registers, without the ring: 2.06 against 1.52;
+// three pairs ahead at three blocks: 1.66): what bounds it is the latency of
+// the gathers against the bytes under way (6.1 KB a pair through L2), then f
+// and dE/df in HBM.  96,000-atom water (2.58 M pairs): 3.04 -> 1.52 ms; 3,000
+// atoms 105 -> 50 us.  Offsets are 32-bit (the host checks the sizes).
+constexpr int kPairRun = 32;       // consecutive pairs a warp takes at a time
+constexpr int kPairBlocks = 4;     // resident blocks per SM, and the grid: one wave
+constexpr int kPairDepth = 2;      // pairs under way per warp
+constexpr int kPairBytes = 12 * 128 * 4;
 struct F4 {  // four FP32 values as two packed pairs
     uint64_t v[2];
 };
@@ -1903,40 +1912,55 @@ __global__ void __launch_bounds__(128, kPairBlocks) k_emb_bwd_pairs_v4(const flo
                                                           float4 *__restrict__ pair_g) {
     pdl_entry();
     static_assert(F == 128, "one float4 per lane and row");
+    extern __shared__ __align__(128) uint8_t pair_ring[];
     const int lane = threadIdx.x & 31;
     const int U = *nu;
     const uint32_t c4 = 4u * lane;
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t share = (U + warps - 1) / warps;
-    const int per = (int)(share < kPairRun ? share : kPairRun);
+    // equal runs of at most kPairRun pairs
+    const int64_t rounds = (share + kPairRun - 1) / kPairRun;
+    const int per = (int)(rounds > 0 ? (share + rounds - 1) / rounds : 1);
     int cur = -1;
     F4 gi[9], tai, tbi;
     auto elem = [&](int a) {
         const int q = z[a];
         return (q < 0 || q >= max_z) ? 0 : q;
     };
-    for (int64_t u0 = wid * per; u0 < U; u0 += warps * per) {
-        const int u_end = (int)(u0 + per < U ? u0 + per : U);
-        for (int u = (int)u0; u < u_end; ++u) {
-            const int2 p = uij[u];
-            const float4 gu = geo[u];
-            if (p.x != cur) {  // the same in every lane
-                cur = p.x;
-                const uint32_t zi = (uint32_t)elem(cur) * F + c4;
-                tai = ld4p(Ta + zi);
-                tbi = ld4p(Tb + zi);
+    // gX_raw_j and f of a pair through the lane's own places of a ring, kPairDepth
+    // pairs ahead (each lane copies what it will read: no barrier)
+    uint8_t *ring = pair_ring + (threadIdx.x >> 5) * kPairDepth * kPairBytes + 16 * lane;
+    auto fetch = [&](int64_t u, int j, int place) {
+        uint8_t *d = ring + place * kPairBytes;
+        const float *f = fu + u * 3 * F + c4, *h = gXraw + (int64_t)j * F + c4;
+        const float *hA = gXraw + ((int64_t)N + 3LL * j) * F + c4, *hS = gXraw + (4LL * N + 5LL * j) * F + c4;
+        cp_lane<16>(d, h);
 #pragma unroll
-                for (int q = 0; q < 9; ++q) gi[q] = ld4p(gXraw + coord_row(q, (uint32_t)cur, (uint32_t)N, F) + c4);
-            }
-            const uint32_t zj = (uint32_t)elem(p.y) * F + c4;
-            const uint32_t fb = (uint32_t)u * 3u * F + c4;
-            F4 h[9];
+        for (int q = 0; q < 3; ++q) cp_lane<16>(d + (1 + q) * F * 4, hA + q * F);
 #pragma unroll
-            for (int q = 0; q < 9; ++q) h[q] = ld4p(gXraw + coord_row(q, (uint32_t)p.y, (uint32_t)N, F) + c4);
-            const F4 f0 = ld4p(fu + fb), f1 = ld4p(fu + fb + F), f2 = ld4p(fu + fb + 2 * F);
-            const F4 taj = ld4p(Ta + zj), tbj = ld4p(Tb + zj);
-            const float ux = gu.x, uy = gu.y, uz = gu.z;
+        for (int q = 0; q < 5; ++q) cp_lane<16>(d + (4 + q) * F * 4, hS + q * F);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) cp_lane<16>(d + (9 + q) * F * 4, f + q * F);
+    };
+    auto use = [&](int u, int i, int zj_, const float4 gu, int place) {
+        F4 h[9], f[3];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) h[q] = ld4p(reinterpret_cast<const float *>(ring + place * kPairBytes + q * F * 4));
+#pragma unroll
+        for (int q = 0; q < 3; ++q) f[q] = ld4p(reinterpret_cast<const float *>(ring + place * kPairBytes + (9 + q) * F * 4));
+        if (i != cur) {  // the same in every lane
+            cur = i;
+            const uint32_t zi = (uint32_t)elem(cur) * F + c4;
+            tai = ld4p(Ta + zi);
+            tbi = ld4p(Tb + zi);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) gi[q] = ld4p(gXraw + coord_row(q, (uint32_t)cur, (uint32_t)N, F) + c4);
+        }
+        const uint32_t zj = (uint32_t)zj_ * F + c4;
+        const uint32_t fb = (uint32_t)u * 3u * F + c4;
+        const F4 taj = ld4p(Ta + zj), tbj = ld4p(Tb + zj);
+        const float ux = gu.x, uy = gu.y, uz = gu.z;
             auto dup = [](float x) { return f2_pack(x, x); };
             const uint64_t x2 = dup(ux), y2 = dup(uy), z2 = dup(uz), xx2 = dup(2.f * ux), yy2 = dup(2.f * uy);
             const uint64_t bxx = dup(ux * ux - (1.0f / 3.0f)), byy = dup(uy * uy - (1.0f / 3.0f));
@@ -1954,13 +1978,13 @@ __global__ void __launch_bounds__(128, kPairBlocks) k_emb_bwd_pairs_v4(const flo
                     q[c] = f2_fma((c >= 1 && c < 4) ? nji : zji, h[c].v[k], f2_mul(zij, gi[c].v[k]));
                 const uint64_t q1 = f2_fma(z2, q[3], f2_fma(y2, q[2], f2_mul(x2, q[1])));
                 const uint64_t q2 = f2_fma(byz, q[8], f2_fma(bxz, q[7], f2_fma(bxy, q[6], f2_fma(byy, q[5], f2_mul(bxx, q[4])))));
-                sp = f2_fma(f2.v[k], q2, f2_fma(f1.v[k], q1, f2_fma(f0.v[k], q[0], sp)));
+                sp = f2_fma(f[2].v[k], q2, f2_fma(f[1].v[k], q1, f2_fma(f[0].v[k], q[0], sp)));
                 const uint64_t dx = f2_fma(z2, q[7], f2_fma(y2, q[6], f2_mul(xx2, q[4])));
                 const uint64_t dy = f2_fma(z2, q[8], f2_fma(x2, q[6], f2_mul(yy2, q[5])));
                 const uint64_t dz = f2_fma(y2, q[8], f2_mul(x2, q[7]));
-                sx = f2_fma(f2.v[k], dx, f2_fma(f1.v[k], q[1], sx));
-                sy = f2_fma(f2.v[k], dy, f2_fma(f1.v[k], q[2], sy));
-                sz = f2_fma(f2.v[k], dz, f2_fma(f1.v[k], q[3], sz));
+                sx = f2_fma(f[2].v[k], dx, f2_fma(f[1].v[k], q[1], sx));
+                sy = f2_fma(f[2].v[k], dy, f2_fma(f[1].v[k], q[2], sy));
+                sz = f2_fma(f[2].v[k], dz, f2_fma(f[1].v[k], q[3], sz));
                 o[0].v[k] = f2_mul(ph2, q[0]);
                 o[1].v[k] = f2_mul(ph2, q1);
                 o[2].v[k] = f2_mul(ph2, q2);
@@ -1986,7 +2010,37 @@ __global__ void __launch_bounds__(128, kPairBlocks) k_emb_bwd_pairs_v4(const flo
             a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
             if ((lane & 7) == 0)
                 reinterpret_cast<float *>(pair_g)[4LL * u + (lane >> 3)] = lane == 0 ? a0 : gu.w * a0;
+    };
+    for (int64_t u0 = wid * per; u0 < U; u0 += warps * per) {
+        const int u_end = (int)(u0 + per < U ? u0 + per : U);
+        // the run's pairs, one per lane
+        const int n = u_end - (int)u0;
+        int2 p = make_int2(0, 0);
+        float4 gl = make_float4(0.f, 0.f, 0.f, 0.f);
+        int zl = 0;
+        if (lane < n) {
+            p = uij[u0 + lane];
+            gl = geo[u0 + lane];
+            zl = elem(p.y);
         }
+#pragma unroll
+        for (int d = 0; d < kPairDepth; ++d) {
+            if (d < n) fetch(u0 + d, __shfl_sync(0xffffffffu, p.y, d), d);
+            cp_commit();
+        }
+        int place = 0;
+        for (int k = 0; k < n; ++k) {
+            const float4 gu = make_float4(__shfl_sync(0xffffffffu, gl.x, k), __shfl_sync(0xffffffffu, gl.y, k),
+                                          __shfl_sync(0xffffffffu, gl.z, k), __shfl_sync(0xffffffffu, gl.w, k));
+            const int i = __shfl_sync(0xffffffffu, p.x, k), zj = __shfl_sync(0xffffffffu, zl, k);
+            const int jn = __shfl_sync(0xffffffffu, p.y, k + kPairDepth < n ? k + kPairDepth : 0);
+            cp_wait<kPairDepth - 1>();  // one copy group per pair: the oldest has landed
+            use((int)u0 + k, i, zj, gu, place);
+            if (k + kPairDepth < n) fetch(u0 + k + kPairDepth, jn, place);
+            cp_commit();
+            place = place + 1 == kPairDepth ? 0 : place + 1;
+        }
+        cp_wait<0>();
     }
 }
 
@@ -2661,7 +2715,8 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     // the staged kernels (exact mode, F = 128, 32-bit offsets), 1 or 4 = that
     // many consecutive rows per block of F threads (one thread per channel)
     const int rows_pb = ctx->tune[T_MSG_KERNEL] == 4 ? 4 : 1;
-    const bool warp_rows = (ctx->tune[T_MSG_KERNEL] == 0 || ctx->tune[T_MSG_KERNEL] == 3) && !tab && F == 128 &&
+    const bool warp_rows = (ctx->tune[T_MSG_KERNEL] == 0 || ctx->tune[T_MSG_KERNEL] == 3) && !tab &&
+                           F == 128 &&
                            9LL * N * F < (1LL << 31) && (int64_t)maxU * 3 * F < (1LL << 31);
     // rows per group of the staged message kernels: at most `most`, and as few
     // as let every SM have the same number of groups
@@ -2779,14 +2834,17 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                                       N, M);                                                                 \
     else launch_message<FF, false>(rows_pb, atom_blocks, st, row_ptr, col, pair_of, a3l, phiu, tabfn(1 + l), Y, \
                                    N, M)
-        if (warp_rows) {
-            using T = MsgTile<128, false>;
-            TRY(ensure_smem_attr((const void *)k_message_tile<128, false>, T::SMEM));
+        auto staged = [&](auto channels) -> int {
+            constexpr int FF = decltype(channels)::value;
+            using T = MsgTile<FF, false>;
+            TRY(ensure_smem_attr((const void *)k_message_tile<FF, false>, T::SMEM));
             int run, grid;
             msg_shape(T::G, run, grid);
-            launch(k_message_tile<128, false>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3l, phiu, Y,
+            launch(k_message_tile<FF, false>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3l, phiu, Y,
                    (const float *)nullptr, N, run, M, none, (float *)nullptr, none, (float *)nullptr, (int64_t)0, status);
-        }
+            return TNET_OK;
+        };
+        if (warp_rows) TRY(staged(Channels<128>{}));
         else {
             TNET_F_SWITCH(F, MSG_FWD);
         }
@@ -2904,12 +2962,17 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         if (tab) {
             TNET_F_SWITCH(F, MSG_BWD_TAB);
         } else if (warp_rows) {
-            using T = MsgTile<128, true>;
-            TRY(ensure_smem_attr((const void *)k_message_tile<128, true>, T::SMEM));
-            int run, grid;
-            msg_shape(T::G, run, grid);
-            launch(k_message_tile<128, true>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3, phiu, gM, Y, N,
-                   run, gY, nbf, ga3_out, ga3_cp, gphiu, (int64_t)maxU, status);
+            auto staged = [&](auto channels) -> int {
+                constexpr int FF = decltype(channels)::value;
+                using T = MsgTile<FF, true>;
+                TRY(ensure_smem_attr((const void *)k_message_tile<FF, true>, T::SMEM));
+                int run, grid;
+                msg_shape(T::G, run, grid);
+                launch(k_message_tile<FF, true>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3, phiu, gM, Y,
+                       N, run, gY, nbf, ga3_out, ga3_cp, gphiu, (int64_t)maxU, status);
+                return TNET_OK;
+            };
+            TRY(staged(Channels<128>{}));
         } else {
             TNET_F_SWITCH(F, MSG_BWD);
         }
@@ -3012,8 +3075,10 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         launch(k_emb_bwd_pairs<CPL, false>, pair_grid, 256, 0, st, geo, z, uij, ue, rev, nu, N, d.max_z, fu, tf0, Ta, \
                                                              Tb, gXraw, gfu, edge_g, gfu_cp, nullptr)
     const bool by_pair = !wg && !tab && warp_rows;
+    constexpr int pair_smem = 4 * kPairDepth * kPairBytes;
+    if (by_pair) TRY(ensure_smem_attr((const void *)k_emb_bwd_pairs_v4<128>, pair_smem));
     if (by_pair)
-        launch(k_emb_bwd_pairs_v4<128>, kPairBlocks * sms, 128, 0, st, geo, z, uij, nu, N, d.max_z, fu, Ta, Tb, gXraw, gfu,
+        launch(k_emb_bwd_pairs_v4<128>, kPairBlocks * sms, 128, pair_smem, st, geo, z, uij, nu, N, d.max_z, fu, Ta, Tb, gXraw, gfu,
                edge_g);
     else
     switch (F / 32) {
