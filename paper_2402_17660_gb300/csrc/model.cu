@@ -1130,7 +1130,7 @@ __global__ void __launch_bounds__(F * RB, (512 / (F * RB)) > 0 ? 512 / (F * RB) 
 }
 
 // ------------------------------------------------ staged message kernels ---
-// The same sums as k_message and k_message_bwd (exact mode, F = 128), with the
+// The same sums as k_message and k_message_bwd (exact mode, F = 64 or 128), with the
 // gathered node rows shared by a group of rows.  A block takes up to G
 // consecutive rows at a time.  One warp merges the rows' column lists (they
 // ascend), three copy each distinct column's node rows into a ring of
@@ -1228,7 +1228,7 @@ template <int N>
 using Channels = std::integral_constant<int, N>;
 template <int F, bool BWD>
 struct MsgTile {
-    static constexpr int HW = BWD ? 2 : 1, G = 12 / HW, NS = BWD ? 4 : 8, ST = BWD ? 4 : 3, D = BWD ? 4 : 3;
+    static constexpr int HW = BWD && F > 64 ? 2 : 1, G = 12 / HW, NS = BWD ? 4 : 8, ST = BWD ? 4 : 3, D = BWD ? 4 : 3;
     static constexpr int CAP = 100, C = G * HW, CW = 3, THREADS = 32 * (C + 1 + CW), FH = F / HW, NP = FH / 64;
     static constexpr int NODE = 9 * F * 4, SLOT = (BWD ? 2 : 1) * NODE, A3 = 3 * FH * 4;
     static constexpr int o_ring = ST * NS * SLOT, o_col = o_ring + C * D * A3, o_u = o_col + 2 * G * CAP * 4;
@@ -1238,6 +1238,9 @@ struct MsgTile {
     static_assert(NP >= 1 && FH == 64 * NP && SMEM <= 232448 - 256, "shared memory above 227 KB");
 };
 
+// F = 64 runs both at one warp per row, two channels a lane (12,003 atoms, 612,000
+// edges, per launch against a thread per channel: messages 205 -> 147 us, adjoint
+// 377 -> 264 us).
 // BWD false: V = Y, out = M, M_i = sum_j g_ij Y_j.
 // BWD true: V = gM, V2 = Y, out = gY (added to), and per upper edge (j > i)
 // dE/dg = <gM_i, Y_j> + <gM_j, Y_i>, ga3 = dE/dg phi SiLU'(a3) and gphi[half][u]
@@ -2712,11 +2715,11 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     float2 *ln0 = wsp<float2>(ctx, Lw.ln0);
     const int atom_blocks = N < sms * ctx->tune[T_ROW_BLOCKS] ? N : sms * ctx->tune[T_ROW_BLOCKS];
     // message kernels (and the pair-parallel embedding adjoint): knob 0 or 3 =
-    // the staged kernels (exact mode, F = 128, 32-bit offsets), 1 or 4 = that
+    // the staged kernels (exact mode, F = 64 or 128, 32-bit offsets), 1 or 4 = that
     // many consecutive rows per block of F threads (one thread per channel)
     const int rows_pb = ctx->tune[T_MSG_KERNEL] == 4 ? 4 : 1;
     const bool warp_rows = (ctx->tune[T_MSG_KERNEL] == 0 || ctx->tune[T_MSG_KERNEL] == 3) && !tab &&
-                           F == 128 &&
+                           (F == 64 || F == 128) &&
                            9LL * N * F < (1LL << 31) && (int64_t)maxU * 3 * F < (1LL << 31);
     // rows per group of the staged message kernels: at most `most`, and as few
     // as let every SM have the same number of groups
@@ -2844,7 +2847,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                    (const float *)nullptr, N, run, M, none, (float *)nullptr, none, (float *)nullptr, (int64_t)0, status);
             return TNET_OK;
         };
-        if (warp_rows) TRY(staged(Channels<128>{}));
+        if (warp_rows) TRY(F == 64 ? staged(Channels<64>{}) : staged(Channels<128>{}));
         else {
             TNET_F_SWITCH(F, MSG_FWD);
         }
@@ -2972,7 +2975,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                        N, run, gY, nbf, ga3_out, ga3_cp, gphiu, (int64_t)maxU, status);
                 return TNET_OK;
             };
-            TRY(staged(Channels<128>{}));
+            TRY(F == 64 ? staged(Channels<64>{}) : staged(Channels<128>{}));
         } else {
             TNET_F_SWITCH(F, MSG_BWD);
         }
@@ -3074,7 +3077,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     else                                                                                                     \
         launch(k_emb_bwd_pairs<CPL, false>, pair_grid, 256, 0, st, geo, z, uij, ue, rev, nu, N, d.max_z, fu, tf0, Ta, \
                                                              Tb, gXraw, gfu, edge_g, gfu_cp, nullptr)
-    const bool by_pair = !wg && !tab && warp_rows;
+    const bool by_pair = !wg && !tab && warp_rows && F == 128;
     constexpr int pair_smem = 4 * kPairDepth * kPairBytes;
     if (by_pair) TRY(ensure_smem_attr((const void *)k_emb_bwd_pairs_v4<128>, pair_smem));
     if (by_pair)
