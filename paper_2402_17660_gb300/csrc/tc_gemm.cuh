@@ -76,10 +76,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -102,22 +98,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     }
     return false;
 }
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            smem_u32(dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-// the same into every CTA of the cluster in `mask` (same shared-memory offset;
-// each destination's barrier at the offset of `bar` receives the bytes)
-__device__ __forceinline__ void tma_load_2d_mc(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
-                                               uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
-        "{%2, %3}], [%4], %5;" ::"r"(smem_u32(dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask)
-        : "memory");
+// the same for a converged warp: the verdict is the warp's, in a uniform register
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+                                               uint32_t limit) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));
 }
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -139,26 +123,68 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D (TMEM) (+)= A (smem desc) * B (smem desc)^T, kind::f16 with bf16 inputs
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accum) {
+// The producer's and the MMA issuer's instructions take the elected lane as a
+// predicate instead of standing in an `if (lane == 0)`: the warp stays
+// converged, so descriptors, coordinates and addresses are computed and held in
+// uniform registers, which these instructions read.  In a divergent branch every
+// operand went through a vector register first: 85-105 cycles an MMA, whatever
+// its width, where one of 32 columns takes 16 and one of 192 takes 96.
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p;
+}
+__device__ __forceinline__ void expect_tx_if(uint32_t lead, uint64_t *bar, uint32_t bytes) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accum)
+        "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(
+            smem_u32(bar)),
+        "r"(bytes), "r"(lead)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_2d_if(uint32_t lead, void *dst, const CUtensorMap *map, int x, int y,
+                                               uint64_t *bar) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %5, 0;\n @q "
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n}\n" ::"r"(
+            smem_u32(dst)),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "r"(lead)
+        : "memory");
+}
+// the same into every CTA of the cluster in `mask` (same shared-memory offset;
+// each destination's barrier at the offset of `bar` receives the bytes)
+__device__ __forceinline__ void tma_load_2d_mc_if(uint32_t lead, void *dst, const CUtensorMap *map, int x, int y,
+                                                  uint64_t *bar, uint16_t mask) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %6, 0;\n @q "
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
+        "{%2, %3}], [%4], %5;\n}\n" ::"r"(smem_u32(dst)),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask), "r"(lead)
+        : "memory");
+}
+// D (TMEM) (+)= A (smem desc) * B (smem desc)^T, kind::f16 with bf16 inputs
+__device__ __forceinline__ void umma_bf16(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                          uint32_t idesc, uint32_t accum) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q "
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accum), "r"(lead)
         : "memory");
 }
 // the mbarrier arrives once all previously issued MMAs of this thread complete
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
+__device__ __forceinline__ void umma_commit(uint32_t lead, uint64_t *bar) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n @q "
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
+        "r"(lead)
+        : "memory");
 }
 // the same arrival on the barrier at this offset in every CTA of `mask`
-__device__ __forceinline__ void umma_commit_mc(uint64_t *bar, uint16_t mask) {
+__device__ __forceinline__ void umma_commit_mc(uint32_t lead, uint64_t *bar, uint16_t mask) {
     asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q "
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n" ::"r"(
             smem_u32(bar)),
-        "h"(mask)
+        "h"(mask), "r"(lead)
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
@@ -198,22 +224,22 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 // D (TMEM) (+)= A * B^T, kind::tf32 (fp32 containers read as TF32)
-__device__ __forceinline__ void umma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accum) {
+__device__ __forceinline__ void umma_tf32(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                          uint32_t idesc, uint32_t accum) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accum)
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q "
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accum), "r"(lead)
         : "memory");
 }
 // The same with A in TMEM: row m of A in lane m, one TF32 element of K per
 // 32-bit column (8 columns per k-step)
-__device__ __forceinline__ void umma_tf32_at(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                             uint32_t accum) {
+__device__ __forceinline__ void umma_tf32_at(uint32_t lead, uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc,
+                                             uint32_t idesc, uint32_t accum) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(
-            d_tmem),
-        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accum)
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n @q "
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accum), "r"(lead)
         : "memory");
 }
 // this thread's 16 consecutive 32-bit columns of its TMEM lane
@@ -350,6 +376,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
         const int md = *P.rows_dev * P.rows_mul;
         M0 = md < M0 ? md : M0;
     }
+    M0 = __shfl_sync(0xffffffffu, M0, 0);  // (uniform registers: see elect_lane)
     TileIter it;
     it.tilesN = (P.N + BN - 1) / BN;
     it.nclass = P.nclass;
@@ -357,7 +384,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
     it.mt1 = (M1 + BM - 1) / BM;
     it.mt2 = (M2 + BM - 1) / BM;
     const int nk = (P.K + BK - 1) / BK;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t lim = P.spin_limit;
     // tile walk: over this CTA's tiles, or over its cluster's tiles
     const int cl = P.cl > 1 ? P.cl : 1;
@@ -392,113 +419,111 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
     if (cl > 1) cluster_sync();  // every CTA's barriers exist before any multicast reaches them
     else __syncthreads();
     fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-    if (warp == 0) {
-        if (lane == 0) {  // TMA producer
-            int kg = 0;
-            int z, m0, n0;
-            for (int t = t_first; next_tile(t, z, m0, n0) && !*abort_flag; t += t_step) {
-                for (int kb = 0; kb < nk; ++kb, ++kg) {
-                    const int s = kg % STAGES;
-                    if (kg >= STAGES && !mbar_wait(&empty[s], ((kg / STAGES) - 1) & 1, abort_flag, lim)) {
-                        set_status(status, TNET_ERR_TIMEOUT);
-                        *abort_flag = 1;
-                        break;
-                    }
-                    mbar_expect_tx(&full[s], C::STAGE_TX);
-                    const int ya = (int)(sel3(z, P.row0[0], P.row0[1], P.row0[2]) + m0);
-                    const int yb = (int)(sel3(z, P.brow0[0], P.brow0[1], P.brow0[2]) + n0);
-                    tma_load_2d(sA + s * C::A_BYTES, &tmA, kb * BK, ya, &full[s]);
-                    if (cl > 1) {  // this CTA's 1/cl of the B rows, into every CTA
-                        const int hb = BN / cl;
-                        const uint32_t off = (uint32_t)(crank * hb * C::ROW);
-                        tma_load_2d_mc(sB + s * C::B_BYTES + off, &tmB, kb * BK, yb + crank * hb, &full[s], cmask);
-                        if (X3)
-                            tma_load_2d_mc(sBlo + s * C::B_BYTES + off, &tmBlo, kb * BK, yb + crank * hb, &full[s],
-                                           cmask);
-                    } else {
-                        tma_load_2d(sB + s * C::B_BYTES, &tmB, kb * BK, yb, &full[s]);
-                        if (X3) tma_load_2d(sBlo + s * C::B_BYTES, &tmBlo, kb * BK, yb, &full[s]);
-                    }
+    if (warp == 0) {  // TMA producer
+        const uint32_t lead = elect_lane();
+        int kg = 0;
+        int z, m0, n0;
+        bool ok = true;
+        for (int t = t_first; ok && next_tile(t, z, m0, n0); t += t_step) {
+            const int ya = (int)(sel3(z, P.row0[0], P.row0[1], P.row0[2]) + m0);
+            const int yb = (int)(sel3(z, P.brow0[0], P.brow0[1], P.brow0[2]) + n0);
+            for (int kb = 0; kb < nk; ++kb, ++kg) {
+                const int s = kg % STAGES;
+                if (kg >= STAGES && !mbar_wait_warp(&empty[s], ((kg / STAGES) - 1) & 1, abort_flag, lim)) {
+                    set_status(status, TNET_ERR_TIMEOUT);
+                    *abort_flag = 1;
+                    ok = false;
+                    break;
                 }
-            }
-            // own copies must land before the CTA exits: a wait that runs out is
-            // recorded and taken up again (bounded) on the same barrier
-            for (int k = kg > STAGES ? kg - STAGES : 0; k < kg; ++k) {
-                bool landed = false;
-                for (int r = 0; r < 64 && !landed; ++r) {
-                    landed = mbar_wait(&full[k % STAGES], (k / STAGES) & 1, nullptr, lim);
-                    if (!landed) set_status(status, TNET_ERR_TIMEOUT);
+                expect_tx_if(lead, &full[s], C::STAGE_TX);
+                tma_load_2d_if(lead, sA + s * C::A_BYTES, &tmA, kb * BK, ya, &full[s]);
+                if (cl > 1) {  // this CTA's 1/cl of the B rows, into every CTA
+                    const int hb = BN / cl;
+                    const uint32_t off = (uint32_t)(crank * hb * C::ROW);
+                    tma_load_2d_mc_if(lead, sB + s * C::B_BYTES + off, &tmB, kb * BK, yb + crank * hb, &full[s], cmask);
+                    if (X3)
+                        tma_load_2d_mc_if(lead, sBlo + s * C::B_BYTES + off, &tmBlo, kb * BK, yb + crank * hb, &full[s],
+                                          cmask);
+                } else {
+                    tma_load_2d_if(lead, sB + s * C::B_BYTES, &tmB, kb * BK, yb, &full[s]);
+                    if (X3) tma_load_2d_if(lead, sBlo + s * C::B_BYTES, &tmBlo, kb * BK, yb, &full[s]);
                 }
             }
         }
-    } else if (warp == 1) {
-        if (lane == 0) {  // MMA issuer
-            const uint32_t idesc = X3 ? idesc_tf32(BM, BN) : idesc_bf16(BM, BN);
-            int kg = 0, lt = 0;
-            int z, m0, n0;
-            for (int t = t_first; !P.skip_mma && next_tile(t, z, m0, n0) && !*abort_flag; t += t_step, ++lt) {
-                const int buf = lt & 1;
-                if (lt >= 2 && !mbar_wait(&acc_empty[buf], ((lt >> 1) - 1) & 1, abort_flag, lim)) {
-                    set_status(status, TNET_ERR_TIMEOUT);
-                    *abort_flag = 1;
+        // own copies must land before the CTA exits: a wait that runs out is
+        // recorded and taken up again (bounded) on the same barrier
+        for (int k = kg > STAGES ? kg - STAGES : 0; k < kg; ++k) {
+            bool landed = false;
+            for (int r = 0; r < 64 && !landed; ++r) {
+                landed = mbar_wait_warp(&full[k % STAGES], (k / STAGES) & 1, nullptr, lim);
+                if (!landed) set_status(status, TNET_ERR_TIMEOUT);
+            }
+        }
+    } else if (warp == 1) {  // MMA issuer (one lane issues, the same throughout)
+        const uint32_t lead = elect_lane();
+        const uint32_t idesc = X3 ? idesc_tf32(BM, BN) : idesc_bf16(BM, BN);
+        const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB), sAlo0 = smem_u32(sAlo), sBlo0 = smem_u32(sBlo);
+        int kg = 0, lt = 0;
+        int z, m0, n0;
+        bool ok = true;
+        for (int t = t_first; ok && !P.skip_mma && next_tile(t, z, m0, n0); t += t_step, ++lt) {
+            const int buf = lt & 1;
+            if (lt >= 2 && !mbar_wait_warp(&acc_empty[buf], ((lt >> 1) - 1) & 1, abort_flag, lim)) {
+                ok = false;
+                break;
+            }
+            fence_after();
+            const uint32_t d = tmem + (uint32_t)(buf * BN);
+            for (int kb = 0; kb < nk; ++kb, ++kg) {
+                const int s = kg % STAGES;
+                if (!mbar_wait_warp(&full[s], (kg / STAGES) & 1, abort_flag, lim) ||
+                    (X3 && !mbar_wait_warp(&conv[s], (kg / STAGES) & 1, abort_flag, lim))) {
+                    ok = false;
                     break;
                 }
                 fence_after();
-                const uint32_t d = tmem + (uint32_t)(buf * BN);
-                bool ok = true;
-                for (int kb = 0; kb < nk; ++kb, ++kg) {
-                    const int s = kg % STAGES;
-                    if (!mbar_wait(&full[s], (kg / STAGES) & 1, abort_flag, lim) ||
-                        (X3 && !mbar_wait(&conv[s], (kg / STAGES) & 1, abort_flag, lim))) {
-                        ok = false;
-                        break;
-                    }
-                    fence_after();
-                    const uint32_t a0 = smem_u32(sA + s * C::A_BYTES), b0 = smem_u32(sB + s * C::B_BYTES);
-                    // 32-byte k-steps: four per 128-byte k-block (bf16), two per
-                    // 64-byte k-block (3xTF32)
+                const uint64_t da = sdesc_sw<C::ROW>(sA0 + s * C::A_BYTES), db = sdesc_sw<C::ROW>(sB0 + s * C::B_BYTES);
+                const uint64_t dal = sdesc_sw<C::ROW>(sAlo0 + s * C::A_BYTES);
+                const uint64_t dbl = sdesc_sw<C::ROW>(sBlo0 + s * C::B_BYTES);
+                // slot kg mod A_SLOTS: A_hi, then A_lo ROW / 4 columns further
+                const uint32_t ah = tmem + C::A_COL + (uint32_t)(C::A_SLOT_COLS * (kg % C::A_SLOTS));
+                // 32-byte k-steps: four per 128-byte k-block, two per 64-byte one
+                // (2 in the descriptors' 16-byte units)
 #pragma unroll
-                    for (int k = 0; k < C::KSTEPS; ++k) {
-                        const uint64_t da = sdesc_sw<C::ROW>(a0 + k * 32), db = sdesc_sw<C::ROW>(b0 + k * 32);
-                        const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
-                        if constexpr (C::A_TMEM) {
-                            // slot kg mod A_SLOTS: A_hi, then A_lo ROW / 4 columns further
-                            const uint32_t ah =
-                                tmem + C::A_COL + (uint32_t)(C::A_SLOT_COLS * (kg % C::A_SLOTS) + 8 * k);
-                            const uint32_t bl = smem_u32(sBlo + s * C::B_BYTES);
-                            umma_tf32_at(d, ah, db, idesc, acc);
-                            umma_tf32_at(d, ah + C::ROW / 4, db, idesc, 1u);
-                            umma_tf32_at(d, ah, sdesc_sw<C::ROW>(bl + k * 32), idesc, 1u);
-                        } else if (X3) {
-                            const uint32_t al = smem_u32(sAlo + s * C::A_BYTES), bl = smem_u32(sBlo + s * C::B_BYTES);
-                            umma_tf32(d, da, db, idesc, acc);
-                            umma_tf32(d, sdesc_sw<C::ROW>(al + k * 32), db, idesc, 1u);
-                            umma_tf32(d, da, sdesc_sw<C::ROW>(bl + k * 32), idesc, 1u);
-                        } else {
-                            umma_bf16(d, da, db, idesc, acc);
-                        }
+                for (int k = 0; k < C::KSTEPS; ++k) {
+                    const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
+                    if constexpr (C::A_TMEM) {
+                        umma_tf32_at(lead, d, ah + 8 * k, db + 2 * k, idesc, acc);
+                        umma_tf32_at(lead, d, ah + 8 * k + C::ROW / 4, db + 2 * k, idesc, 1u);
+                        umma_tf32_at(lead, d, ah + 8 * k, dbl + 2 * k, idesc, 1u);
+                    } else if (X3) {
+                        umma_tf32(lead, d, da + 2 * k, db + 2 * k, idesc, acc);
+                        umma_tf32(lead, d, dal + 2 * k, db + 2 * k, idesc, 1u);
+                        umma_tf32(lead, d, da + 2 * k, dbl + 2 * k, idesc, 1u);
+                    } else {
+                        umma_bf16(lead, d, da + 2 * k, db + 2 * k, idesc, acc);
                     }
-                    if (cl > 1) umma_commit_mc(&empty[s], cmask);  // the stage is free in every CTA's view
-                    else umma_commit(&empty[s]);
-                    if constexpr (C::A_TMEM) umma_commit(&aempty[kg % C::A_SLOTS]);
                 }
-                if (!ok) {
-                    set_status(status, TNET_ERR_TIMEOUT);
-                    *abort_flag = 1;
-                    break;
-                }
-                umma_commit(&acc_full[buf]);
+                if (cl > 1) umma_commit_mc(lead, &empty[s], cmask);  // the stage is free in every CTA's view
+                else umma_commit(lead, &empty[s]);
+                if constexpr (C::A_TMEM) umma_commit(lead, &aempty[kg % C::A_SLOTS]);
             }
-            // on every path: all MMAs this thread issued retire before the
-            // block frees TMEM (a wait that runs out is taken up again)
-            umma_commit(drain);
-            bool retired = false;
-            for (int r = 0; r < 64 && !retired; ++r) {
-                retired = mbar_wait(drain, 0, nullptr, lim);
-                if (!retired) set_status(status, TNET_ERR_TIMEOUT);
-            }
+            if (!ok) break;
+            umma_commit(lead, &acc_full[buf]);
+        }
+        if (!ok) {
+            set_status(status, TNET_ERR_TIMEOUT);
+            *abort_flag = 1;
+        }
+        // on every path: all MMAs this thread issued retire before the
+        // block frees TMEM (a wait that runs out is taken up again)
+        umma_commit(lead, drain);
+        bool retired = false;
+        for (int r = 0; r < 64 && !retired; ++r) {
+            retired = mbar_wait_warp(drain, 0, nullptr, lim);
+            if (!retired) set_status(status, TNET_ERR_TIMEOUT);
         }
     } else if (warp >= 2 + C::EPI) {
         if (X3) {  // converters: A -> (A_hi, A_lo) for every stage, in k order
