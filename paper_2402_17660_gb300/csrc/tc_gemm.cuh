@@ -12,7 +12,7 @@
 //          arrays of TF32-representable values, see tf32_split); three
 //          kind::tf32 MMAs per k-step, A_hi B_hi + A_lo B_hi + A_hi B_lo,
 //          within about 3 * 2^-22 |a||b| per product of the fp32 product.
-//          A's split is formed in shared memory: two converter warps rewrite
+//          A's split is formed in shared memory: converter warps rewrite
 //          each landed A tile into A_hi (in place) and A_lo (a second buffer)
 //          at the same byte offsets (an elementwise map, so the 128-byte
 //          swizzle carries over), fence it for the async proxy and release
@@ -42,7 +42,7 @@
 namespace tnet {
 namespace tc {
 
-constexpr int BM = 128, CONV_WARPS = 2;
+constexpr int BM = 128;
 constexpr int STG_LD = 20;  // floats per staged row (16 + pad, keeps float4 alignment)
 constexpr uint32_t kSpinLimit = 1u << 22;
 
@@ -278,7 +278,14 @@ struct TileCfg {
     // bytes TMA brings per pipeline stage: A, B (+ B_lo for TF32X3; A_lo is
     // formed in shared memory or TMEM)
     static constexpr uint32_t STAGE_TX = A_BYTES + (X3 ? 2 : 1) * B_BYTES;
-    static constexpr int CONV = A_TMEM ? 4 : CONV_WARPS;
+    // Converter warps.  A k-block's split takes four warps 780-1,370 cycles (with
+    // SiLU), longer than its MMAs: with A in TMEM two sets of four take the
+    // k-blocks in turn; in shared memory four warps share each (two for NK,
+    // whose epilogue is the longer).  Per call at 96,000 atoms, before and after:
+    // radial layer 3 (192) 4.04 -> 3.85 ms, its adjoint (256) 4.55 -> 4.25, the
+    // 32-wide GEMMs 1.64 -> 1.50; eight in shared memory 4.33.
+    static constexpr int CONV = A_TMEM ? 8 : (X3 && !NK ? 4 : 2);
+    static constexpr int CONV_ARRIVE = A_TMEM ? 4 : CONV;  // converter warps per stage
     // A_TMEM: slot a holds a k-block's A_hi (ROW / 4 columns) then A_lo at
     // A_COL + a * A_SLOT_COLS; the slots fill TMEM beside the accumulators
     // (2 at BN = 192, 4 at 128) and are released by their own commit barriers
@@ -403,7 +410,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], cl);  // released by the MMA issuer of every CTA of the cluster
-            mbar_init(&conv[s], C::CONV);
+            mbar_init(&conv[s], C::CONV_ARRIVE);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -534,6 +541,8 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
             for (int t = t_first; ok && next_tile(t, z, m0, n0) && !*abort_flag; t += t_step) {
                 for (int kb = 0; kb < nk; ++kb, ++kg) {
                     const int s = kg % STAGES;
+                    // two sets of converter warps take the k-blocks in turn
+                    if (C::CONV > C::CONV_ARRIVE && (kg & 1) != ct / (32 * C::CONV_ARRIVE)) continue;
                     if (!mbar_wait(&full[s], (kg / STAGES) & 1, abort_flag, lim)) {
                         ok = false;
                         break;
@@ -578,7 +587,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
                         float4 *hi = reinterpret_cast<float4 *>(sA + s * C::A_BYTES);
                         float4 *lo = reinterpret_cast<float4 *>(sAlo + s * C::A_BYTES);
 #pragma unroll 4
-                        for (int i = ct; i < (int)(C::A_BYTES / 16); i += 32 * CONV_WARPS) {
+                        for (int i = ct; i < (int)(C::A_BYTES / 16); i += 32 * C::CONV) {
                             float4 v = hi[i], l;
                             if (P.a_silu) {
                                 v.x = silu_f(v.x); v.y = silu_f(v.y); v.z = silu_f(v.z); v.w = silu_f(v.w);
