@@ -16,8 +16,8 @@ from tests.gpu_helpers import (DEV, E_TOL, F_TOL, energy_errors, force_errors, g
 
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs CUDA")]
 
-SHAPE = synth.ModelShape()
-W = synth.init_weights(SHAPE, seed=0)
+SHAPES = {F: synth.ModelShape(F=F) for F in (64, 128)}
+WEIGHTS = {F: synth.init_weights(s, seed=0) for F, s in SHAPES.items()}
 KNOB, STAGED, CHANNEL = 6, 3, 1
 
 
@@ -34,26 +34,27 @@ def _cloud(n, side, seed):
 # (atoms, cube side): group remainders of 6 and 12 rows; 130 and 280 atoms in
 # 5 A have rows of up to 129 and about 270 active edges (two and three passes);
 # 2,000 atoms pass one group per SM; 40 atoms in 60 A have none
+@pytest.mark.parametrize("F", [64, 128])
 @pytest.mark.parametrize("n,side", [(1, 3.0), (5, 4.0), (12, 5.0), (13, 5.0), (40, 60.0), (130, 5.0), (280, 5.0),
                                     (2000, 30.0)])
-def test_staged_form(n, side):
+def test_staged_form(n, side, F):
     s = _cloud(n, side, seed=n)
     got = {}
     for form in (STAGED, CHANNEL):
-        m = TensorNet(W, max_atoms=n, max_pairs=max(64, min(n * n, 600 * n)), device=DEV)
+        m = TensorNet(WEIGHTS[F], F=F, max_atoms=n, max_pairs=max(64, min(n * n, 600 * n)), device=DEV)
         knobs = m.get_tuning()
         knobs[KNOB] = form
         m.set_tuning(knobs)
         nl = gpu_pairs(m, s)
         z, pos, _, _ = to_dev(s)
-        E, F, _ = m.energy_forces(z, pos, nl)
+        E, Fo, _ = m.energy_forces(z, pos, nl)
         m.check_status("energy_forces")
-        got[form] = E.cpu().numpy(), F.cpu().numpy()
+        got[form] = E.cpu().numpy(), Fo.cpu().numpy()
     assert np.array_equal(got[STAGED][0], got[CHANNEL][0])
-    Es, Ei, Fo = oracle_energy_forces(W, s)
-    E, F = got[STAGED]
+    Es, Ei, Fo = oracle_energy_forces(WEIGHTS[F], s, SHAPES[F])
+    E, Fg = got[STAGED]
     assert energy_errors(E, Es, Ei, s.batch).max() <= E_TOL
     if np.abs(Fo).max() > 0:
-        assert force_errors(F, Fo)[0] <= F_TOL
+        assert force_errors(Fg, Fo)[0] <= F_TOL
     else:
-        assert np.abs(F).max() == 0
+        assert np.abs(Fg).max() == 0
