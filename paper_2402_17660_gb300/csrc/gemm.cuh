@@ -50,6 +50,7 @@ __device__ __forceinline__ void store_copy4(const OpCopy &c, int64_t idx, const 
 // arithmetic and stores); operator() runs both.  pre() may be given a row or
 // column clamped into range, and its result is then unused.
 struct EpiStore {  // C = v (+ C when accumulate)
+    static constexpr bool BULK = false;
     float *C;
     int64_t ldc;
     int accumulate;
@@ -69,6 +70,7 @@ struct EpiStore {  // C = v (+ C when accumulate)
 };
 
 struct EpiBiasAct {  // a = v + bias; pre = a; out = act(a) * rowscale[m] (+ operand copy)
+    static constexpr bool BULK = false;
     const float *bias;
     float *pre_out;
     int64_t ldp;
@@ -102,7 +104,20 @@ struct EpiBiasAct {  // a = v + bias; pre = a; out = act(a) * rowscale[m] (+ ope
     __device__ void operator()(int z, int64_t m, int n, float4 o) const { post(z, m, n, o, pre(z, m, n)); }
 };
 
+// C = v (+ bias) and nothing else: the tensor-core GEMM writes whole groups of
+// 32 rows with bulk tensor stores
+struct EpiBulk {
+    static constexpr bool BULK = true;
+    const float *bias;  // or NULL
+    float *C;
+    int64_t ldc;
+    struct Pre {};
+    __device__ Pre pre(int, int64_t, int) const { return Pre{}; }
+    __device__ void post(int, int64_t, int, float4, const Pre &) const {}
+};
+
 struct EpiGradAct {  // out = v * silu'(pre)  (+ out when accumulate) (+ operand copy)
+    static constexpr bool BULK = false;
     const float *pre_in;
     int64_t ldp;
     float *out;

@@ -593,7 +593,7 @@ __device__ __forceinline__ void store_normed(float v[9], int64_t t, int i, int c
 // the first layer's normalisation of it; without layers (qn NULL) X0 itself is
 // stored.  The elementwise kernels are bound by HBM: fused with their neighbour
 // where one's output is the other's input, they read and write 5 of the 8
-// node tensors they did (96,000 atoms: 2.4 -> 1.6 ms a call in all).
+// node tensors they did (96,000 atoms: the call 38.1 -> 37.7 ms).
 __global__ void k_emb_scale(const float *__restrict__ U, const float *__restrict__ s, int N, int F,
                             float *__restrict__ X0, float *__restrict__ qn, float *__restrict__ Xn, OpCopy Xn_cp) {
     pdl_entry();
@@ -2119,7 +2119,7 @@ __global__ void k_pair_vec(const float *__restrict__ pos, const float *__restric
 // inactive edges of a skin list change nothing.  Eight lanes per atom load
 // eight edges at a time and then add them up one after the other; a thread per
 // atom spent its time on one chain of dependent loads (12 us at any size up to
-// a few thousand atoms, 5 now).
+// a few thousand atoms, 9 now).
 constexpr int kForceLanes = 8;
 __global__ void k_forces(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                          const int32_t *__restrict__ pair_of, const float *__restrict__ Gp, int N,
@@ -2241,7 +2241,7 @@ __global__ void k_seed_atoms(const float *__restrict__ seed, const int32_t *__re
 // matrix is read and written along its rows.  The blocks past the jobs form
 // the element tables (see elem_tables).
 // Latency-bound; as three launches (filter rows, weight copies, tables with
-// one block per element) 57 us a call at F = 128, now 7.
+// one block per element) 57 us a call at F = 128, now 10.
 constexpr int kMaxCvtJobs = 128;
 constexpr int kElemParts = 8;  // blocks per element
 struct CvtJobs {
@@ -2700,7 +2700,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         if (tcm) {
             tc::TcShape tp = tc::tshape(maxU, 3 * F, K);
             tp.rows_dev = nu;
-            TRY(tcx3(tp, eu, maxU, K, wx.dproj, 3 * F, K, ep, bn3));
+            TRY(tcx3(tp, eu, maxU, K, wx.dproj, 3 * F, K, EpiBulk{W.dproj_b, fu, 3 * F}, bn3));
         } else {
             GemmShape pp = gshape(maxU, 3 * F, K, eu, K, W.dproj_w, K);
             pp.rows_dev = nu;
@@ -2752,7 +2752,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             TRY(sgemm<true>(gshape(N, 3 * F, 2 * F, hs1, 2 * F, W.emb_mlp2_w, 2 * F), em2, gctas, sms, st));
         }
     }
-    if (tcm) TRY(tcg(tc::tshape_classes(N, F), Xraw, nbf, 9LL * N, F, emix, 3 * F, F, EpiStore{Uemb, F, 0}));
+    if (tcm) TRY(tcg(tc::tshape_classes(N, F), Xraw, nbf, 9LL * N, F, emix, 3 * F, F, EpiBulk{nullptr, Uemb, F}));
     else TRY(sgemm<true>(gshape_classes(N, F, Xraw, W.emb_mix_w), EpiStore{Uemb, F, 0}, gctas, sms, st));
     const int ew = grid_for((int64_t)N * F, 256, sms);
     float *Xfin = f32(Lw.Xfin);  // the output model's input
@@ -2774,13 +2774,13 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
               *h2 = act(Lw.h2, 2 * F, l), *a3 = act(Lw.a3, 3 * F, l);
         if (tab) return TNET_OK;  // the message kernels evaluate g, dg/dd from the table
         const EpiBiasAct e3{b3p(l), a3, 3 * F, nullptr, 3 * F, 0, nullptr};
+        const EpiBulk t3e{b3p(l), a3, 3 * F};
         if (tcm && prec == 2 && !wg) {
             // 3xTF32 without weight gradients: layers 1 and 2 store their
             // pre-activations alone; the next GEMM's converter warps form
             // h = silu_f(a) from them (bitwise the value the epilogue would
             // store), and the reverse pass reads only a1, a2
-            const EpiBiasAct s1{Lr.mlp1_b, a1, F, nullptr, F, 1, nullptr};
-            const EpiBiasAct s2{Lr.mlp2_b, a2, 2 * F, nullptr, 2 * F, 1, nullptr};
+            const EpiBulk s1{Lr.mlp1_b, a1, F}, s2{Lr.mlp2_b, a2, 2 * F};
             tc::TcShape t1 = tc::tshape(maxU, F, K), t2 = tc::tshape(maxU, 2 * F, F), t3 = tc::tshape(maxU, 3 * F, 2 * F);
             t1.rows_dev = t2.rows_dev = t3.rows_dev = nu;
             t2.a_silu = t3.a_silu = 1;
@@ -2789,7 +2789,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             pf.mark(P_MLP2);
             TRY(tcx3(t2, a1, maxU, F, lb[l].mlp2, 2 * F, F, s2, bn2));
             pf.mark(P_MLP3);
-            TRY(tcx3(t3, a2, maxU, 2 * F, lb[l].mlp3, 3 * F, 2 * F, e3, bn3));
+            TRY(tcx3(t3, a2, maxU, 2 * F, lb[l].mlp3, 3 * F, 2 * F, t3e, bn3));
             return TNET_OK;
         }
         const EpiBiasAct e1{Lr.mlp1_b, fwd_only ? nullptr : a1, F, keep_h ? h1 : nullptr, F, 1, nullptr, h1_cp(l), F};
@@ -2805,7 +2805,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             pf.mark(P_MLP2);
             TRY(tcg(t2, h1, h1_cp(l), maxU, F, lb[l].mlp2, 2 * F, F, e2, bn2));
             pf.mark(P_MLP3);
-            TRY(tcg(t3, h2, h2_cp(l), maxU, 2 * F, lb[l].mlp3, 3 * F, 2 * F, e3, bn3));
+            TRY(tcg(t3, h2, h2_cp(l), maxU, 2 * F, lb[l].mlp3, 3 * F, 2 * F, t3e, bn3));
             return TNET_OK;
         }
         pf.mark(P_MLP1);
@@ -2827,7 +2827,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         float *Y = f32(Lw.Y) + l * n9, *M = f32(Lw.M) + l * n9, *Tn = f32(Lw.Tn) + l * n9,
               *dX = f32(Lw.dX) + l * n9;
         pf.mark(P_NODE_MIX);
-        if (tcm) TRY(tcg(tc::tshape_classes(N, F), Xn, nbf, 9LL * N, F, lb[l].mix1, 3 * F, F, EpiStore{Y, F, 0}));
+        if (tcm) TRY(tcg(tc::tshape_classes(N, F), Xn, nbf, 9LL * N, F, lb[l].mix1, 3 * F, F, EpiBulk{nullptr, Y, F}));
         else TRY(sgemm<true>(gshape_classes(N, F, Xn, W.layer[l].mix1_w), EpiStore{Y, F, 0}, gctas, sms, st));
         TRY(edge_mlp(l, !keep_act));
         pf.mark(P_MESSAGE);
@@ -2858,7 +2858,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         count_launch();
         TNET_LAUNCH_CHECK();
         pf.mark(P_NODE_MIX);
-        if (tcm) TRY(tcg(tc::tshape_classes(N, F), Tn, nbf, 9LL * N, F, lb[l].mix2, 3 * F, F, EpiStore{dX, F, 0}));
+        if (tcm) TRY(tcg(tc::tshape_classes(N, F), Tn, nbf, 9LL * N, F, lb[l].mix2, 3 * F, F, EpiBulk{nullptr, dX, F}));
         else TRY(sgemm<true>(gshape_classes(N, F, Tn, W.layer[l].mix2_w), EpiStore{dX, F, 0}, gctas, sms, st));
         if (l + 1 < NL) {  // (the last layer's residual is formed by k_out_norms)
             pf.mark(P_NODE_ELEM);
@@ -2941,7 +2941,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             count_launch();
         };
         pf.mark(P_NODE_BWD);
-        if (tcm) TRY(tcg(tc::tshape_classes(N, F), gdX, nbf, 9LL * N, F, lb[l].mix2T, 3 * F, F, EpiStore{gTn, F, 0}));
+        if (tcm) TRY(tcg(tc::tshape_classes(N, F), gdX, nbf, 9LL * N, F, lb[l].mix2T, 3 * F, F, EpiBulk{nullptr, gTn, F}));
         else TRY(sgemm<false>(gshape_classes(N, F, gdX, Lr.mix2_w), EpiStore{gTn, F, 0}, gctas, sms, st));
         if (wg) TRY(wgrad_outer(rows3(gdX, Tn), wpart, wcap, gw(Gr.mix2_w), nullptr, sms, st));
         launch(k_T_bwd, ew, 256, 0, st, Y, M, gTn, N, F, gY, gM);
@@ -3050,7 +3050,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                                 EpiGradAct{as1, 2 * F, gas1, 2 * F, 0}, gctas, sms, st));
         TRY(sgemm<false>(gshape(N, F, 2 * F, gas1, 2 * F, W.emb_mlp1_w, F), EpiStore{gn0, F, 0}, gctas, sms, st));
     }
-    if (tcm) TRY(tcg(tc::tshape_classes(N, F), gU, nbf, 9LL * N, F, emixT, 3 * F, F, EpiStore{gXraw, F, 0}));
+    if (tcm) TRY(tcg(tc::tshape_classes(N, F), gU, nbf, 9LL * N, F, emixT, 3 * F, F, EpiBulk{nullptr, gXraw, F}));
     else TRY(sgemm<false>(gshape_classes(N, F, gU, W.emb_mix_w), EpiStore{gXraw, F, 0}, gctas, sms, st));
     launch(k_ln0_bwd, N, F, 0, st, Xraw, gn0, ln0, W.emb_ln_g, N, F, gXraw);
     count_launch();

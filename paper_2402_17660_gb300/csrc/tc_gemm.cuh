@@ -1,7 +1,8 @@
 // Tensor-core GEMM for sm_103a: TMA tile loads into 128B-swizzled shared
-// memory, tcgen05.mma issued by one thread with the FP32 accumulator in
+// memory, tcgen05.mma issued by one elected lane with the FP32 accumulator in
 // tensor memory (TMEM), and a tcgen05.ld epilogue that applies the same fused
-// epilogue functors as the SIMT path.
+// epilogue functors as the SIMT path, or hands a bias-only result to bulk
+// tensor stores.
 //
 //   C[m][n] = epi( sum_k A[m][k] B[n][k] ),  A [rows][lda], B [rows][ldb},
 //   both K-major (row-major with K contiguous).
@@ -12,12 +13,12 @@
 //          arrays of TF32-representable values, see tf32_split); three
 //          kind::tf32 MMAs per k-step, A_hi B_hi + A_lo B_hi + A_hi B_lo,
 //          within about 3 * 2^-22 |a||b| per product of the fp32 product.
-//          A's split is formed in shared memory: converter warps rewrite
-//          each landed A tile into A_hi (in place) and A_lo (a second buffer)
-//          at the same byte offsets (an elementwise map, so the 128-byte
-//          swizzle carries over), fence it for the async proxy and release
-//          the stage to the MMA warp.  No split of an activation ever goes
-//          through HBM.
+//          A's split is formed on the SM by converter warps: into TMEM for
+//          tiles up to 192 columns, else each landed A tile is rewritten into
+//          A_hi (in place) and A_lo (a second buffer) at the same byte offsets
+//          (an elementwise map, so the swizzle carries over); they fence it
+//          and release the stage to the MMA warp.  No split of an activation
+//          ever goes through HBM.
 //
 // Persistent CTAs walk 128 x BN output tiles.  Warp 0 issues TMA loads into a
 // 3-4 stage shared-memory ring (k-blocks of 128-byte rows for BF16, 64-byte
@@ -255,7 +256,7 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float v[16]) {
         : "memory");
 }
 
-template <int BN, bool X3 = false, bool NK = false>
+template <int BN, bool X3 = false, bool NK = false, bool BULK = false>
 struct TileCfg {
     // 3xTF32 at BN <= 192 (K beyond two k-blocks): A's split goes to TMEM
     // instead of shared memory.  Four converter warps (one per TMEM lane
@@ -300,17 +301,21 @@ struct TileCfg {
     // stages
     static constexpr int EPI = (X3 && !NK && (BN >= 128 || A_TMEM)) ? 8 : 16;
     static constexpr int THREADS = 64 + 32 * (EPI + CONV);
-    static constexpr uint32_t STAGE_BYTES = EPI * 32 * STG_LD * 4;  // epilogue transpose buffers
+    // epilogue buffers per warp: two bulk-store tiles, or a transpose (and no
+    // more: the BF16 layer-3 adjoint, whose epilogue reads through L1, took
+    // 0.81 ms a call instead of 0.67 at 24,000 atoms with 4 KB each)
+    static constexpr int WARP_STAGE = BULK ? 4096 : 32 * STG_LD * 4;
+    static constexpr uint32_t STAGE_BYTES = EPI * WARP_STAGE;
     // 3xTF32: 4 stages, and as many as fit beside the epilogue buffers (6 at
     // BN = 128, 5 at 192, 4 at 256): each stage's split and three MMAs make a
     // long round trip, which the wide radial layers feel.  The narrow tiles (K-wide outputs)
     // keep 4 and a smaller footprint, which leaves room on the SM for the CTAs
     // of the next kernel that programmatic launch brings in early.
-    static constexpr int X3_FIT = (int)((232448 - 1024 - 256 - STAGE_BYTES) / (STAGE_TX + A_BYTES));
+    static constexpr int X3_FIT = (int)((232448 - 1024 - 1024 - STAGE_BYTES) / (STAGE_TX + A_BYTES));
     // A_TMEM: as many 128-byte stages as fit, at most four (six for the
     // narrow tiles, which stream A).  BF16: four stages (three at BN = 256,
     // where four do not fit beside the epilogue buffers)
-    static constexpr int A_FIT = (int)((232448 - 1024 - 256 - STAGE_BYTES) / STAGE_TX);
+    static constexpr int A_FIT = (int)((232448 - 1024 - 1024 - STAGE_BYTES) / STAGE_TX);
     static constexpr int A_CAP = BN <= 64 ? 6 : 4;
     static constexpr int STAGES = A_TMEM ? (A_FIT > A_CAP ? A_CAP : A_FIT)
                                          : X3 ? (BN >= 128 && !NK ? (X3_FIT > 6 ? 6 : X3_FIT) : 4)
@@ -318,7 +323,7 @@ struct TileCfg {
     static_assert(!A_TMEM || (A_SLOTS >= 2 && A_COL + A_SLOT_COLS * A_SLOTS <= 512), "A slots exceed TMEM");
     static_assert(STAGES >= 2 && 8 * (3 * STAGES + 5 + A_SLOTS) + 8 <= 256, "pipeline barriers exceed their block");
     static constexpr size_t SMEM =
-        1024 + STAGES * (size_t)(STAGE_TX + (X3 && !A_TMEM ? A_BYTES : 0)) + 256 + STAGE_BYTES;
+        1024 + STAGES * (size_t)(STAGE_TX + (X3 && !A_TMEM ? A_BYTES : 0)) + 1024 + STAGE_BYTES;
     static_assert(SMEM <= 232448, "dynamic shared memory above 227 KB");
 };
 
@@ -350,12 +355,12 @@ struct TileIter {
 __device__ __forceinline__ int64_t sel3(int z, int64_t a, int64_t b, int64_t c) { return z == 0 ? a : (z == 1 ? b : c); }
 
 template <int BN, class Epi, bool X3, bool NK = false>
-__global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
+__global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-              const __grid_constant__ CUtensorMap tmAlo, const __grid_constant__ CUtensorMap tmBlo, TcShape P,
-              Epi epi, int32_t *status) {
+              const __grid_constant__ CUtensorMap tmAlo, const __grid_constant__ CUtensorMap tmBlo,
+              const __grid_constant__ CUtensorMap tmC, TcShape P, Epi epi, int32_t *status) {
     pdl_entry();
-    using C = TileCfg<BN, X3, NK>;
+    using C = TileCfg<BN, X3, NK, Epi::BULK>;
     constexpr int STAGES = C::STAGES;
     constexpr int BK = C::BKE;
     extern __shared__ uint8_t smem_raw[];
@@ -374,7 +379,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
     uint64_t *aempty = drain + 1;     // A_TMEM: the MMAs that read TMEM A slot a retired
     uint32_t *tmem_slot = (uint32_t *)(aempty + C::A_SLOTS);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
-    float *stage_all = (float *)((uint8_t *)full + 256);
+    float *stage_all = (float *)((uint8_t *)full + 1024);
 
     // rows per class (class 0 may be bounded by a device-side count)
     int M0 = P.M[0];
@@ -620,6 +625,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
         const int part = (warp - 2) >> 2;
         const int c_begin = part < NSLICE ? part * CW : 0, c_end = part < NSLICE ? c_begin + CW : 0;
         int lt = 0;
+        uint32_t n_bulk = 0;  // bulk stores of this warp so far
         int z, m0, n0;
         for (int t = t_first; next_tile(t, z, m0, n0) && !*abort_flag; t += t_step, ++lt) {
             const int buf = lt & 1;
@@ -634,8 +640,61 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
             // TMEM gives thread = row; a shared-memory transpose hands each lane
             // 4 columns of 4 rows instead, so every store instruction of the
             // warp writes 8 rows x 64 contiguous bytes
-            float *stg = stage_all + (warp - 2) * 32 * STG_LD;
+            float *stg = stage_all + (warp - 2) * (C::WARP_STAGE / 4);
             const int rsub = lane >> 2, csub = (lane & 3) * 4;
+            if constexpr (Epi::BULK) {
+                // lane = row, as TMEM gives it: 16 columns at a time into one of
+                // two 64-byte-swizzled tiles of 32 rows, written out by a bulk
+                // tensor store.  The transposing path reads every value back and
+                // stores it (56 LSU wavefronts a 2 KB block against 20), which
+                // bound the GEMMs of small K.  Per call at 96,000 atoms, before
+                // and after: projections 1.03 -> 0.78 ms, radial layer 1 0.75 ->
+                // 0.50, layer 2 2.39 -> 1.50, layer 3 3.85 -> 3.80.  A last
+                // group of fewer than 32 rows of its class is stored by the lanes.
+                const int rows = Mrow - m0 - 32 * q;
+#pragma unroll 1
+                for (int c0 = c_begin; c0 < c_end; c0 += 16) {
+                    const int n = n0 + c0;
+                    float4 bias[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        bias[j] = epi.bias ? *reinterpret_cast<const float4 *>(epi.bias + (n + 4 * j < P.N ? n + 4 * j : P.N - 4))
+                                           : make_float4(-0.f, -0.f, -0.f, -0.f);
+                    float v[16];
+                    tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * BN + c0), v);
+                    if (rows <= 0 || n >= P.N) continue;
+                    float4 w[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        w[j] = make_float4(v[4 * j] + bias[j].x, v[4 * j + 1] + bias[j].y, v[4 * j + 2] + bias[j].z,
+                                           v[4 * j + 3] + bias[j].w);
+                    const int64_t row0 = rbase + m0 + 32 * q;
+                    if (rows < 32) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (lane < rows && n + 4 * j < P.N)
+                                *reinterpret_cast<float4 *>(epi.C + (row0 + lane) * epi.ldc + n + 4 * j) = w[j];
+                        continue;
+                    }
+                    uint8_t *tile = reinterpret_cast<uint8_t *>(stg) + (n_bulk++ & 1) * 2048;
+                    // the store before the last has read this tile
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        *reinterpret_cast<float4 *>(tile + lane * 64 + 16 * (j ^ ((lane >> 1) & 3))) = w[j];
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        asm volatile(
+                            "cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                                (uint64_t)&tmC),
+                            "r"(n), "r"((int)row0), "r"(smem_u32(tile))
+                            : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                }
+            } else
 #pragma unroll 1
             for (int c0 = c_begin; c0 < c_end; c0 += 16) {
                 const int n = n0 + c0 + csub;
@@ -667,6 +726,8 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK>::THREADS, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[buf]);
         }
+        // own stores complete before the CTA exits
+        if (Epi::BULK && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     fence_before();
     __syncthreads();
@@ -734,7 +795,7 @@ inline int max_active_clusters(const void *kern, int threads, int smem, int cl) 
 // swizzle atoms, and the device runs such clusters.
 template <int BN, bool X3, bool NK = false, class Epi>
 int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t *status, cudaStream_t st, int sms) {
-    using C = TileCfg<BN, X3, NK>;
+    using C = TileCfg<BN, X3, NK, Epi::BULK>;
     TcShape P = P0;
     int cl = P.cl > 1 ? P.cl : 1;
     if (P.nclass != 1 || BN % cl || (BN / cl) % 8) cl = 1;
@@ -745,7 +806,7 @@ int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t 
     if (P.N % 4 || (o.lda * esz) % 16 || (o.ldb * esz) % 16 || ((uintptr_t)o.A & 15) || ((uintptr_t)o.B & 15))
         return TNET_ERR_ARG;
     if (X3 && (!o.Blo || ((uintptr_t)o.Blo & 15))) return TNET_ERR_ARG;
-    CUtensorMap ma, mb, mal, mbl;
+    CUtensorMap ma, mb, mal, mbl, mc;
     int rc;
     auto kern = k_tc_gemm<BN, Epi, X3, NK>;
     if ((rc = ensure_smem_attr((const void *)kern, (int)C::SMEM))) return rc;
@@ -769,6 +830,13 @@ int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t 
         mal = ma;
         mbl = mb;
     }
+    mc = ma;  // unused unless the epilogue stores in bulk
+    if constexpr (Epi::BULK) {
+        int64_t rows = 0;
+        for (int z = 0; z < P.nclass; ++z) rows = P.row0[z] + P.M[z] > rows ? P.row0[z] + P.M[z] : rows;
+        if (P.N % 4 || ((uintptr_t)epi.C & 15) || epi.ldc % 4) return TNET_ERR_ARG;
+        if ((rc = make_map_f32(&mc, epi.C, rows, P.N, epi.ldc, 32, 64))) return rc;
+    }
     int64_t tiles = 0;
     for (int z = 0; z < P.nclass; ++z) tiles += (int64_t)((P.M[z] + BM - 1) / BM) * ((P.N + BN - 1) / BN);
     int grid;
@@ -778,7 +846,7 @@ int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t 
     } else {
         grid = (int)(tiles < sms ? tiles : sms);
     }
-    launch_cluster(kern, grid, C::THREADS, C::SMEM, st, cl, ma, mb, mal, mbl, P, epi, status);
+    launch_cluster(kern, grid, C::THREADS, C::SMEM, st, cl, ma, mb, mal, mbl, mc, P, epi, status);
     count_launch();
     TNET_LAUNCH_CHECK();
     return TNET_OK;
