@@ -320,6 +320,7 @@ struct TileCfg {
     static constexpr int STAGES = A_TMEM ? (A_FIT > A_CAP ? A_CAP : A_FIT)
                                          : X3 ? (BN >= 128 && !NK ? (X3_FIT > 6 ? 6 : X3_FIT) : 4)
                                               : (BN >= 256 ? 3 : 4);
+    static_assert(CONV == CONV_ARRIVE || (A_SLOTS % 2 == 0 && A_SLOTS <= STAGES), "a converter set could miss a phase");
     static_assert(!A_TMEM || (A_SLOTS >= 2 && A_COL + A_SLOT_COLS * A_SLOTS <= 512), "A slots exceed TMEM");
     static_assert(STAGES >= 2 && 8 * (3 * STAGES + 5 + A_SLOTS) + 8 <= 256, "pipeline barriers exceed their block");
     static constexpr size_t SMEM =
@@ -548,6 +549,18 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
                     const int s = kg % STAGES;
                     // two sets of converter warps take the k-blocks in turn
                     if (C::CONV > C::CONV_ARRIVE && (kg & 1) != ct / (32 * C::CONV_ARRIVE)) continue;
+                    // The slot's last readers, the MMAs of k-block kg - A_SLOTS, must
+                    // have retired.  Waited for first: a set that sees every
+                    // other k-block skips every other use of a stage when STAGES is
+                    // odd, and a parity wait on `full` tells its phase from the
+                    // next but not from the one after; with A_SLOTS <= STAGES the
+                    // retired MMAs show that the stage's last use is over.
+                    const int a = kg % C::A_SLOTS;
+                    if (C::A_TMEM && kg >= C::A_SLOTS &&
+                        !mbar_wait(&aempty[a], ((kg / C::A_SLOTS) - 1) & 1, abort_flag, lim)) {
+                        ok = false;
+                        break;
+                    }
                     if (!mbar_wait(&full[s], (kg / STAGES) & 1, abort_flag, lim)) {
                         ok = false;
                         break;
@@ -558,14 +571,6 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
                         // (TMA's 128-byte swizzle)
                         const int q = warp & 3, r = 32 * q + lane;
                         const float4 *row = reinterpret_cast<const float4 *>(sA + s * C::A_BYTES + r * C::ROW);
-                        // the slot's last readers, the MMAs of k-block kg - A_SLOTS,
-                        // must have retired
-                        const int a = kg % C::A_SLOTS;
-                        if (kg >= C::A_SLOTS &&
-                            !mbar_wait(&aempty[a], ((kg / C::A_SLOTS) - 1) & 1, abort_flag, lim)) {
-                            ok = false;
-                            break;
-                        }
                         fence_after();
                         const uint32_t ta =
                             tmem + ((uint32_t)(32 * q) << 16) + C::A_COL + (uint32_t)(C::A_SLOT_COLS * a);
