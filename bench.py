@@ -363,6 +363,8 @@ def stage_work(tag, nu, N, E, F, K, prec, table=0, rec=False):
             return None
     pre = 0.5 if rec else 1.0            # share of instances that store the pre-activation
     hw = (f if not bf16 else 0.0) + cp   # bytes stored per activation element (fp32 unless BF16 copies only)
+    if prec == "tf32x3":                 # layers 1 and 2 store their pre-activations alone, in every instance
+        pre, hw = 1.0, 0.0
     if tag == "mlp1":
         return 2.0 * nu * K * F, nu * (K * f + pre * F * f + F * hw), "alu"
     if tag == "mlp2":
