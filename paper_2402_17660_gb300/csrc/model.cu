@@ -2242,7 +2242,10 @@ __global__ void k_seed_atoms(const float *__restrict__ seed, const int32_t *__re
 // the element tables (see elem_tables).
 // Latency-bound; as three launches (filter rows, weight copies, tables with
 // one block per element) 57 us a call at F = 128, now 10.
-constexpr int kMaxCvtJobs = 128;
+// at most 16 per layer (two filter copies, ten operands, two of them by class)
+// of at most 8 layers, 4 + 2 + 8 beside them
+constexpr int kMaxCvtJobs = 144;
+static_assert(8 * 16 + 14 <= kMaxCvtJobs, "conversion jobs");
 constexpr int kElemParts = 8;  // blocks per element
 struct CvtJobs {
     const float *src[kMaxCvtJobs];
@@ -2619,7 +2622,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             wx.head1 = job3(W.head1_w, H, F, 0);
             wx.head1T = job3(W.head1_w, H, F, 1);
         }
-        if (woff > Lw.wbf_bytes) return TNET_ERR_WORKSPACE;
+        if (woff > Lw.wbf_bytes || J.n > kMaxCvtJobs) return TNET_ERR_WORKSPACE;
     }
     {
         const ElemTables et{W.emb, W.emb2_w, W.emb2_b, F, d.max_z, Ta, Tb};
