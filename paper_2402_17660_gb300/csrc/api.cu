@@ -44,6 +44,7 @@ int build_layout(const tnet_model_desc *d, int N, int S, int64_t E, Layout *L) {
     // neighbor search
     L->sys_start = take(i * S);
     L->sys_end = take(i * S);
+    L->rows_bad = take(i);
     L->sysinfo = take(sizeof(SysInfo) * S);
     L->sys_ncell = take(i * (S + 1));
     L->cell_count = take(i * (cells + 1));

@@ -445,7 +445,7 @@ __device__ __forceinline__ int mark_bounds(const int32_t *__restrict__ batch, in
 // ------------------------------------------------------------ workspace ---
 struct Layout {
     // neighbor search
-    size_t sys_start, sys_end, sysinfo, sys_ncell, cell_count, cell_start, cell_fill, cell_of,
+    size_t sys_start, sys_end, rows_bad, sysinfo, sys_ncell, cell_count, cell_start, cell_fill, cell_of,
         sorted, spos, rowcnt, scan_tmp;
     // single-pass search: each row's sorted columns, kSlabWidth per atom, and
     // the flag of a row that did not fit (slab_width 0: two passes)

@@ -108,16 +108,22 @@ __device__ __forceinline__ int32_t row_offset(const int32_t *__restrict__ row_pt
 // One warp per row: the clamped copy of the row offsets that every later
 // kernel reads (offsets out of range or decreasing are reported as ARG, or
 // CAPACITY when they pass the capacity), the system bounds, the reverse edges
-// rev[e] = position of (j, i) in row j, and the count of the row's upper
-// (j > i) edges with d < rc.  Every edge starts inactive.  One launch in the
+// rev[e] = position of (j, i) in row j (e itself: none, reported as ARG), and
+// the count of the row's upper (j > i) edges with d < rc that have a reverse:
+// those become pairs, so a list that lacks half of its edges (a half list, a
+// truncated one) never has more pairs than half of its edges, which is what
+// the pair buffers hold.  Every edge starts inactive.  Decreasing offsets make
+// rows overlap, and rows that share edges would write each other's rev: they
+// raise rows_bad, and the list then has no pairs at all.  One launch in the
 // place of four (launches and their gaps were most of the time of small
 // systems' graph preparation).
 __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restrict__ box,
                              const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
                              const int32_t *__restrict__ col, int N, int S, int64_t cap, float rc,
                              int32_t *__restrict__ safe, int32_t *__restrict__ sys_start,
-                             int32_t *__restrict__ sys_end, int32_t *__restrict__ rev, int32_t *__restrict__ pair_of,
-                             int32_t *__restrict__ ucnt, int32_t *status) {
+                             int32_t *__restrict__ sys_end, int32_t *__restrict__ rows_bad,
+                             int32_t *__restrict__ rev, int32_t *__restrict__ pair_of, int32_t *__restrict__ ucnt,
+                             int32_t *status) {
     pdl_entry();
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (i >= N) return;
@@ -128,6 +134,7 @@ __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restr
         const int32_t v0 = row_ptr[i], v1 = row_ptr[i + 1];
         if (v0 < 0 || (i == 0 && v0 != 0) || v1 < 0 || v0 > v1) set_status(status, TNET_ERR_ARG);
         if (v0 > cap || v1 > cap) set_status(status, TNET_ERR_CAPACITY);
+        if (e0 > e1) *rows_bad = 1;
         safe[i] = e0;
         if (i == N - 1) safe[N] = e1;
     }
@@ -154,7 +161,7 @@ __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restr
             }
             rev[e] = r;
             pair_of[e] = -1;
-            if (j > i && j < N) {
+            if (r != e && j > i) {
                 float x, y, zz;
                 pair_vec(pos, box, batch, i, j, x, y, zz);
                 up = sqrtf(norm2_rn(x, y, zz)) < rc;
@@ -166,13 +173,21 @@ __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restr
 }
 
 // Numbers the active undirected pairs by their upper edges and tells both
-// directed edges (a lower edge without a reverse stays inactive).
+// directed edges (an edge without a reverse stays inactive).  Columns that
+// ascend strictly give at most E / 2 pairs; repeated columns (reported) can
+// give more, and those past maxU, the size of the pair buffers, stay inactive.
+// nu, the scan's total, is brought in line: the kernels after this one take
+// their pairs from it.
 __global__ void k_upper_assign(const float *__restrict__ pos, const float *__restrict__ box,
                                const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
                                const int32_t *__restrict__ col, const int32_t *__restrict__ rev, int N, float rc,
-                               const int32_t *__restrict__ uoff, int32_t *__restrict__ pair_of,
-                               int2 *__restrict__ uij, int32_t *__restrict__ ue) {
+                               const int32_t *__restrict__ uoff, const int32_t *__restrict__ rows_bad, int maxU,
+                               int32_t *__restrict__ nu, int32_t *__restrict__ pair_of, int2 *__restrict__ uij,
+                               int32_t *__restrict__ ue) {
     pdl_entry();
+    const bool bad = *rows_bad != 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && (bad || *nu > maxU)) *nu = bad ? 0 : maxU;
+    if (bad) return;
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (i >= N) return;
     const int lane = threadIdx.x & 31;
@@ -180,23 +195,23 @@ __global__ void k_upper_assign(const float *__restrict__ pos, const float *__res
     for (int e0 = row_ptr[i]; e0 < row_ptr[i + 1]; e0 += 32) {
         const int e = e0 + lane;
         bool up = false;
-        int j = -1;
+        int j = -1, r = -1;
         if (e < row_ptr[i + 1]) {
             j = col[e];
-            if (j > i && j < N) {
+            r = rev[e];
+            if (r != e && j > i) {
                 float x, y, zz;
                 pair_vec(pos, box, batch, i, j, x, y, zz);
                 up = sqrtf(norm2_rn(x, y, zz)) < rc;
             }
         }
         const unsigned m = __ballot_sync(0xffffffffu, up);
-        if (up) {
-            const int u = base + __popc(m & ((1u << lane) - 1u));
+        const int u = base + __popc(m & ((1u << lane) - 1u));
+        if (up && u < maxU) {
             pair_of[e] = u;
             uij[u] = make_int2(i, j);
             ue[u] = e;
-            const int r = rev[e];
-            if (r != e) pair_of[r] = u;
+            pair_of[r] = u;
         }
         base += __popc(m);
     }
@@ -2664,15 +2679,16 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
         }
         return tcx3(P, A32, a_rows, lda, w, b_rows, ldb, epi, bn);
     };
-    // (sys_start and sys_end are adjacent in the layout)
+    // (sys_start, sys_end and rows_bad are adjacent in the layout)
+    int32_t *rows_bad = i32(Lw.rows_bad);
     TNET_CUDA_TRY(cudaMemsetAsync(sys_start, 0, Lw.sysinfo - Lw.sys_start, st));
     launch(k_graph_rows, warps_grid, 256, 0, st, pos, box, batch, row_ptr_in, col, N, S, ctx->max_pairs, rp.rc, row_ptr,
-           sys_start, sys_end, rev, pair_of, ucnt, status);
+           sys_start, sys_end, rows_bad, rev, pair_of, ucnt, status);
     count_launch();
     TNET_LAUNCH_CHECK();
     TRY(scan_exclusive_i32(ucnt, ucnt, N, i32(Lw.scan_tmp), nu, nullptr, st));
-    launch(k_upper_assign, warps_grid, 256, 0, st, pos, box, batch, row_ptr, col, rev, N, rp.rc, ucnt, pair_of, uij,
-           ue);
+    launch(k_upper_assign, warps_grid, 256, 0, st, pos, box, batch, row_ptr, col, rev, N, rp.rc, ucnt, rows_bad, maxU,
+           nu, pair_of, uij, ue);
     count_launch();
     TNET_LAUNCH_CHECK();
     float *eu = f32(Lw.eu), *phiu = f32(Lw.phiu), *fu = f32(Lw.fu);
