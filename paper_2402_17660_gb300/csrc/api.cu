@@ -145,21 +145,14 @@ int build_layout(const tnet_model_desc *d, int N, int S, int64_t E, Layout *L) {
     L->tab = take(f * (nt > 0 ? (NL + 1) * (nt - 1) * 4 * 3 * F : 0));
     L->tab_tmp = take(8 * (nt > 0 ? nt * (2 * K + 2 + 12 * F) : 0));
     L->dist = take(f * (nt > 0 ? U : 0));
-    // tensor-core modes: weight operands (bf16 forward + transposed copies,
-    // or fp32 TF32 residuals + transposed high parts; the 3xTF32 GEMMs of the
-    // BF16 mode use the latter), and in BF16 mode the bf16 copies of the node
+    // tensor-core modes: weight operands (bf16 copies, forward and transposed,
+    // or TF32 high parts and residuals of both, 16 bytes a weight; the 3xTF32
+    // GEMMs of the BF16 mode use the latter), and in BF16 mode the bf16 copies of the node
     // tensor and radial-MLP activations the BF16 GEMMs read (3xTF32 reads the
     // fp32 activations themselves)
     const int prec = d->precision;
     const int64_t esz = prec == 1 ? 2 : 0;
-    int64_t nw = 0;
-    {
-        nw += Z * F + F * 2 * F + F + 3 * F * K + 3 * F + 2 * F + 2 * F * F + 2 * F + 3 * F * 2 * F + 3 * F +
-              3 * F * F;
-        nw += NL * (F * K + F + 2 * F * F + 2 * F + 3 * F * 2 * F + 3 * F + 6 * F * F);
-        nw += 6 * F + F * 3 * F + F + F / 2 * F + F / 2 + F / 2 + 1;
-    }
-    L->wbf_bytes = prec ? 3 * nw * 4 + 128 * 256 : 0;
+    L->wbf_bytes = weight_operand_bytes(d);
     L->wbf = take(L->wbf_bytes);
     L->nbf = take(esz * n9);
     L->eu_bf = 0;

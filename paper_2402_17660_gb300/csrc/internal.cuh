@@ -580,6 +580,7 @@ int scan_exclusive_i32(const int32_t *in, int32_t *out, int n, int32_t *tmp, int
                        int64_t *total64_dev, cudaStream_t st, const int32_t *gate = nullptr);
 int tnet_kernel_setup(tnet_ctx *c);
 int64_t weight_offsets(const tnet_model_desc *d, const float *base, struct Weights *w);
+int64_t weight_operand_bytes(const tnet_model_desc *d);  // of the tensor-core modes
 int neighbors_impl(tnet_ctx *ctx, int n_atoms, int n_systems, const float *pos, const int32_t *batch,
                    const float *box, float cutoff, int32_t *row_ptr, int32_t *col, int64_t cap,
                    int64_t *n_pairs_dev, int32_t *status_dev, cudaStream_t st, const int32_t *gate = nullptr);

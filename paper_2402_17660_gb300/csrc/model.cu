@@ -2339,6 +2339,113 @@ static void filter_row_jobs(CvtJobs &J, const LayerW &L, int F, float *w3p, floa
     }
 }
 
+// The tensor-core modes' weight operands, one set per call.
+// WeightOps::x3 holds 3xTF32 operands: of the num_rbf-wide radial layers in
+// both modes (rounding the narrow expnorm basis to bf16 costs more force
+// accuracy than any other operand), and of the per-atom embedding and output
+// MLPs in BF16 mode.  In the FP32-accurate mode those per-atom MLPs stay on
+// FP32 FMA: they are cheap, and the energy is the quantity most sensitive to
+// them (3xTF32 there costs an order of magnitude of energy accuracy).
+struct LayerOps {
+    WOp mlp2, mlp3, mlp2T, mlp3T, mix1, mix1T, mix2, mix2T, mlp1, mlp1T;
+};
+struct X3W {
+    WOp dproj, dprojT, emb_mlp1, emb_mlp1T, emb_mlp2, emb_mlp2T, out, outT, head1, head1T;
+};
+struct WeightOps {
+    LayerOps layer[8];
+    WOp emix, emixT;
+    X3W x3;
+};
+// Lays the operands out from wb and adds their jobs to J; returns the bytes
+// they take (none in FP32 mode).  The workspace is sized by the same walk (wb
+// NULL), so what a call lays out is what the context was given room for.
+static int64_t weight_operands(const tnet_model_desc &d, const Weights &W, char *wb, CvtJobs &J, WeightOps &o) {
+    o = WeightOps{};
+    const int F = d.F, K = d.K, NL = d.L, H = F / 2, prec = d.precision;
+    const bool tab = d.radial_table > 0;
+    if (!prec) return 0;
+    int64_t woff = 0;
+    auto alloc = [&](int64_t elems, int esz) {
+        void *p = wb ? wb + woff : nullptr;
+        woff += (elems * esz + 255) & ~(int64_t)255;
+        return p;
+    };
+    // forward operands keep the (out, in) = K-major layout; backward
+    // operands are transposed
+    auto job_m = [&](const float *src, int rows, int cols, int tr, int mode, int perm = 0) {
+        WOp w{};
+        const int esz = mode == 1 ? 2 : 4;
+        void *hi = alloc((int64_t)rows * cols, esz);
+        void *lo = mode == 2 ? alloc((int64_t)rows * cols, esz) : nullptr;
+        J.src[J.n] = src; J.hi[J.n] = hi; J.lo[J.n] = lo;
+        J.rows[J.n] = rows; J.cols[J.n] = cols; J.tr[J.n] = (signed char)tr; J.mode[J.n] = (signed char)mode;
+        J.perm[J.n] = (short)perm;
+        ++J.n;
+        w.b = hi;
+        w.blo = lo;
+        return w;
+    };
+    auto job = [&](const float *src, int rows, int cols, int tr) { return job_m(src, rows, cols, tr, prec); };
+    auto job3 = [&](const float *src, int rows, int cols, int tr) { return job_m(src, rows, cols, tr, 2); };
+    // [3][F][F] -> per-class transposes; the three classes' high parts (and
+    // residuals) must stay stacked contiguously [3F][F] for the GEMM
+    auto job_classes_T = [&](const float *src) {
+        const int64_t ff = (int64_t)F * F;
+        const int esz = prec == 1 ? 2 : 4;
+        char *hi = (char *)alloc(3 * ff, esz), *lo = prec == 2 ? (char *)alloc(3 * ff, esz) : nullptr;
+        for (int q = 0; q < 3; ++q) {
+            J.src[J.n] = src ? src + q * ff : nullptr;
+            J.hi[J.n] = hi ? hi + q * ff * esz : nullptr;
+            J.lo[J.n] = lo ? lo + q * ff * esz : nullptr;
+            J.rows[J.n] = F; J.cols[J.n] = F; J.tr[J.n] = 1; J.mode[J.n] = (signed char)prec; J.perm[J.n] = 0;
+            ++J.n;
+        }
+        return WOp{hi, lo};
+    };
+    o.emix = job(W.emb_mix_w, 3 * F, F, 0);
+    o.emixT = job_classes_T(W.emb_mix_w);
+    for (int l = 0; l < NL; ++l) {
+        const LayerW &Lr = W.layer[l];
+        LayerOps &lo = o.layer[l];
+        lo.mix1 = job(Lr.mix1_w, 3 * F, F, 0);
+        lo.mix1T = job_classes_T(Lr.mix1_w);
+        lo.mix2 = job(Lr.mix2_w, 3 * F, F, 0);
+        lo.mix2T = job_classes_T(Lr.mix2_w);
+        if (tab) continue;  // no per-pair radial MLP
+        lo.mlp2 = job(Lr.mlp2_w, 2 * F, F, 0);
+        lo.mlp3 = job_m(Lr.mlp3_w, 3 * F, 2 * F, 0, prec, F);
+        lo.mlp2T = job(Lr.mlp2_w, 2 * F, F, 1);
+        lo.mlp3T = job_m(Lr.mlp3_w, 3 * F, 2 * F, 1, prec, F);
+        lo.mlp1 = job3(Lr.mlp1_w, F, K, 0);
+        lo.mlp1T = job3(Lr.mlp1_w, F, K, 1);
+    }
+    if (!tab) {
+        o.x3.dproj = job3(W.dproj_w, 3 * F, K, 0);
+        o.x3.dprojT = job3(W.dproj_w, 3 * F, K, 1);
+    }
+    if (prec == 1) {  // (see X3W)
+        o.x3.emb_mlp1 = job3(W.emb_mlp1_w, 2 * F, F, 0);
+        o.x3.emb_mlp1T = job3(W.emb_mlp1_w, 2 * F, F, 1);
+        o.x3.emb_mlp2 = job3(W.emb_mlp2_w, 3 * F, 2 * F, 0);
+        o.x3.emb_mlp2T = job3(W.emb_mlp2_w, 3 * F, 2 * F, 1);
+        o.x3.out = job3(W.out_w, F, 3 * F, 0);
+        o.x3.outT = job3(W.out_w, F, 3 * F, 1);
+        o.x3.head1 = job3(W.head1_w, H, F, 0);
+        o.x3.head1T = job3(W.head1_w, H, F, 1);
+    }
+    return woff;
+}
+
+int64_t weight_operand_bytes(const tnet_model_desc *d) {
+    Weights W;
+    weight_offsets(d, nullptr, &W);
+    CvtJobs J;
+    J.n = 0;
+    WeightOps o;
+    return weight_operands(*d, W, nullptr, J, o);
+}
+
 // Per-context kernel set-up (nothing needs opting in at present).
 int tnet_kernel_setup(tnet_ctx *c) {
     (void)c;
@@ -2541,21 +2648,6 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     auto slab = [&](int l) { return keep_act ? (int64_t)l : 0; };
     auto h1_cp = [&](int l) { return cp(Lw.h1_bf + (size_t)(slab(l) * maxU * F * esz_cp)); };
     auto h2_cp = [&](int l) { return cp(Lw.h2_bf + (size_t)(slab(l) * maxU * 2 * F * esz_cp)); };
-    struct LayerB {
-        WOp mlp2, mlp3, mlp2T, mlp3T, mix1, mix1T, mix2, mix2T, mlp1, mlp1T;
-    } lb[8] = {};
-    WOp emix{}, emixT{};
-    // 3xTF32 weight operands of the num_rbf-wide radial layers, in both
-    // tensor-core modes (rounding the narrow expnorm basis to bf16 costs more
-    // force accuracy than any other operand), and of the per-atom embedding
-    // and output MLPs in BF16 mode.  In the FP32-accurate mode those per-atom
-    // MLPs stay on FP32 FMA: they are cheap, and the energy is the quantity
-    // most sensitive to them (3xTF32 there costs an order of magnitude of
-    // energy accuracy).
-    const bool atom_x3 = prec == 1;
-    struct X3W {
-        WOp dproj, dprojT, emb_mlp1, emb_mlp1T, emb_mlp2, emb_mlp2T, out, outT, head1, head1T;
-    } wx{};
 
     // ---- graph prep
     ProfSeq pf(ctx, st);
@@ -2567,78 +2659,12 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     J.n = 0;
     if (!tab)
         for (int l = 0; l < NL; ++l) filter_row_jobs(J, W.layer[l], F, w3p(l), b3p(l));
-    if (tcm) {
-        char *wb = ctx->ws + Lw.wbf;
-        int64_t woff = 0;  // bytes
-        auto alloc = [&](int64_t elems, int esz) {
-            void *p = wb + woff;
-            woff += (elems * esz + 255) & ~(int64_t)255;
-            return p;
-        };
-        // forward operands keep the (out, in) = K-major layout; backward
-        // operands are transposed
-        auto job_m = [&](const float *src, int rows, int cols, int tr, int mode, int perm = 0) {
-            WOp w{};
-            const int esz = mode == 1 ? 2 : 4;
-            void *hi = alloc((int64_t)rows * cols, esz);
-            void *lo = mode == 2 ? alloc((int64_t)rows * cols, esz) : nullptr;
-            J.src[J.n] = src; J.hi[J.n] = hi; J.lo[J.n] = lo;
-            J.rows[J.n] = rows; J.cols[J.n] = cols; J.tr[J.n] = (signed char)tr; J.mode[J.n] = (signed char)mode;
-            J.perm[J.n] = (short)perm;
-            ++J.n;
-            w.b = hi;
-            w.blo = lo;
-            return w;
-        };
-        auto job = [&](const float *src, int rows, int cols, int tr) { return job_m(src, rows, cols, tr, prec); };
-        auto job3 = [&](const float *src, int rows, int cols, int tr) { return job_m(src, rows, cols, tr, 2); };
-        // [3][F][F] -> per-class transposes; the three classes' high parts (and
-        // residuals) must stay stacked contiguously [3F][F] for the GEMM
-        auto job_classes_T = [&](const float *src) {
-            const int64_t ff = (int64_t)F * F;
-            const int esz = prec == 1 ? 2 : 4;
-            char *hi = (char *)alloc(3 * ff, esz), *lo = prec == 2 ? (char *)alloc(3 * ff, esz) : nullptr;
-            for (int q = 0; q < 3; ++q) {
-                J.src[J.n] = src + q * ff;
-                J.hi[J.n] = hi + q * ff * esz;
-                J.lo[J.n] = lo ? lo + q * ff * esz : nullptr;
-                J.rows[J.n] = F; J.cols[J.n] = F; J.tr[J.n] = 1; J.mode[J.n] = (signed char)prec; J.perm[J.n] = 0;
-                ++J.n;
-            }
-            return WOp{hi, lo};
-        };
-        emix = job(W.emb_mix_w, 3 * F, F, 0);
-        emixT = job_classes_T(W.emb_mix_w);
-        for (int l = 0; l < NL; ++l) {
-            const LayerW &Lr = W.layer[l];
-            lb[l].mix1 = job(Lr.mix1_w, 3 * F, F, 0);
-            lb[l].mix1T = job_classes_T(Lr.mix1_w);
-            lb[l].mix2 = job(Lr.mix2_w, 3 * F, F, 0);
-            lb[l].mix2T = job_classes_T(Lr.mix2_w);
-            if (tab) continue;  // no per-pair radial MLP
-            lb[l].mlp2 = job(Lr.mlp2_w, 2 * F, F, 0);
-            lb[l].mlp3 = job_m(Lr.mlp3_w, 3 * F, 2 * F, 0, prec, F);
-            lb[l].mlp2T = job(Lr.mlp2_w, 2 * F, F, 1);
-            lb[l].mlp3T = job_m(Lr.mlp3_w, 3 * F, 2 * F, 1, prec, F);
-            lb[l].mlp1 = job3(Lr.mlp1_w, F, K, 0);
-            lb[l].mlp1T = job3(Lr.mlp1_w, F, K, 1);
-        }
-        if (!tab) {
-            wx.dproj = job3(W.dproj_w, 3 * F, K, 0);
-            wx.dprojT = job3(W.dproj_w, 3 * F, K, 1);
-        }
-        if (atom_x3) {
-            wx.emb_mlp1 = job3(W.emb_mlp1_w, 2 * F, F, 0);
-            wx.emb_mlp1T = job3(W.emb_mlp1_w, 2 * F, F, 1);
-            wx.emb_mlp2 = job3(W.emb_mlp2_w, 3 * F, 2 * F, 0);
-            wx.emb_mlp2T = job3(W.emb_mlp2_w, 3 * F, 2 * F, 1);
-            wx.out = job3(W.out_w, F, 3 * F, 0);
-            wx.outT = job3(W.out_w, F, 3 * F, 1);
-            wx.head1 = job3(W.head1_w, H, F, 0);
-            wx.head1T = job3(W.head1_w, H, F, 1);
-        }
-        if (woff > Lw.wbf_bytes || J.n > kMaxCvtJobs) return TNET_ERR_WORKSPACE;
-    }
+    WeightOps wo;
+    if (weight_operands(d, W, ctx->ws + Lw.wbf, J, wo) > Lw.wbf_bytes || J.n > kMaxCvtJobs) return TNET_ERR_WORKSPACE;
+    const LayerOps *lb = wo.layer;
+    const X3W &wx = wo.x3;
+    const bool atom_x3 = prec == 1;  // per-atom MLPs on 3xTF32
+    const WOp emix = wo.emix, emixT = wo.emixT;
     {
         const ElemTables et{W.emb, W.emb2_w, W.emb2_b, F, d.max_z, Ta, Tb};
         const int extra = (d.max_z * kElemParts + 63) / 64;  // grid rows of the element tables
