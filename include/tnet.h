@@ -275,11 +275,9 @@ int tnet_debug_tc_gemm(int M, int N, int K, const void *A, const void *B, float 
 int tnet_debug_tc_gemm_f32(int M, int N, int K, const float *A, const float *B, float *B_split, float *C,
                            int32_t *status_dev, tnet_stream_t stream);
 /* Either of the two above (x3 = 1: 3xTF32, B_split as there; x3 = 0: BF16,
- * B_split unused) with the CTAs in thread-block clusters of `cluster` (1, 2
- * or 4) that share each weight stage through TMA multicast, the form the
- * library uses for one-class GEMMs; TNET_ERR_ARG for another cluster size or
- * the shape errors above.  A tile whose rows do not split into whole 8-row
- * groups per CTA runs without clusters. */
+ * B_split unused).  `cluster` (1, 2 or 4, else TNET_ERR_ARG) is kept for
+ * callers of the form in which CTAs shared weight stages across a
+ * thread-block cluster; every value runs the CTAs on their own. */
 int tnet_debug_tc_gemm_cluster(int M, int N, int K, int x3, int cluster, const void *A, const void *B,
                                float *B_split, float *C, int32_t *status_dev, tnet_stream_t stream);
 /* Test of the failure path of the tensor-core kernel (no counterpart in the
@@ -300,7 +298,8 @@ int tnet_debug_tc_gemm_timeout(int M, int N, int K, const float *A, const float 
  * choice only changes speed.  Knob k takes
  * one of tnet_tuning_candidates(k, ...) (the count is returned; values are
  * written up to max).  tnet_set_tuning rejects values outside the candidate
- * lists.  A new context starts from fixed defaults, with programmatic launch
+ * lists.  The knob tc_cluster is retired: it keeps its place and its values,
+ * which all run the same.  A new context starts from fixed defaults, with programmatic launch
  * on only when max_atoms <= 1024.  An autotuner times the candidates on a
  * real input (as CUDA-graph replays) and sets the fastest
  * (paper_2402_17660_gb300.tnet.autotune). */

@@ -211,7 +211,7 @@ thread_local int tnet::tl_pdl = 1;
 
 // Candidate values of each tuning knob (TuneKnob) and the default's index.
 static const int kTuneCandidates[T_NKNOBS][4] = {{1, 2, 3, 4}, {192, 128, 0, 0}, {256, 128, 0, 0}, {4, 8, 16, 0},
-                                                 {4, 8, 16, 0}, {1, 0, 0, 0}, {0, 1, 4, 3}, {2, 1, 4, 0}};
+                                                 {4, 8, 16, 0}, {1, 0, 0, 0}, {0, 1, 4, 3}, {1, 2, 4, 0}};
 static const int kTuneCount[T_NKNOBS] = {4, 2, 2, 3, 3, 2, 4, 3};
 // Defaults: the shapes the autotuner picks on most measured workloads (24k to
 // 96k atoms, both tensor-core precisions).  Programmatic launch is on only for

@@ -59,12 +59,6 @@ struct TcShape {
     // bounded waits run out with no MMA and no unconsumed copy in flight
     uint32_t spin_limit;
     int skip_mma;
-    // CTAs per thread-block cluster (0 or 1: none; 2 or 4 for a one-class
-    // GEMM): the cluster's CTAs take consecutive 128-row tiles of the same
-    // column tile, and each loads 1/cl of every B (and B_lo) stage with TMA
-    // multicast into all of them, so the weights stream from L2 once per
-    // cl * 128 rows instead of once per 128
-    int cl;
     // 3xTF32: the operand is SiLU(A) (the converter warps apply silu_f to each
     // landed element before the split), so a layer's activation need not be
     // stored beside its pre-activation
@@ -104,15 +98,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, v
                                                uint32_t limit) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit));
 }
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// every thread of every CTA of the cluster
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(ncols)
                  : "memory");
@@ -151,17 +136,6 @@ __device__ __forceinline__ void tma_load_2d_if(uint32_t lead, void *dst, const C
         "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "r"(lead)
         : "memory");
 }
-// the same into every CTA of the cluster in `mask` (same shared-memory offset;
-// each destination's barrier at the offset of `bar` receives the bytes)
-__device__ __forceinline__ void tma_load_2d_mc_if(uint32_t lead, void *dst, const CUtensorMap *map, int x, int y,
-                                                  uint64_t *bar, uint16_t mask) {
-    asm volatile(
-        "{\n .reg .pred q;\n setp.ne.b32 q, %6, 0;\n @q "
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, "
-        "{%2, %3}], [%4], %5;\n}\n" ::"r"(smem_u32(dst)),
-        "l"((uint64_t)map), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask), "r"(lead)
-        : "memory");
-}
 // D (TMEM) (+)= A (smem desc) * B (smem desc)^T, kind::f16 with bf16 inputs
 __device__ __forceinline__ void umma_bf16(uint32_t lead, uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
                                           uint32_t idesc, uint32_t accum) {
@@ -177,15 +151,6 @@ __device__ __forceinline__ void umma_commit(uint32_t lead, uint64_t *bar) {
         "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n @q "
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(smem_u32(bar)),
         "r"(lead)
-        : "memory");
-}
-// the same arrival on the barrier at this offset in every CTA of `mask`
-__device__ __forceinline__ void umma_commit_mc(uint32_t lead, uint64_t *bar, uint16_t mask) {
-    asm volatile(
-        "{\n .reg .pred q;\n setp.ne.b32 q, %2, 0;\n @q "
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n" ::"r"(
-            smem_u32(bar)),
-        "h"(mask), "r"(lead)
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
@@ -342,16 +307,6 @@ struct TileIter {
         n0 = (t % tilesN) * BN_;
         return true;
     }
-    // cl > 1 (one class): cluster tile T -> this CTA's tile, rank r of the
-    // cluster taking row tile cl * (T / tilesN) + r (past the last row tile
-    // its rows are out of range: TMA fills them with zeros and the epilogue
-    // stores nothing, but the CTA still loads its share of B for the others)
-    __device__ __forceinline__ bool get_cl(int T, int cl, int r, int &m0, int &n0, int BN_) const {
-        if (T >= ((mt0 + cl - 1) / cl) * tilesN) return false;
-        m0 = ((T / tilesN) * cl + r) * BM;
-        n0 = (T % tilesN) * BN_;
-        return true;
-    }
 };
 __device__ __forceinline__ int64_t sel3(int z, int64_t a, int64_t b, int64_t c) { return z == 0 ? a : (z == 1 ? b : c); }
 
@@ -399,23 +354,13 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
     const int nk = (P.K + BK - 1) / BK;
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t lim = P.spin_limit;
-    // tile walk: over this CTA's tiles, or over its cluster's tiles
-    const int cl = P.cl > 1 ? P.cl : 1;
-    const int crank = cl > 1 ? (int)cluster_rank() : 0;
-    const uint16_t cmask = (uint16_t)((1u << cl) - 1u);
-    const int t_first = blockIdx.x / cl, t_step = gridDim.x / cl;
-    auto next_tile = [&](int t, int &z, int &m0, int &n0) -> bool {
-        if (cl > 1) {
-            z = 0;
-            return it.get_cl(t, cl, crank, m0, n0, BN);
-        }
-        return it.get(t, z, m0, n0, BN);
-    };
+    const int t_first = blockIdx.x, t_step = gridDim.x;
+    auto next_tile = [&](int t, int &z, int &m0, int &n0) { return it.get(t, z, m0, n0, BN); };
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], cl);  // released by the MMA issuer of every CTA of the cluster
+            mbar_init(&empty[s], 1);
             mbar_init(&conv[s], C::CONV_ARRIVE);
         }
         for (int b = 0; b < 2; ++b) {
@@ -429,8 +374,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
     }
     if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);
     fence_before();
-    if (cl > 1) cluster_sync();  // every CTA's barriers exist before any multicast reaches them
-    else __syncthreads();
+    __syncthreads();
     fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
@@ -452,17 +396,8 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
                 }
                 expect_tx_if(lead, &full[s], C::STAGE_TX);
                 tma_load_2d_if(lead, sA + s * C::A_BYTES, &tmA, kb * BK, ya, &full[s]);
-                if (cl > 1) {  // this CTA's 1/cl of the B rows, into every CTA
-                    const int hb = BN / cl;
-                    const uint32_t off = (uint32_t)(crank * hb * C::ROW);
-                    tma_load_2d_mc_if(lead, sB + s * C::B_BYTES + off, &tmB, kb * BK, yb + crank * hb, &full[s], cmask);
-                    if (X3)
-                        tma_load_2d_mc_if(lead, sBlo + s * C::B_BYTES + off, &tmBlo, kb * BK, yb + crank * hb, &full[s],
-                                          cmask);
-                } else {
-                    tma_load_2d_if(lead, sB + s * C::B_BYTES, &tmB, kb * BK, yb, &full[s]);
-                    if (X3) tma_load_2d_if(lead, sBlo + s * C::B_BYTES, &tmBlo, kb * BK, yb, &full[s]);
-                }
+                tma_load_2d_if(lead, sB + s * C::B_BYTES, &tmB, kb * BK, yb, &full[s]);
+                if (X3) tma_load_2d_if(lead, sBlo + s * C::B_BYTES, &tmBlo, kb * BK, yb, &full[s]);
             }
         }
         // own copies must land before the CTA exits: a wait that runs out is
@@ -519,8 +454,7 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
                         umma_bf16(lead, d, da + 2 * k, db + 2 * k, idesc, acc);
                     }
                 }
-                if (cl > 1) umma_commit_mc(lead, &empty[s], cmask);  // the stage is free in every CTA's view
-                else umma_commit(lead, &empty[s]);
+                umma_commit(lead, &empty[s]);
                 if constexpr (C::A_TMEM) umma_commit(lead, &aempty[kg % C::A_SLOTS]);
             }
             if (!ok) break;
@@ -736,9 +670,6 @@ __global__ void __launch_bounds__(TileCfg<BN, X3, NK, Epi::BULK>::THREADS, 1)
     }
     fence_before();
     __syncthreads();
-    // no CTA leaves while another may still multicast into its shared memory
-    // or release its stages
-    if (cl > 1) cluster_sync();
     if (warp == 1) {
         fence_after();
         tmem_dealloc(tmem, C::TMEM_COLS);
@@ -763,47 +694,11 @@ struct TcOperands {
     int64_t a_rows, lda, b_rows, ldb;
 };
 
-// How many clusters of `cl` CTAs of this kernel the device runs at once (0
-// if the query fails); cached per kernel handle, device and cluster size.
-inline int max_active_clusters(const void *kern, int threads, int smem, int cl) {
-    static std::mutex mu;
-    static std::vector<std::pair<std::pair<const void *, int>, int>> done;  // ((kernel, device * 8 + cl), count)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    const int key = dev * 8 + cl;
-    std::lock_guard<std::mutex> g(mu);
-    for (const auto &d : done)
-        if (d.first.first == kern && d.first.second == key) return d.second;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)cl, 1, 1);
-    cfg.blockDim = dim3((unsigned)threads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cudaLaunchAttribute a[1];
-    a[0].id = cudaLaunchAttributeClusterDimension;
-    a[0].val.clusterDim.x = (unsigned)cl;
-    a[0].val.clusterDim.y = 1;
-    a[0].val.clusterDim.z = 1;
-    cfg.attrs = a;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        n = 0;
-    }
-    done.push_back({{kern, key}, n});
-    return n;
-}
-
 // Launches one persistent GEMM: min(tiles, sms) CTAs, one per SM (`sms` is
-// the SM count of the device the stream runs on), in clusters of P.cl when
-// the GEMM has one class, the tile splits into cl row groups of whole 8-row
-// swizzle atoms, and the device runs such clusters.
+// the SM count of the device the stream runs on).
 template <int BN, bool X3, bool NK = false, class Epi>
-int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t *status, cudaStream_t st, int sms) {
+int tc_gemm_ops(const TcShape &P, const TcOperands &o, const Epi &epi, int32_t *status, cudaStream_t st, int sms) {
     using C = TileCfg<BN, X3, NK, Epi::BULK>;
-    TcShape P = P0;
-    int cl = P.cl > 1 ? P.cl : 1;
-    if (P.nclass != 1 || BN % cl || (BN / cl) % 8) cl = 1;
     const int esz = X3 ? 4 : 2;
     int maxM = 0;
     for (int z = 0; z < P.nclass; ++z) maxM = P.M[z] > maxM ? P.M[z] : maxM;
@@ -816,22 +711,14 @@ int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t 
     auto kern = k_tc_gemm<BN, Epi, X3, NK>;
     if ((rc = ensure_smem_attr((const void *)kern, (int)C::SMEM))) return rc;
     if (sms < 1) sms = 1;
-    int maxc = 0;
-    if (cl > 1) {
-        maxc = max_active_clusters((const void *)kern, C::THREADS, (int)C::SMEM, cl);
-        if (maxc > sms / cl) maxc = sms / cl;
-        if (maxc < 1) cl = 1;
-    }
-    P.cl = cl;
-    const int bbox = BN / cl;  // B rows each CTA loads per stage
     if (X3) {
         if ((rc = make_map_f32(&ma, o.A, o.a_rows, P.K, o.lda, BM, C::ROW))) return rc;
-        if ((rc = make_map_f32(&mb, o.B, o.b_rows, P.K, o.ldb, bbox, C::ROW))) return rc;
-        if ((rc = make_map_f32(&mbl, o.Blo, o.b_rows, P.K, o.ldb, bbox, C::ROW))) return rc;
+        if ((rc = make_map_f32(&mb, o.B, o.b_rows, P.K, o.ldb, BN, C::ROW))) return rc;
+        if ((rc = make_map_f32(&mbl, o.Blo, o.b_rows, P.K, o.ldb, BN, C::ROW))) return rc;
         mal = ma;  // unused: A_lo is formed in shared memory or TMEM
     } else {
         if ((rc = make_map_bf16(&ma, o.A, o.a_rows, P.K, o.lda, BM))) return rc;
-        if ((rc = make_map_bf16(&mb, o.B, o.b_rows, P.K, o.ldb, bbox))) return rc;
+        if ((rc = make_map_bf16(&mb, o.B, o.b_rows, P.K, o.ldb, BN))) return rc;
         mal = ma;
         mbl = mb;
     }
@@ -844,14 +731,7 @@ int tc_gemm_ops(const TcShape &P0, const TcOperands &o, const Epi &epi, int32_t 
     }
     int64_t tiles = 0;
     for (int z = 0; z < P.nclass; ++z) tiles += (int64_t)((P.M[z] + BM - 1) / BM) * ((P.N + BN - 1) / BN);
-    int grid;
-    if (cl > 1) {  // clusters over cluster tiles (cl row tiles of one column tile)
-        const int64_t ctiles = (int64_t)((P.M[0] + BM * cl - 1) / (BM * cl)) * ((P.N + BN - 1) / BN);
-        grid = (int)(ctiles < maxc ? ctiles : maxc) * cl;
-    } else {
-        grid = (int)(tiles < sms ? tiles : sms);
-    }
-    launch_cluster(kern, grid, C::THREADS, C::SMEM, st, cl, ma, mb, mal, mbl, mc, P, epi, status);
+    launch(kern, (unsigned)(tiles < sms ? tiles : sms), C::THREADS, C::SMEM, st, ma, mb, mal, mbl, mc, P, epi, status);
     count_launch();
     TNET_LAUNCH_CHECK();
     return TNET_OK;

@@ -234,6 +234,7 @@ class EnergyFn(torch.autograd.Function):
 
 
 # ------------------------------------------------------------------ autotuner
+RETIRED_KNOBS = ("tc_cluster",)   # whose values all run the same
 TUNE_CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tune", "tuning.json")
 
 
@@ -301,6 +302,8 @@ def autotune(model: TensorNet, z, pos, nl: NeighborList, batch=None, box=None, n
     for _ in range(passes):
         before = list(knobs)
         for k, (name, cands) in enumerate(tuning_knobs(model.lib)):
+            if name in RETIRED_KNOBS:
+                cands = [knobs[k]]
             res = {}
             for v in cands:
                 trial = list(knobs)
