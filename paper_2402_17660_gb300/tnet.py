@@ -204,30 +204,39 @@ class EnergyFn(torch.autograd.Function):
     d/dpos = -forces scaled per system by the incoming gradient.  When the
     weights need gradients, backward runs one pass seeded with the incoming
     gradient, which gives d/dweights and d/dpos together, and forward
-    evaluates the energies alone."""
+    evaluates the energies alone.  That pass reads the system again, so
+    forward keeps copies of z, the pair list, batch and box: they are written
+    in place between calls (neighbors(out=nl), a changing box), the list by
+    the library itself, which autograd's version counters do not see."""
 
     @staticmethod
     def forward(ctx, pos, weights, model: TensorNet, z, nl, batch, box, n_systems):
         model.set_weights(weights)
         want_pos, want_w = ctx.needs_input_grad[:2]
         E, Fo, _ = model.energy_forces(z, pos.detach(), nl, batch, box, n_systems, forces=want_pos and not want_w)
-        ctx.model, ctx.args = model, (z, nl, batch, box, n_systems)
-        ctx.save_for_backward(pos, weights, Fo)
+        ctx.model, ctx.n_systems = model, n_systems
+        if want_w:
+            kept = [t if t is None else t.clone() for t in (z, nl.row_ptr, nl.col, batch, box)]
+            ctx.save_for_backward(pos, weights, *kept)
+        else:
+            ctx.save_for_backward(pos, weights, Fo)
+            ctx.batch = batch
         return E
 
     @staticmethod
     def backward(ctx, gE):
-        pos, weights, Fo = ctx.saved_tensors
-        z, nl, batch, box, n_systems = ctx.args
-        model = ctx.model
         want_pos, want_w = ctx.needs_input_grad[:2]
+        model = ctx.model
         gpos = gw = None
         if want_w:
+            pos, weights, z, row_ptr, col, batch, box = ctx.saved_tensors
+            nl = NeighborList(row_ptr, col, None, float("nan"))
             model.set_weights(weights)
-            _, Fs, gw = model.energy_forces(z, pos.detach(), nl, batch, box, n_systems, forces=want_pos,
+            _, Fs, gw = model.energy_forces(z, pos.detach(), nl, batch, box, ctx.n_systems, forces=want_pos,
                                             grad_weights=True, seed=gE.to(torch.float32).contiguous())
             gpos = -Fs if want_pos else None
         elif want_pos:
+            Fo, batch = ctx.saved_tensors[2], ctx.batch
             scale = gE.to(torch.float32)[batch.long()] if batch is not None else gE.to(torch.float32)[0]
             gpos = -Fo * (scale[:, None] if batch is not None else scale)
         return gpos, gw, None, None, None, None, None, None
