@@ -181,7 +181,14 @@ int tnet_neighbors(tnet_ctx *ctx, int n_atoms, int n_systems, const float *pos,
  *   forces   [N][3] float32 output, or NULL to skip the reverse pass
  *   grad_weights  [tnet_weights_count] float32 output (overwritten) or NULL.
  * Results do not depend on the order of columns within a row beyond float
- * rounding; with the CSR of tnet_neighbors they are deterministic. */
+ * rounding; with the CSR of tnet_neighbors they are deterministic.  The same
+ * system alone, in a batch or in a context of other capacities agrees to
+ * float rounding and not always bit for bit: the number of rows chooses the
+ * tile of the FP32 layers (precisions 0 and 2), and small tiles add the terms
+ * of a dot product in two or four parts.
+ * A pair list that is not symmetric is reported (ARG) and its edges without a
+ * reverse contribute nothing; one whose row offsets decrease (ARG) is
+ * evaluated without pairs. */
 int tnet_energy_forces(tnet_ctx *ctx, const float *weights, int n_atoms, int n_systems,
                        const int32_t *z, const float *pos, const int32_t *batch,
                        const float *box, const int32_t *row_ptr, const int32_t *col,

@@ -186,9 +186,15 @@ __device__ __forceinline__ float4 f2_four(const uint64_t v[2]) {
 // What bounds it: the FP32 pipe (70 TFLOP/s from registers alone, scalar or
 // packed) and the issue slots beside it; packing halves the FMA instructions,
 // which leaves the issue slots to the shared-memory loads.  Each output is one
-// chain of FMAs in ascending k (KS = 1), so the tile sizes agree bit for bit;
+// chain of FMAs in ascending k (KS = 1), so those tile sizes agree bit for bit;
 // with KS > 1 the groups take every KS-th 4-deep slice and their sums are
-// added in group order, which cuts the chain that sets a small GEMM's time.
+// added in group order.  The tile follows from the rows a launch may have, so
+// a system's bits depend on the company it is evaluated in and on the
+// context's capacities (tnet.h says so); one chain in every tile (64 x 32 and
+// 32 x 32 with more warps of fewer outputs instead) would end that at the same
+// speed (32 atoms 307 us against 305, 3,000 atoms 3.51 ms against 3.52), but the
+// shorter chains are the more exact: forces of 32 atoms are 8.6e-7 from 64-bit
+// ones, 1.7e-6 with one chain.
 // Measured (GB300, us, the former 128 x 64 tile with 8-deep blocks first):
 //   M 82,000 N 384 K 256: 407 -> 318 (51 TFLOP/s); weights (out, in) 433 -> 353
 //   M 96,000 N 128 K 384: 233 -> 209      M 82,000 N 32 K 384: 121 -> 60
