@@ -298,6 +298,23 @@ int tnet_debug_tc_gemm_cluster(int M, int N, int K, int x3, int cluster, const v
 int tnet_debug_tc_gemm_timeout(int M, int N, int K, const float *A, const float *B, float *B_split, float *C,
                                uint32_t spin_limit, int32_t *status_dev, tnet_stream_t stream);
 
+/* The staged message kernels of F = 64 and 128 on the caller's arrays, and a
+ * test of their failure path.  row_ptr [N+1], col, pair_of (pair of each
+ * directed edge, -1: none), a3 [n_pairs][3][F] (planes I, A, S), phi [n_pairs];
+ * node tensors hold I rows [0, N), A rows [N, 4N), S rows [4N, 9N) of F floats,
+ * 16-byte aligned.
+ *   backward 0: out_i = sum_j phi SiLU(a3) V_j
+ *   backward 1: V = dE/dM, V2 = Y; out (dE/dY) is added to, ga3 is written,
+ *               gphi [2][n_pairs] is added to (the sum of its two rows counts)
+ * hold_copies 1 (with spin_limit >= 1 tries per wait): the copying warps bring
+ * nothing, the bounded waits run out, the kernel records TNET_ERR_TIMEOUT in
+ * *status_dev and returns without writing out, leaving the context usable.
+ * Otherwise spin_limit 0 is the library's limit. */
+int tnet_debug_message_tile(int F, int backward, int n_atoms, const int32_t *row_ptr, const int32_t *col,
+                            const int32_t *pair_of, const float *a3, const float *phi, const float *V,
+                            const float *V2, float *out, float *ga3, float *gphi, int64_t n_pairs,
+                            uint32_t spin_limit, int hold_copies, int32_t *status_dev, tnet_stream_t stream);
+
 /* ---- tuning (no counterpart in the paper) ---------------------------------
  * Launch-shape knobs of a context: grid sizes, GEMM column tiles and whether
  * kernels use programmatic dependent launch (the next kernel is scheduled

@@ -41,6 +41,7 @@ SIGNATURES = {
     "tnet_debug_tc_gemm_cluster": (_i32, [_i32, _i32, _i32, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _vp]),
     "tnet_debug_tc_gemm_f32": (_i32, [_i32, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _vp]),
     "tnet_debug_tc_gemm_timeout": (_i32, [_i32, _i32, _i32, _vp, _vp, _vp, _vp, ctypes.c_uint32, _vp, _vp]),
+    "tnet_debug_message_tile": (_i32, [_i32, _i32, _i32] + [_vp] * 10 + [_i64, ctypes.c_uint32, _i32, _vp, _vp]),
     "tnet_tuning_knobs": (_i32, []),
     "tnet_tuning_name": (ctypes.c_char_p, [_i32]),
     "tnet_tuning_candidates": (_i32, [_i32, ctypes.POINTER(_i32), _i32]),

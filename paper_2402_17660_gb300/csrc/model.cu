@@ -1260,15 +1260,18 @@ struct MsgTile {
 // BWD true: V = gM, V2 = Y, out = gY (added to), and per upper edge (j > i)
 // dE/dg = <gM_i, Y_j> + <gM_j, Y_i>, ga3 = dE/dg phi SiLU'(a3) and gphi[half][u]
 // += sum dE/dg SiLU(a3) over the warp's channels.
-// Every wait is bounded: on expiry the block records TIMEOUT, the roles stop
-// and each warp waits for its own copies.
+// Every wait is bounded and its verdict is the warp's: on expiry the block
+// records TIMEOUT, each warp stops as a whole and waits for its own copies.
+// Testing only (zero in every library call): spin_limit, a smaller bound on
+// each wait, and hold_copies, copying warps that copy nothing and arrive
+// nowhere, so that the consumers' waits run out.
 template <int F, bool BWD>
 __global__ void __launch_bounds__(MsgTile<F, BWD>::THREADS, 1)
     k_message_tile(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                    const int32_t *__restrict__ pair_of, const float *__restrict__ a3, const float *__restrict__ phiu,
                    const float *__restrict__ V, const float *__restrict__ V2, int N, int R, float *__restrict__ out,
                    OpCopy out_cp, float *__restrict__ ga3, OpCopy ga3_cp, float *__restrict__ gphi,
-                   int64_t gphi_stride, int32_t *status) {
+                   int64_t gphi_stride, int32_t *status, uint32_t spin_limit, int hold_copies) {
     pdl_entry();
     using T = MsgTile<F, BWD>;
     constexpr int NP = T::NP, FH = T::FH, G = T::G, HW = T::HW, NS = T::NS, ST = T::ST, D = T::D, C = T::C, CAP = T::CAP;
@@ -1303,7 +1306,7 @@ __global__ void __launch_bounds__(MsgTile<F, BWD>::THREADS, 1)
     const int groups = (N + R - 1) / R;
     bool ok = true;
     auto wait = [&](uint64_t *bar, uint32_t parity) {
-        if (!tc::mbar_wait(bar, parity, abort_flag)) {
+        if (!tc::mbar_wait_warp(bar, parity, abort_flag, spin_limit)) {
             if (!*abort_flag) set_status(status, TNET_ERR_TIMEOUT);
             *abort_flag = 1;
             ok = false;
@@ -1362,7 +1365,7 @@ __global__ void __launch_bounds__(MsgTile<F, BWD>::THREADS, 1)
             g = g_next;
         }
     } else if (w > C) {  // -------------------------------- copy the node rows in
-        for (int n_stage = 0;; ++n_stage) {
+        for (int n_stage = 0; !hold_copies; ++n_stage) {
             const int s = n_stage % ST;
             if (!wait(&named[s], (n_stage / ST) & 1)) break;
             const int meta = s_meta[s];
@@ -1389,7 +1392,8 @@ __global__ void __launch_bounds__(MsgTile<F, BWD>::THREADS, 1)
             cp_arrive(&full[s]);  // each lane, once its copies have landed
             if (meta & 512) break;
         }
-        cp_wait<0>();  // own copies land before the block exits
+        // own copies, which are in no copy group, land before the warp exits
+        asm volatile("cp.async.wait_all;" ::: "memory");
     } else {  // ----------------------------------------------------- consumers
         const int r = w / HW, half = w % HW;
         const uint32_t c0 = half * FH + 2 * NP * lane;
@@ -1581,6 +1585,29 @@ __global__ void __launch_bounds__(MsgTile<F, BWD>::THREADS, 1)
         }
         cp_wait<0>();
     }
+}
+
+// Rows per group of the staged message kernels: at most `most`, and as few as
+// let every SM have the same number of groups.
+static void msg_shape(int N, int sms, int most, int &run, int &grid) {
+    const int64_t rounds = (N + (int64_t)most * sms - 1) / ((int64_t)most * sms);
+    run = (int)((N + rounds * sms - 1) / (rounds * sms));
+    const int groups = (N + run - 1) / run;
+    grid = groups < sms ? groups : sms;
+}
+template <int F, bool BWD>
+static int message_tile(int sms, cudaStream_t st, const int32_t *row_ptr, const int32_t *col, const int32_t *pair_of,
+                        const float *a3, const float *phiu, const float *V, const float *V2, int N, float *out,
+                        OpCopy out_cp, float *ga3, OpCopy ga3_cp, float *gphi, int64_t gphi_stride, int32_t *status,
+                        uint32_t spin_limit = 0, int hold_copies = 0) {
+    using T = MsgTile<F, BWD>;
+    const int rc = ensure_smem_attr((const void *)k_message_tile<F, BWD>, T::SMEM);
+    if (rc) return rc;
+    int run, grid;
+    msg_shape(N, sms, T::G, run, grid);
+    launch(k_message_tile<F, BWD>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3, phiu, V, V2, N, run, out,
+           out_cp, ga3, ga3_cp, gphi, gphi_stride, status, spin_limit, hold_copies);
+    return TNET_OK;
 }
 
 // Xn = X / (q + 1), q = ||X||:  gX = gXn / (q + 1) - <gXn, X> / (q + 1)^2 * dq/dX
@@ -2761,14 +2788,6 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     const bool warp_rows = (ctx->tune[T_MSG_KERNEL] == 0 || ctx->tune[T_MSG_KERNEL] == 3) && !tab &&
                            (F == 64 || F == 128) &&
                            9LL * N * F < (1LL << 31) && (int64_t)maxU * 3 * F < (1LL << 31);
-    // rows per group of the staged message kernels: at most `most`, and as few
-    // as let every SM have the same number of groups
-    auto msg_shape = [&](int most, int &run, int &grid) {
-        const int64_t rounds = (N + (int64_t)most * sms - 1) / ((int64_t)most * sms);
-        run = (int)((N + rounds * sms - 1) / (rounds * sms));
-        const int groups = (N + run - 1) / run;
-        grid = groups < sms ? groups : sms;
-    };
 #define EMB_FWD(FF)                                                                                           \
     if (tab)                                                                                                  \
         launch(k_emb_edges<FF, true>, atom_blocks, FF, 0, st, geo, z, row_ptr, col, pair_of, N, d.max_z, fu, tf0, Ta, \
@@ -2878,14 +2897,8 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
     else launch_message<FF, false>(rows_pb, atom_blocks, st, row_ptr, col, pair_of, a3l, phiu, tabfn(1 + l), Y, \
                                    N, M)
         auto staged = [&](auto channels) -> int {
-            constexpr int FF = decltype(channels)::value;
-            using T = MsgTile<FF, false>;
-            TRY(ensure_smem_attr((const void *)k_message_tile<FF, false>, T::SMEM));
-            int run, grid;
-            msg_shape(T::G, run, grid);
-            launch(k_message_tile<FF, false>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3l, phiu, Y,
-                   (const float *)nullptr, N, run, M, none, (float *)nullptr, none, (float *)nullptr, (int64_t)0, status);
-            return TNET_OK;
+            return message_tile<decltype(channels)::value, false>(sms, st, row_ptr, col, pair_of, a3l, phiu, Y, nullptr,
+                                                                  N, M, none, nullptr, none, nullptr, 0, status);
         };
         if (warp_rows) TRY(F == 64 ? staged(Channels<64>{}) : staged(Channels<128>{}));
         else {
@@ -3006,14 +3019,8 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
             TNET_F_SWITCH(F, MSG_BWD_TAB);
         } else if (warp_rows) {
             auto staged = [&](auto channels) -> int {
-                constexpr int FF = decltype(channels)::value;
-                using T = MsgTile<FF, true>;
-                TRY(ensure_smem_attr((const void *)k_message_tile<FF, true>, T::SMEM));
-                int run, grid;
-                msg_shape(T::G, run, grid);
-                launch(k_message_tile<FF, true>, grid, T::THREADS, T::SMEM, st, row_ptr, col, pair_of, a3, phiu, gM, Y,
-                       N, run, gY, nbf, ga3_out, ga3_cp, gphiu, (int64_t)maxU, status);
-                return TNET_OK;
+                return message_tile<decltype(channels)::value, true>(sms, st, row_ptr, col, pair_of, a3, phiu, gM, Y, N,
+                                                                     gY, nbf, ga3_out, ga3_cp, gphiu, maxU, status);
             };
             TRY(F == 64 ? staged(Channels<64>{}) : staged(Channels<128>{}));
         } else {
@@ -3174,3 +3181,28 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
 }
 
 }  // namespace tnet
+
+extern "C" int tnet_debug_message_tile(int F, int backward, int n_atoms, const int32_t *row_ptr, const int32_t *col,
+                                       const int32_t *pair_of, const float *a3, const float *phi, const float *V,
+                                       const float *V2, float *out, float *ga3, float *gphi, int64_t n_pairs,
+                                       uint32_t spin_limit, int hold_copies, int32_t *status, tnet_stream_t stream) {
+    using namespace tnet;
+    if ((F != 64 && F != 128) || n_atoms < 1 || 9LL * n_atoms * F >= (1LL << 31) || n_pairs < 0 ||
+        n_pairs * 3 * F >= (1LL << 31) || (hold_copies && spin_limit < 1))
+        return TNET_ERR_ARG;
+    if (!row_ptr || !col || !pair_of || !a3 || !phi || !V || !out || !status || (backward && (!V2 || !ga3 || !gphi)))
+        return TNET_ERR_ARG;
+    int dev = 0, sms = 0;
+    TNET_CUDA_TRY(cudaGetDevice(&dev));
+    TNET_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const OpCopy none{nullptr, 0};
+    auto run = [&](auto channels, auto bwd) -> int {
+        return message_tile<decltype(channels)::value, decltype(bwd)::value>(
+            sms, (cudaStream_t)stream, row_ptr, col, pair_of, a3, phi, V, V2, n_atoms, out, none, ga3, none, gphi,
+            n_pairs, status, spin_limit, hold_copies);
+    };
+    TRY(F == 64 ? (backward ? run(Channels<64>{}, std::true_type{}) : run(Channels<64>{}, std::false_type{}))
+                : (backward ? run(Channels<128>{}, std::true_type{}) : run(Channels<128>{}, std::false_type{})));
+    TNET_LAUNCH_CHECK();
+    return TNET_OK;
+}
