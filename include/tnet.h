@@ -322,8 +322,9 @@ int tnet_debug_message_tile(int F, int backward, int n_atoms, const int32_t *row
  * choice only changes speed.  Knob k takes
  * one of tnet_tuning_candidates(k, ...) (the count is returned; values are
  * written up to max).  tnet_set_tuning rejects values outside the candidate
- * lists.  The knob tc_cluster is retired: it keeps its place and its values,
- * which all run the same.  A new context starts from fixed defaults, with programmatic launch
+ * lists (message_kernel 0, a former candidate, is accepted and runs as 3).
+ * The knob tc_cluster is retired: it keeps its place and its values, which
+ * all run the same.  A new context starts from fixed defaults, with programmatic launch
  * on only when max_atoms <= 1024.  An autotuner times the candidates on a
  * real input (as CUDA-graph replays) and sets the fastest
  * (paper_2402_17660_gb300.tnet.autotune). */

@@ -211,13 +211,17 @@ thread_local int tnet::tl_pdl = 1;
 
 // Candidate values of each tuning knob (TuneKnob) and the default's index.
 static const int kTuneCandidates[T_NKNOBS][4] = {{1, 2, 3, 4}, {192, 128, 0, 0}, {256, 128, 0, 0}, {4, 8, 16, 0},
-                                                 {4, 8, 16, 0}, {1, 0, 0, 0}, {0, 1, 4, 3}, {1, 2, 4, 0}};
-static const int kTuneCount[T_NKNOBS] = {4, 2, 2, 3, 3, 2, 4, 3};
+                                                 {4, 8, 16, 0}, {1, 0, 0, 0}, {3, 1, 4, 0}, {1, 2, 4, 0}};
+static const int kTuneCount[T_NKNOBS] = {4, 2, 2, 3, 3, 2, 3, 3};
+// A value a knob had of its own before and tuning files may hold: accepted, run
+// like another.  message_kernel 0 and 3 were two forms of the message adjoint
+// and both chose the staged kernels since.
+static bool former_value(int knob, int v) { return knob == T_MSG_KERNEL && v == 0; }
 // Defaults: the shapes the autotuner picks on most measured workloads (24k to
 // 96k atoms, both tensor-core precisions).  Programmatic launch is on only for
 // contexts of at most kPdlMaxAtoms atoms, the launch-bound systems it speeds up;
 // from a few thousand atoms on it was measured to slow the step by 5-15%.
-static const int kTuneDefault[T_NKNOBS] = {2, 0, 0, 2, 2, 1, 3, 0};
+static const int kTuneDefault[T_NKNOBS] = {2, 0, 0, 2, 2, 1, 0, 0};
 static const int64_t kPdlMaxAtoms = 1024;
 static const char *kTuneNames[T_NKNOBS] = {"gemm_ctas_per_sm",   "tc_tile_n_3f",        "tc_tile_n_2f",
                                            "row_blocks_per_sm",  "pair_blocks_per_sm",  "programmatic_launch",
@@ -332,7 +336,7 @@ int tnet_get_tuning(tnet_ctx *c, int32_t *knobs, int n) {
 int tnet_set_tuning(tnet_ctx *c, const int32_t *knobs, int n) {
     if (!c || !knobs || n < 0 || n > T_NKNOBS) return TNET_ERR_ARG;
     for (int k = 0; k < n; ++k) {
-        bool ok = false;
+        bool ok = former_value(k, knobs[k]);
         for (int i = 0; i < kTuneCount[k]; ++i) ok |= kTuneCandidates[k][i] == knobs[k];
         if (!ok) return TNET_ERR_ARG;
     }

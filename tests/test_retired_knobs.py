@@ -41,3 +41,22 @@ def test_former_cluster_values_are_accepted_and_change_nothing(precision):
     with pytest.raises(Exception):
         knobs[CLUSTER] = 3
         m.set_tuning(knobs)
+
+
+def test_every_message_form_is_listed_once():
+    assert tuning_knobs()[6] == ("message_kernel", [3, 1, 4])   # 3 and the former 0 are the same kernels
+
+
+@pytest.mark.gpu
+@pytest.mark.skipif(not torch.cuda.is_available(), reason="needs CUDA")
+def test_former_message_form_is_accepted_and_runs_like_its_equal():
+    from tests.gpu_helpers import DEV, gpu_energy_forces
+    s = synth.random_cluster(90, seed=5)
+    m = TensorNet(synth.init_weights(synth.ModelShape(), seed=0), max_atoms=90, max_pairs=90 * 89, device=DEV)
+    knobs = m.get_tuning()
+    assert knobs[6] == 3
+    E0, F0 = gpu_energy_forces(m, s)
+    m.set_tuning(knobs[:6] + [0] + knobs[7:])
+    assert m.get_tuning()[6] == 0
+    E1, F1 = gpu_energy_forces(m, s)
+    assert (E1 == E0).all() and (F1 == F0).all()
