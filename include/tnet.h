@@ -187,8 +187,8 @@ int tnet_neighbors(tnet_ctx *ctx, int n_atoms, int n_systems, const float *pos,
  * tile of the FP32 layers (precisions 0 and 2), and small tiles add the terms
  * of a dot product in two or four parts.
  * A pair list that is not symmetric is reported (ARG) and its edges without a
- * reverse contribute nothing; one whose row offsets decrease (ARG) is
- * evaluated without pairs. */
+ * reverse contribute nothing; one whose row offsets decrease, or with a row of
+ * more than N edges (ARG), is evaluated without pairs. */
 int tnet_energy_forces(tnet_ctx *ctx, const float *weights, int n_atoms, int n_systems,
                        const int32_t *z, const float *pos, const int32_t *batch,
                        const float *box, const int32_t *row_ptr, const int32_t *col,

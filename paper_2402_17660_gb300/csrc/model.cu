@@ -113,10 +113,11 @@ __device__ __forceinline__ int32_t row_offset(const int32_t *__restrict__ row_pt
 // those become pairs, so a list that lacks half of its edges (a half list, a
 // truncated one) never has more pairs than half of its edges, which is what
 // the pair buffers hold.  Every edge starts inactive.  Decreasing offsets make
-// rows overlap, and rows that share edges would write each other's rev: they
-// raise rows_bad, and the list then has no pairs at all.  One launch in the
-// place of four (launches and their gaps were most of the time of small
-// systems' graph preparation).
+// rows overlap, and rows that share edges would write each other's rev and be
+// walked once per row; a row of more than N edges repeats columns: either
+// raises rows_bad (reported as ARG), and the list is then taken as empty.  One
+// launch in the place of four (launches and their gaps were most of the time of
+// small systems' graph preparation).
 __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restrict__ box,
                              const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
                              const int32_t *__restrict__ col, int N, int S, int64_t cap, float rc,
@@ -134,10 +135,14 @@ __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restr
         const int32_t v0 = row_ptr[i], v1 = row_ptr[i + 1];
         if (v0 < 0 || (i == 0 && v0 != 0) || v1 < 0 || v0 > v1) set_status(status, TNET_ERR_ARG);
         if (v0 > cap || v1 > cap) set_status(status, TNET_ERR_CAPACITY);
-        if (e0 > e1) *rows_bad = 1;
+        if (e0 > e1 || e1 - e0 > N) {
+            set_status(status, TNET_ERR_ARG);
+            *rows_bad = 1;
+        }
         safe[i] = e0;
         if (i == N - 1) safe[N] = e1;
     }
+    if (e1 - e0 > N) return;  // (see rows_bad)
     int cnt = 0;
     for (int eb = e0; eb < e1; eb += 32) {
         const int e = eb + lane;
@@ -177,9 +182,9 @@ __global__ void k_graph_rows(const float *__restrict__ pos, const float *__restr
 // ascend strictly give at most E / 2 pairs; repeated columns (reported) can
 // give more, and those past maxU, the size of the pair buffers, stay inactive.
 // nu, the scan's total, is brought in line: the kernels after this one take
-// their pairs from it.
+// their pairs from it.  rows_bad: no pairs, and every row empty.
 __global__ void k_upper_assign(const float *__restrict__ pos, const float *__restrict__ box,
-                               const int32_t *__restrict__ batch, const int32_t *__restrict__ row_ptr,
+                               const int32_t *__restrict__ batch, int32_t *__restrict__ row_ptr,
                                const int32_t *__restrict__ col, const int32_t *__restrict__ rev, int N, float rc,
                                const int32_t *__restrict__ uoff, const int32_t *__restrict__ rows_bad, int maxU,
                                int32_t *__restrict__ nu, int32_t *__restrict__ pair_of, int2 *__restrict__ uij,
@@ -187,10 +192,16 @@ __global__ void k_upper_assign(const float *__restrict__ pos, const float *__res
     pdl_entry();
     const bool bad = *rows_bad != 0;
     if (blockIdx.x == 0 && threadIdx.x == 0 && (bad || *nu > maxU)) *nu = bad ? 0 : maxU;
-    if (bad) return;
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (i >= N) return;
     const int lane = threadIdx.x & 31;
+    if (bad) {  // no warp reads the offsets
+        if (lane == 0) {
+            row_ptr[i] = 0;
+            if (i == N - 1) row_ptr[N] = 0;
+        }
+        return;
+    }
     int base = uoff[i];
     for (int e0 = row_ptr[i]; e0 < row_ptr[i + 1]; e0 += 32) {
         const int e = e0 + lane;

@@ -36,13 +36,15 @@ def _lists(s):
     yield "overlapping", (np.where(np.arange(N + 1) % 2 == 0, 0, len(col)).astype(np.int32), col), None
     a = np.argsort(np.linalg.norm(s.pos - s.pos[0], axis=1))[1:5]   # four neighbours of atom 0
     a = np.sort(a)
-    m = 40
+    m = 24
     yield "repeated", _csr(np.concatenate([np.zeros(4 * m, int), a]),
                            np.concatenate([np.tile(a, m), np.zeros(4, int)])), "any"
+    yield "overlong", _csr(np.concatenate([np.zeros(N + 4, int), a]),
+                           np.concatenate([np.tile(a, N // 4 + 1), np.zeros(4, int)])), None
 
 
 @pytest.mark.parametrize("precision", [0, 2])
-@pytest.mark.parametrize("name", ["half", "truncated", "overlapping", "repeated"])
+@pytest.mark.parametrize("name", ["half", "truncated", "overlapping", "repeated", "overlong"])
 def test_malformed_list_is_reported_and_stays_inside_the_buffers(name, precision):
     s = synth.random_cluster(N, seed=12)
     (row_ptr, col), want = next((c, w) for k, c, w in _lists(s) if k == name)
