@@ -190,24 +190,26 @@ __global__ void k_upper_assign(const float *__restrict__ pos, const float *__res
                                int32_t *__restrict__ nu, int32_t *__restrict__ pair_of, int2 *__restrict__ uij,
                                int32_t *__restrict__ ue) {
     pdl_entry();
-    const bool bad = *rows_bad != 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && (bad || *nu > maxU)) *nu = bad ? 0 : maxU;
     const int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     if (i >= N) return;
     const int lane = threadIdx.x & 31;
-    if (bad) {  // no warp reads the offsets
+    // one round of loads: the flag does not hold up what follows
+    const bool bad = *rows_bad != 0;
+    const int total = *nu, r0 = row_ptr[i], r1 = row_ptr[i + 1];
+    int base = uoff[i];
+    if (i == 0 && lane == 0 && (bad || total > maxU)) *nu = bad ? 0 : maxU;
+    if (bad) {
         if (lane == 0) {
             row_ptr[i] = 0;
             if (i == N - 1) row_ptr[N] = 0;
         }
         return;
     }
-    int base = uoff[i];
-    for (int e0 = row_ptr[i]; e0 < row_ptr[i + 1]; e0 += 32) {
+    for (int e0 = r0; e0 < r1; e0 += 32) {
         const int e = e0 + lane;
         bool up = false;
         int j = -1, r = -1;
-        if (e < row_ptr[i + 1]) {
+        if (e < r1) {
             j = col[e];
             r = rev[e];
             if (r != e && j > i) {
