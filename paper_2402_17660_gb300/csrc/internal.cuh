@@ -464,7 +464,8 @@ void count_launch();
 // Stages timed by the optional CUDA-event profiler (tnet_profile).
 // Tuning knobs: 0 SIMT-GEMM CTAs per SM, 1 tcgen05 column tile for N = 3F,
 // 2 tcgen05 column tile for N = 2F, 3 row-kernel blocks per SM, 4 pair-kernel
-// blocks (256 threads) per SM, 5 programmatic dependent launch on (1) or off,
+// blocks (256 threads) per SM (the run-of-pairs embedding adjoint of F = 128
+// has a grid of its own), 5 programmatic dependent launch on (1) or off,
 // 6 message-kernel form, 7 retired (thread-block clusters of the tcgen05 GEMMs;
 // its values all run the same).
 enum TuneKnob {

@@ -1172,9 +1172,11 @@ __global__ void __launch_bounds__(F * RB, (512 / (F * RB)) > 0 ? 512 / (F * RB) 
 // What bounded the gathers was not bandwidth but latency (long-scoreboard
 // stalls, 12 warps with 24 row loads each in flight, 115 SM cycles an edge with
 // every pipe below half); both rings keep their loads ahead of the warps.  Now
-// the consumers' own instructions bound the adjoint (half of the issue slots,
-// three to four warps a scheduler) and the merge (about 250 cycles a column)
-// the messages.  Per launch, 96,000 atoms (5.2 M edges): messages 2.00 -> 1.46
+// the consumers' own work bounds both, with four warps a scheduler to hide it:
+// at 24,000 atoms a consumer waits for a stage a quarter of the time in the
+// messages and 13% in the adjoint, the merge (213 cycles a column) 44% and 62%
+// for a free one; half of the issue slots and 60-66% of the shared-memory
+// wavefronts are used (ncu).  Per launch, 96,000 atoms (5.2 M edges): messages 2.00 -> 1.46
 // ms, adjoint 4.16 -> 3.46; 3,000 atoms 76 -> 55 us and 148 -> 140.
 __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
     uint64_t r;
@@ -2019,55 +2021,55 @@ __global__ void __launch_bounds__(128, kPairBlocks) k_emb_bwd_pairs_v4(const flo
         const uint32_t fb = (uint32_t)u * 3u * F + c4;
         const F4 taj = ld4p(Ta + zj), tbj = ld4p(Tb + zj);
         const float ux = gu.x, uy = gu.y, uz = gu.z;
-            auto dup = [](float x) { return f2_pack(x, x); };
-            const uint64_t x2 = dup(ux), y2 = dup(uy), z2 = dup(uz), xx2 = dup(2.f * ux), yy2 = dup(2.f * uy);
-            const uint64_t bxx = dup(ux * ux - (1.0f / 3.0f)), byy = dup(uy * uy - (1.0f / 3.0f));
-            const uint64_t bxy = dup(ux * uy), bxz = dup(ux * uz), byz = dup(uy * uz);
-            const uint64_t ph2 = dup(gu.w), neg = dup(-1.f);
-            uint64_t sp = 0, sx = 0, sy = 0, sz = 0;
-            F4 o[3];
+        auto dup = [](float x) { return f2_pack(x, x); };
+        const uint64_t x2 = dup(ux), y2 = dup(uy), z2 = dup(uz), xx2 = dup(2.f * ux), yy2 = dup(2.f * uy);
+        const uint64_t bxx = dup(ux * ux - (1.0f / 3.0f)), byy = dup(uy * uy - (1.0f / 3.0f));
+        const uint64_t bxy = dup(ux * uy), bxz = dup(ux * uz), byz = dup(uy * uz);
+        const uint64_t ph2 = dup(gu.w), neg = dup(-1.f);
+        uint64_t sp = 0, sx = 0, sy = 0, sz = 0;
+        F4 o[3];
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const uint64_t zij = f2_add(tai.v[k], tbj.v[k]), zji = f2_add(taj.v[k], tbi.v[k]);
-                const uint64_t nji = f2_mul(zji, neg);
-                uint64_t q[9];
+        for (int k = 0; k < 2; ++k) {
+            const uint64_t zij = f2_add(tai.v[k], tbj.v[k]), zji = f2_add(taj.v[k], tbi.v[k]);
+            const uint64_t nji = f2_mul(zji, neg);
+            uint64_t q[9];
 #pragma unroll
-                for (int c = 0; c < 9; ++c)
-                    q[c] = f2_fma((c >= 1 && c < 4) ? nji : zji, h[c].v[k], f2_mul(zij, gi[c].v[k]));
-                const uint64_t q1 = f2_fma(z2, q[3], f2_fma(y2, q[2], f2_mul(x2, q[1])));
-                const uint64_t q2 = f2_fma(byz, q[8], f2_fma(bxz, q[7], f2_fma(bxy, q[6], f2_fma(byy, q[5], f2_mul(bxx, q[4])))));
-                sp = f2_fma(f[2].v[k], q2, f2_fma(f[1].v[k], q1, f2_fma(f[0].v[k], q[0], sp)));
-                const uint64_t dx = f2_fma(z2, q[7], f2_fma(y2, q[6], f2_mul(xx2, q[4])));
-                const uint64_t dy = f2_fma(z2, q[8], f2_fma(x2, q[6], f2_mul(yy2, q[5])));
-                const uint64_t dz = f2_fma(y2, q[8], f2_mul(x2, q[7]));
-                sx = f2_fma(f[2].v[k], dx, f2_fma(f[1].v[k], q[1], sx));
-                sy = f2_fma(f[2].v[k], dy, f2_fma(f[1].v[k], q[2], sy));
-                sz = f2_fma(f[2].v[k], dz, f2_fma(f[1].v[k], q[3], sz));
-                o[0].v[k] = f2_mul(ph2, q[0]);
-                o[1].v[k] = f2_mul(ph2, q1);
-                o[2].v[k] = f2_mul(ph2, q2);
-            }
+            for (int c = 0; c < 9; ++c)
+                q[c] = f2_fma((c >= 1 && c < 4) ? nji : zji, h[c].v[k], f2_mul(zij, gi[c].v[k]));
+            const uint64_t q1 = f2_fma(z2, q[3], f2_fma(y2, q[2], f2_mul(x2, q[1])));
+            const uint64_t q2 = f2_fma(byz, q[8], f2_fma(bxz, q[7], f2_fma(bxy, q[6], f2_fma(byy, q[5], f2_mul(bxx, q[4])))));
+            sp = f2_fma(f[2].v[k], q2, f2_fma(f[1].v[k], q1, f2_fma(f[0].v[k], q[0], sp)));
+            const uint64_t dx = f2_fma(z2, q[7], f2_fma(y2, q[6], f2_mul(xx2, q[4])));
+            const uint64_t dy = f2_fma(z2, q[8], f2_fma(x2, q[6], f2_mul(yy2, q[5])));
+            const uint64_t dz = f2_fma(y2, q[8], f2_mul(x2, q[7]));
+            sx = f2_fma(f[2].v[k], dx, f2_fma(f[1].v[k], q[1], sx));
+            sy = f2_fma(f[2].v[k], dy, f2_fma(f[1].v[k], q[2], sy));
+            sz = f2_fma(f[2].v[k], dz, f2_fma(f[1].v[k], q[3], sz));
+            o[0].v[k] = f2_mul(ph2, q[0]);
+            o[1].v[k] = f2_mul(ph2, q1);
+            o[2].v[k] = f2_mul(ph2, q2);
+        }
 #pragma unroll
-            for (int pl = 0; pl < 3; ++pl)
-                *reinterpret_cast<ulonglong2 *>(gfu + fb + pl * F) = make_ulonglong2(o[pl].v[0], o[pl].v[1]);
-            // four warp sums in six exchanges: each step halves the values a lane
-            // carries, so lanes 0, 8, 16, 24 end with one sum each
-            auto fold = [](uint64_t v) {
-                const float2 t = f2_unpack(v);
-                return t.x + t.y;
-            };
-            float a0 = fold(sp), a1 = fold(sx), a2 = fold(sy), a3 = fold(sz);
-            const bool hi = lane & 16, hj = lane & 8;
-            const float r0 = __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 16), r1 = __shfl_xor_sync(0xffffffffu, hi ? a1 : a3, 16);
-            a0 = (hi ? a2 : a0) + r0;
-            a1 = (hi ? a3 : a1) + r1;
-            const float r2 = __shfl_xor_sync(0xffffffffu, hj ? a0 : a1, 8);
-            a0 = (hj ? a1 : a0) + r2;
-            a0 += __shfl_xor_sync(0xffffffffu, a0, 4);
-            a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
-            a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
-            if ((lane & 7) == 0)
-                reinterpret_cast<float *>(pair_g)[4LL * u + (lane >> 3)] = lane == 0 ? a0 : gu.w * a0;
+        for (int pl = 0; pl < 3; ++pl)
+            *reinterpret_cast<ulonglong2 *>(gfu + fb + pl * F) = make_ulonglong2(o[pl].v[0], o[pl].v[1]);
+        // four warp sums in six exchanges: each step halves the values a lane
+        // carries, so lanes 0, 8, 16, 24 end with one sum each
+        auto fold = [](uint64_t v) {
+            const float2 t = f2_unpack(v);
+            return t.x + t.y;
+        };
+        float a0 = fold(sp), a1 = fold(sx), a2 = fold(sy), a3 = fold(sz);
+        const bool hi = lane & 16, hj = lane & 8;
+        const float r0 = __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 16), r1 = __shfl_xor_sync(0xffffffffu, hi ? a1 : a3, 16);
+        a0 = (hi ? a2 : a0) + r0;
+        a1 = (hi ? a3 : a1) + r1;
+        const float r2 = __shfl_xor_sync(0xffffffffu, hj ? a0 : a1, 8);
+        a0 = (hj ? a1 : a0) + r2;
+        a0 += __shfl_xor_sync(0xffffffffu, a0, 4);
+        a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+        a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+        if ((lane & 7) == 0)
+            reinterpret_cast<float *>(pair_g)[4LL * u + (lane >> 3)] = lane == 0 ? a0 : gu.w * a0;
     };
     for (int64_t u0 = wid * per; u0 < U; u0 += warps * per) {
         const int u_end = (int)(u0 + per < U ? u0 + per : U);
@@ -2794,7 +2796,7 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
           *hs1 = f32(Lw.hs1), *as2 = f32(Lw.as2), *s = f32(Lw.s), *q0 = f32(Lw.q0);
     float2 *ln0 = wsp<float2>(ctx, Lw.ln0);
     const int atom_blocks = N < sms * ctx->tune[T_ROW_BLOCKS] ? N : sms * ctx->tune[T_ROW_BLOCKS];
-    // message kernels (and the pair-parallel embedding adjoint): knob 0 or 3 =
+    // message kernels (and the pair-parallel embedding adjoint): knob 3 (or 0) =
     // the staged kernels (exact mode, F = 64 or 128, 32-bit offsets), 1 or 4 = that
     // many consecutive rows per block of F threads (one thread per channel)
     const int rows_pb = ctx->tune[T_MSG_KERNEL] == 4 ? 4 : 1;
@@ -3139,21 +3141,22 @@ int energy_forces_impl(tnet_ctx *ctx, const float *wblob, int N, int S, const in
                                                              Tb, gXraw, gfu, edge_g, gfu_cp, nullptr)
     const bool by_pair = !wg && !tab && warp_rows && F == 128;
     constexpr int pair_smem = 4 * kPairDepth * kPairBytes;
-    if (by_pair) TRY(ensure_smem_attr((const void *)k_emb_bwd_pairs_v4<128>, pair_smem));
-    if (by_pair)
+    if (by_pair) {
+        TRY(ensure_smem_attr((const void *)k_emb_bwd_pairs_v4<128>, pair_smem));
         launch(k_emb_bwd_pairs_v4<128>, kPairBlocks * sms, 128, pair_smem, st, geo, z, uij, nu, N, d.max_z, fu, Ta, Tb, gXraw, gfu,
                edge_g);
-    else
-    switch (F / 32) {
-        case 2: EMB_BWD(2); break;
-        case 4: EMB_BWD(4); break;
-        case 6: EMB_BWD(6); break;
-        case 8: EMB_BWD(8); break;
-        case 10: EMB_BWD(10); break;
-        case 12: EMB_BWD(12); break;
-        case 14: EMB_BWD(14); break;
-        case 16: EMB_BWD(16); break;
-        default: return TNET_ERR_ARG;
+    } else {
+        switch (F / 32) {
+            case 2: EMB_BWD(2); break;
+            case 4: EMB_BWD(4); break;
+            case 6: EMB_BWD(6); break;
+            case 8: EMB_BWD(8); break;
+            case 10: EMB_BWD(10); break;
+            case 12: EMB_BWD(12); break;
+            case 14: EMB_BWD(14); break;
+            case 16: EMB_BWD(16); break;
+            default: return TNET_ERR_ARG;
+        }
     }
 #undef EMB_BWD
     count_launch();

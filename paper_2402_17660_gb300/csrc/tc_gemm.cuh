@@ -21,12 +21,14 @@
 //          ever goes through HBM.
 //
 // Persistent CTAs walk 128 x BN output tiles.  Warp 0 issues TMA loads into a
-// 3-4 stage shared-memory ring (k-blocks of 128-byte rows for BF16, 64-byte
-// rows for 3xTF32, whose stage holds four tiles), warp 1 owns TMEM and issues
-// the MMAs (32-byte k-steps) into one of two accumulators, so the epilogue of
-// a tile overlaps the MMAs of the next.  Sixteen epilogue warps (eight for
-// the 128- and 192-wide 3xTF32 tiles) drain TMEM (warp w reads lanes 32*(w%4) .. +31,
-// a quarter (half) of the tile's columns each) and run the fused epilogue.  Every mbarrier wait is bounded;
+// shared-memory ring of 3 to 6 stages (k-blocks of 128-byte rows for BF16 and
+// for 3xTF32 with A's split in TMEM; 64-byte rows for 3xTF32 with the split in
+// shared memory, whose stage holds A, A_lo, B and B_lo), warp 1 owns TMEM and
+// issues the MMAs (32-byte k-steps) into one of two accumulators, so the
+// epilogue of a tile overlaps the MMAs of the next.  Sixteen epilogue warps
+// (eight for 3xTF32 tiles but the num_rbf-deep ones) drain TMEM (warp w reads
+// lanes 32*(w%4) .. +31, a quarter (half) of the tile's columns each) and run
+// the fused epilogue.  Every mbarrier wait is bounded;
 // on expiry the kernel records TNET_ERR_TIMEOUT, the other roles stop, the
 // producer waits (bounded) for its own copies in flight, TMEM is freed and
 // the kernel returns.
@@ -224,9 +226,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float v[16]) {
 template <int BN, bool X3 = false, bool NK = false, bool BULK = false>
 struct TileCfg {
     // 3xTF32 at BN <= 192 (K beyond two k-blocks): A's split goes to TMEM
-    // instead of shared memory.  Four converter warps (one per TMEM lane
-    // quadrant) read each landed A row, split it and store A_hi and A_lo with
-    // tcgen05.st into a slot of columns after the two accumulators; the MMAs
+    // instead of shared memory.  A set of four converter warps (one per TMEM
+    // lane quadrant; two sets, see CONV) reads each landed A row, splits it and
+    // stores A_hi and A_lo with tcgen05.st into a slot of columns after the two accumulators; the MMAs
     // then read only B from shared memory, and the stage needs no A_lo buffer.
     // The narrow tiles (32 or 64 output columns, whose k-blocks carry little
     // MMA work) gain most: their pace is set by splitting A.
@@ -260,10 +262,9 @@ struct TileCfg {
     static constexpr int A_SLOTS = A_TMEM ? ((512 - 2 * BN) / A_SLOT_COLS > 4 ? 4 : (512 - 2 * BN) / A_SLOT_COLS) : 1;
     static constexpr uint32_t TMEM_COLS =
         A_TMEM ? 512 : (2 * BN <= 64 ? 64 : 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512);
-    // epilogue warps: 16, or 8 for the 128- and 192-wide 3xTF32 tiles, whose
-    // freed transpose buffers make room for a deeper pipeline; NK (a K of at
-    // most two k-blocks, whose epilogue outweighs its MMAs) keeps 16 and 4
-    // stages
+    // epilogue warps: 16, or 8 for 3xTF32, where the freed transpose buffers
+    // make room for a deeper pipeline; NK (a K of at most two k-blocks, whose
+    // epilogue outweighs its MMAs) keeps 16 and 4 stages
     static constexpr int EPI = (X3 && !NK && (BN >= 128 || A_TMEM)) ? 8 : 16;
     static constexpr int THREADS = 64 + 32 * (EPI + CONV);
     // epilogue buffers per warp: two bulk-store tiles, or a transpose (and no
@@ -271,11 +272,9 @@ struct TileCfg {
     // 0.81 ms a call instead of 0.67 at 24,000 atoms with 4 KB each)
     static constexpr int WARP_STAGE = BULK ? 4096 : 32 * STG_LD * 4;
     static constexpr uint32_t STAGE_BYTES = EPI * WARP_STAGE;
-    // 3xTF32: 4 stages, and as many as fit beside the epilogue buffers (6 at
-    // BN = 128, 5 at 192, 4 at 256): each stage's split and three MMAs make a
-    // long round trip, which the wide radial layers feel.  The narrow tiles (K-wide outputs)
-    // keep 4 and a smaller footprint, which leaves room on the SM for the CTAs
-    // of the next kernel that programmatic launch brings in early.
+    // 3xTF32 with the split in shared memory (BN = 256, and NK): as many
+    // 64-byte stages as fit beside the epilogue buffers, which is 4 at 256, and
+    // 4 for NK.
     static constexpr int X3_FIT = (int)((232448 - 1024 - 1024 - STAGE_BYTES) / (STAGE_TX + A_BYTES));
     // A_TMEM: as many 128-byte stages as fit, at most four (six for the
     // narrow tiles, which stream A).  BF16: four stages (three at BN = 256,
