@@ -408,9 +408,11 @@ def stage_roofline(tag, per_launch_ms, nu, N, E, F, K, prec, table, rec, peaks):
     hbm = peaks.get("hbm_gbs", 6800.0)
     bf16_peak = peaks.get("bf16_tflops", 1900.0)
     fp32_peak = SM_COUNT * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12  # TFLOP/s, derived
-    if prec == "tf32x3" and not table and tag in ("mlp2", "mlp3", "mlp3_bwd", "mlp2_bwd"):
+    if not table and (prec == "tf32x3" and tag in ("mlp2", "mlp3", "mlp3_bwd", "mlp2_bwd")
+                      or prec != "fp32" and tag in ("mlp1", "mlp1_bwd")):
         # 3xTF32: three TF32 MMAs per product (the residuals are formed on
-        # chip, so the bytes are those of the fp32 operands)
+        # chip, so the bytes are those of the fp32 operands); the num_rbf-wide
+        # layers run so in both tensor modes
         engine = "tensor_tf32"
     if engine == "tensor":
         cpeak, cname, cnote = bf16_peak, "tensor", "of measured bf16 burst (MEASURED_PEAKS.json)"
